@@ -123,12 +123,63 @@ __device__ __forceinline__ T ldv(const T *p) { return *p; }
 template <typename T>
 __device__ __forceinline__ T ldv(const __nv_bfloat16 *p) { return (T)__bfloat162float(*p); }
 
+// FP64 row dots of the apply.  GB300's FP64 pipe retires about two lane
+// operations per clock per SM, and the whole-warp sum of a row costs five
+// additions on all 32 lanes: more than the seven products a lane has in a row
+// of 225.  So eight lanes take a row and a warp four rows at a time (16-byte
+// loads, four in flight per lane): three additions per four rows.  Measured
+// on the 1023^2 leaf forward step (FP64 pipe bound, floor 274 us): 903 -> 444 us.
+__device__ __forceinline__ void warp_rows_dot4_f64(const double *const (&rp)[kRows],
+                                                   const int (&nq)[kRows], const double *xs,
+                                                   double (&acc)[kRows]) {
+  static_assert(kRows == 4, "a row per eight lanes");
+  const int lane = threadIdx.x & 31, sub = lane & 7;
+  const double *row = rp[0];
+  int np2 = 2 * nq[0];  // pairs of the lane's row
+#pragma unroll
+  for (int u = 1; u < kRows; ++u)
+    if ((lane >> 3) == u) {
+      row = rp[u];
+      np2 = 2 * nq[u];
+    }
+  double a = 0.0, b = 0.0;
+  int p = sub;
+  for (; p + 24 < np2; p += 32) {
+    double2 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const double2 *>(row + 2 * (p + 8 * k));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double2 xv = *reinterpret_cast<const double2 *>(xs + 2 * (p + 8 * k));
+      a += v[k].x * xv.x;
+      b += v[k].y * xv.y;
+    }
+  }
+#pragma unroll 3
+  for (; p < np2; p += 8) {
+    const double2 v = *reinterpret_cast<const double2 *>(row + 2 * p);
+    const double2 xv = *reinterpret_cast<const double2 *>(xs + 2 * p);
+    a += v.x * xv.x;
+    b += v.y * xv.y;
+  }
+  a += b;
+  a += __shfl_xor_sync(0xffffffffu, a, 4);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  a += __shfl_xor_sync(0xffffffffu, a, 1);
+#pragma unroll
+  for (int u = 0; u < kRows; ++u) acc[u] = __shfl_sync(0xffffffffu, a, 8 * u);
+}
+
 // Dot products of kRows padded rows (pointers rp, lengths in quads nq) with
 // the zero-padded shared vector xs by one warp; every row's loads are issued
-// before the FMAs.
+// before the FMAs.  FP64: see warp_rows_dot4_f64.
 template <typename T, typename TV = T>
 __device__ __forceinline__ void warp_rows_dot4(const TV *const (&rp)[kRows], const int (&nq)[kRows],
                                                const T *xs, T (&acc)[kRows]) {
+  if constexpr (sizeof(T) == 8) {
+    warp_rows_dot4_f64(rp, nq, xs, acc);
+    return;
+  }
   const int lane = threadIdx.x & 31;
   int maxq = 0;
 #pragma unroll
@@ -626,6 +677,66 @@ __global__ void __launch_bounds__(256) k_group_cols_split(const int2 *__restrict
   }
 }
 
+// FP64 columns [a, b) of the backward cell step.  Bound by the FP64 pipe, so
+// no lane may sit out a multiply-add that its warp executes: a warp takes
+// blocks of 32 columns and every (NT / 32)-th row of the block, which leaves
+// only the diagonal 32 x 32 blocks of G half empty (14% of the products of a
+// 225-row cell; the quad-pair layout of the FP32 path, whose lanes walk
+// different rows of the triangle, executes 1.85 times the products needed).
+// The warps' sums meet in shared memory, 256 columns at a time.  Measured on
+// the 1023^2 leaf backward step (floor 274 us): 526 -> 374 us.
+template <int NT>
+__device__ __forceinline__ void cell_bwd_cols_f64(const CellItem &it, const CellDesc &c,
+                                                  const int *__restrict__ I, const double *__restrict__ G,
+                                                  const double *__restrict__ V, long long vstride,
+                                                  const double *xs, const double *xb, double *part,
+                                                  double *__restrict__ x) {
+  constexpr int NW = NT / 32, kCols = 256;  // NW * kCols = 8 NT partial sums
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int s0 = it.a; s0 < it.b; s0 += kCols) {
+    const int s1 = min(it.b, s0 + kCols);
+    for (int c0 = s0; c0 < s1; c0 += 32) {
+      const int col = c0 + lane;
+      const bool ok = col < s1;
+      double acc = 0.0, acc2 = 0.0;
+      // rows of the diagonal block: row i holds the columns <= i
+      int i = c0 + warp;
+      for (; i < c0 + 32 && i < c.nI; i += NW)
+        acc += (ok && col <= i ? G[tri_off(i) + col] : 0.0) * xs[i];
+      for (; i + 3 * NW < c.nI; i += 4 * NW) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = ok ? G[tri_off(i + k * NW) + col] : 0.0;
+        acc += v[0] * xs[i];
+        acc2 += v[1] * xs[i + NW];
+        acc += v[2] * xs[i + 2 * NW];
+        acc2 += v[3] * xs[i + 3 * NW];
+      }
+      for (; i < c.nI; i += NW) acc += (ok ? G[tri_off(i) + col] : 0.0) * xs[i];
+      int q = warp;
+      for (; q + 3 * NW < c.nB; q += 4 * NW) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = ok ? V[(long long)(q + k * NW) * vstride + col] : 0.0;
+        acc -= v[0] * xb[q];
+        acc2 -= v[1] * xb[q + NW];
+        acc -= v[2] * xb[q + 2 * NW];
+        acc2 -= v[3] * xb[q + 3 * NW];
+      }
+      for (; q < c.nB; q += NW) acc -= (ok ? V[(long long)q * vstride + col] : 0.0) * xb[q];
+      part[warp * kCols + (c0 - s0) + lane] = acc + acc2;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < s1 - s0; t += NT) {
+      double s = part[t];
+#pragma unroll
+      for (int w = 1; w < NW; ++w) s += part[w * kCols + t];
+      x[I[s0 + t]] = s;
+    }
+    __syncthreads();
+  }
+}
+
 // Backward cell step (E_I): x_I <- G^T xI_I - V^T x_B, for columns [a, b)
 // (a a multiple of 4) of one cell.  A thread owns the column quad pair
 // (qa, qb) = (first + p, last - p), which balances the triangular row counts,
@@ -660,6 +771,10 @@ __device__ __forceinline__ void cell_bwd_unit(const CellItem &it, const CellDesc
   const TV *G = vals + c.G_off;
   const TV *V = vals + c.V_off;
   const long long vstride = pad4(c.nI);
+  if constexpr (sizeof(T) == 8) {
+    cell_bwd_cols_f64<NT>(it, c, I, G, V, vstride, xs, xb, part, x);
+    return;
+  }
   const int q0 = it.a / 4, q1 = (it.b + 3) / 4;  // column quads [q0, q1)
   const int npairs = (q1 - q0 + 1) / 2;
   int PW, RG;
