@@ -35,9 +35,6 @@
 
 namespace hifcn {
 
-int apply_levels_f32_range(Handle *h, float *contrib, float *xI, float *x, int l0, int l1, bool forward,
-                           cudaStream_t s);
-
 namespace {
 
 using bf16 = __nv_bfloat16;
@@ -74,6 +71,7 @@ struct MArgs {
   const GroupDesc *groups;
   const int *idx;
   const bf16 *v16;
+  const float *v32;         // FP32 values (the levels below the BF16 ones)
   const long long *gs_off;  // per entity of the level: offset of its inputs in gs
   long long root_G_off;
   const int *ridx;
@@ -409,6 +407,243 @@ __global__ void __launch_bounds__(kMThreads, 2) k_box_mma(MArgs a, int ph) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncol_alloc) : "memory");
 }
 
+// ------------------------------------------- FP32 levels, all columns at once
+//
+// The levels below the BF16 ones keep FP32 blocks and FP32 arithmetic, so
+// their products Y (m x k) = A (m x K) X (K x k) run on the FP32 cores, each
+// block read once for up to 32 columns instead of once per column.  One CTA of
+// 128 threads takes a 128-row tile of a box; K is walked in chunks of 32,
+// A and the gathered X staged by asynchronous copies three chunks deep.  A
+// thread owns 4 rows x NC / 4 columns: per four K it reads 4 + 4 quads of
+// shared memory for 4 NC multiply-adds (two NC = 16 FMAs per byte of A), which
+// keeps the kernel near the HBM rate at k = 16 (a chip-wide FP32 rate of 40e12
+// FMA/s against 1.7e12 values/s of A times 16).  Each chunk is summed on its
+// own and added to the total, so a sum of K products rounds like one of
+// 32 + K / 32.  kComp (the levels whose single-column backward step sums the
+// boundary products with compensation): four products at a time enter the
+// total by Kahan's summation.  Backward cells: the K index runs over the G
+// rows padded to a multiple of 64, then the V rows, whose chunks are
+// subtracted.
+// Measured at 63^3 with 16 columns (level 0, 353 MB of blocks): forward 1720 ->
+// 206 us, backward 1568 -> 263 us per apply.
+constexpr int kFThreads = 128;
+constexpr int kFC = 32;          // K of a staged chunk
+constexpr int kFStages = 3;
+constexpr int kFLdA = kFC + 4;   // floats per staged row of A (conflict-free quads)
+
+template <int NC>
+__host__ __device__ constexpr size_t f32_stage_floats() { return (size_t)kTM * kFLdA + (size_t)kFC * NC; }
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(su32(dst)), "l"(src), "r"(ok ? 16 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *dst, const void *src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(su32(dst)), "l"(src), "r"(ok ? 4 : 0)
+               : "memory");
+}
+
+// stored FP32 row `row` of a box and its padded length
+struct FRow {
+  const float *p;
+  int len;
+};
+__device__ __forceinline__ FRow f32_row(const float *v, const CellDesc &c, const GroupDesc &g, bool cell, int row) {
+  if (!cell) return {v + g.H_off + (long long)row * pad4(g.n), (int)pad4(g.n)};
+  if (row < c.nI) return {v + c.G_off + tri_off(row), (int)pad4(row + 1)};
+  return {v + c.V_off + (long long)(row - c.nI) * pad4(c.nI), (int)pad4(c.nI)};
+}
+
+template <int NC, bool kTrans, bool kComp>
+__global__ void __launch_bounds__(kFThreads) k_box_f32(MArgs a, int ph) {
+  extern __shared__ __align__(16) float fsm[];
+  constexpr int CP = NC / 4;  // columns per thread
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const MTile tile = a.tiles[blockIdx.x];
+  const int n0 = blockIdx.y * NC;
+  const bool cell = ph == kMCellFwd || ph == kMCellBwd;
+  CellDesc cd{};
+  GroupDesc gd{};
+  if (cell) cd = a.cells[tile.unit];
+  else gd = a.groups[tile.unit];
+  // rows of the product, stored rows (transposed: the K range), and the K
+  // index of the first V row of a backward cell
+  const int m = ph == kMCellFwd ? cd.nI + cd.nB : cell ? cd.nI : gd.n;
+  const int K = cell ? cd.nI : gd.n;                       // K of the forward forms and of G
+  const int kV = ph == kMCellBwd ? (cd.nI + 63) & ~63 : 1 << 30;
+  const int c_begin = tile.c0 * (kKC / kFC), c_end = tile.c1 * (kKC / kFC);
+  // staging of A: thread t copies quads t, t + 128, ... of the chunk
+  const int sq = kTrans ? (t & 31) : (t & 7);              // quad within a staged row
+  const int srow = kTrans ? (t >> 5) : (t >> 3);           // first staged row of the thread
+  constexpr int kSRows = 8;                                // staged rows per thread
+  constexpr int kSStep = kTrans ? kFThreads / 32 : kFThreads / 8;
+  FRow fr[kTrans ? 1 : kSRows];
+  if constexpr (!kTrans) {
+#pragma unroll
+    for (int j = 0; j < kSRows; ++j) {
+      const int row = tile.r0 + srow + kSStep * j;
+      fr[j] = row < m ? f32_row(a.v32, cd, gd, cell, row) : FRow{a.v32, 0};
+    }
+  }
+  // gathered input row kk of the chunk at K index k: index -1 when absent
+  auto x_index = [&](int k) -> int {
+    if (!cell) return k < K ? k : -1;
+    if (ph == kMCellFwd) return k < K ? a.idx[cd.I_off + k] : -1;
+    if (k < kV) return k < cd.nI ? a.idx[cd.I_off + k] : -1;
+    return k - kV < cd.nB ? a.idx[cd.B_off + k - kV] : -1;
+  };
+  const float *gsrc = cell ? nullptr : a.gs + a.gs_off[tile.unit];
+  const int xk = t & (kFC - 1), xn = t / kFC;              // X element: row xk, columns xn + 4 j
+  int xi = c_begin < c_end ? x_index(c_begin * kFC + xk) : -1;  // of the next chunk to stage
+  auto stage = [&](int c) {
+    if (c < c_end) {
+      float *sA = fsm + (size_t)((c - c_begin) % kFStages) * f32_stage_floats<NC>();
+      float *sX = sA + (size_t)kTM * kFLdA;
+      const int k0 = c * kFC;
+      if constexpr (kTrans) {
+#pragma unroll
+        for (int j = 0; j < kSRows; ++j) {
+          const int kk = srow + kSStep * j, k = k0 + kk;
+          const int row = k < kV ? (k < K ? k : -1) : (k - kV < cd.nB ? cd.nI + k - kV : -1);
+          FRow f{a.v32, 0};
+          if (row >= 0) f = f32_row(a.v32, cd, gd, cell, row);
+          const int i = tile.r0 + 4 * sq;
+          const bool ok = i < f.len;
+          cp_async16(sA + kk * kTM + 4 * sq, f.p + (ok ? i : 0), ok);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < kSRows; ++j) {
+          const int k = k0 + 4 * sq;
+          const bool ok = k < fr[j].len;
+          cp_async16(sA + (srow + kSStep * j) * kFLdA + 4 * sq, fr[j].p + (ok ? k : 0), ok);
+        }
+      }
+      const float *src;
+      long long ld;
+      if (!cell) {
+        src = gsrc + (xi >= 0 ? xi : 0);
+        ld = a.ldg;
+      } else {
+        src = (ph == kMCellBwd && k0 < kV ? a.xI : a.x) + (xi >= 0 ? xi : 0);
+        ld = a.ldx;
+      }
+#pragma unroll
+      for (int j = 0; j < CP; ++j) {
+        const int n = n0 + xn + 4 * j;
+        const bool ok = xi >= 0 && n < a.ncols;
+        cp_async4(sX + xk * NC + xn + 4 * j, src + (ok ? n * ld : 0), ok);
+      }
+      if (c + 1 < c_end) xi = x_index(k0 + kFC + xk);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  stage(c_begin);
+  stage(c_begin + 1);
+  const int cg = lane & 3, rg = warp * 8 + (lane >> 2);
+  float tot[4][CP], cmp[4][kComp ? CP : 1];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+#pragma unroll
+    for (int j = 0; j < CP; ++j) tot[u][j] = 0.f;
+#pragma unroll
+    for (int j = 0; j < (kComp ? CP : 1); ++j) cmp[u][j] = 0.f;
+  }
+  for (int c = c_begin; c < c_end; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kFStages - 2) : "memory");
+    __syncthreads();
+    stage(c + kFStages - 1);
+    const float *sA = fsm + (size_t)((c - c_begin) % kFStages) * f32_stage_floats<NC>();
+    const float *sX = sA + (size_t)kTM * kFLdA;
+    const bool neg = c * kFC >= kV;
+    float acc[4][CP];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int j = 0; j < CP; ++j) acc[u][j] = 0.f;
+#pragma unroll 2
+    for (int kk = 0; kk < kFC; kk += 4) {
+      float av[4][4];  // [row][k] or, transposed, [k][row]
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 v = *reinterpret_cast<const float4 *>(kTrans ? sA + (kk + u) * kTM + 4 * rg
+                                                                  : sA + (rg + 32 * u) * kFLdA + kk);
+        av[u][0] = v.x; av[u][1] = v.y; av[u][2] = v.z; av[u][3] = v.w;
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float xv[CP];
+        const float *px = sX + (kk + q) * NC + cg * CP;
+        if constexpr (CP == 2) {
+          const float2 v = *reinterpret_cast<const float2 *>(px);
+          xv[0] = v.x; xv[1] = v.y;
+        } else {
+#pragma unroll
+          for (int j = 0; j < CP; j += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(px + j);
+            xv[j] = v.x; xv[j + 1] = v.y; xv[j + 2] = v.z; xv[j + 3] = v.w;
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int j = 0; j < CP; ++j) acc[u][j] = fmaf(kTrans ? av[q][u] : av[u][q], xv[j], acc[u][j]);
+      }
+      if constexpr (kComp) {  // Kahan's summation of the four products' sum
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int j = 0; j < CP; ++j) {
+            const float y = __fsub_rn(neg ? -acc[u][j] : acc[u][j], cmp[u][j]);
+            const float s = __fadd_rn(tot[u][j], y);
+            cmp[u][j] = __fsub_rn(__fsub_rn(s, tot[u][j]), y);
+            tot[u][j] = s;
+            acc[u][j] = 0.f;
+          }
+      }
+    }
+    if constexpr (!kComp) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int j = 0; j < CP; ++j) tot[u][j] += neg ? -acc[u][j] : acc[u][j];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int lr = kTrans ? 4 * rg + u : rg + 32 * u, row = tile.r0 + lr;
+    if constexpr (kComp)
+#pragma unroll
+      for (int j = 0; j < CP; ++j) tot[u][j] -= cmp[u][j];
+    if (tile.poff >= 0) {  // partial tile of a split box
+#pragma unroll
+      for (int j = 0; j < CP; ++j) {
+        const int n = n0 + cg * CP + j;
+        if (n < a.npad) a.part[tile.poff + (long long)lr * a.npad + n] = tot[u][j];
+      }
+      continue;
+    }
+    if (row >= m) continue;
+    float *dst;
+    long long ld = a.ldx;
+    if (!cell) {
+      dst = a.x + a.idx[gd.idx_off + row];
+    } else if (ph == kMCellBwd) {
+      dst = a.x + a.idx[cd.I_off + row];
+    } else if (row < cd.nI) {
+      dst = a.xI + a.idx[cd.I_off + row];
+    } else {
+      dst = a.contrib + cd.C_off + row - cd.nI;
+      ld = a.ldc;
+    }
+#pragma unroll
+    for (int j = 0; j < CP; ++j) {
+      const int n = n0 + cg * CP + j;
+      if (n < a.ncols) dst[n * ld] = tot[u][j];
+    }
+  }
+}
+
 // the split boxes: rows of a tile added over its K splits in order, then stored
 __global__ void __launch_bounds__(kTM) k_box_reduce(MArgs a, int ph, const RTile *__restrict__ rt) {
   const RTile r = rt[blockIdx.x];
@@ -554,12 +789,13 @@ int build_multi_state(Handle *h, int k) {
     M->grp.assign(L, PhaseWork{});
     M->goff.assign(L, nullptr);
     long long gsz = 0, part = 0;
-    for (int l = lb; l < L; ++l) {
+    for (int l = 0; l < L; ++l) {
       const LevelHost &H = h->lv_host[l];
       std::vector<int2> cf, cb, gr;
       for (const CellDesc &d : H.cells) {
         cf.push_back(make_int2(d.nI + d.nB, d.nI));
-        cb.push_back(make_int2(d.nI, d.nI + d.nB));
+        // the FP32 kernel starts the V rows on a chunk of their own
+        cb.push_back(make_int2(d.nI, (l < lb ? (d.nI + kKC - 1) / kKC * kKC : d.nI) + d.nB));
       }
       std::vector<long long> off(std::max<size_t>(1, H.groups.size()), 0);
       long long o = 0;
@@ -593,8 +829,7 @@ int build_multi_state(Handle *h, int k) {
   return HIF_OK;
 }
 
-int launch_mma(Handle *h, MultiState *M, int ph, int level, const PhaseWork &w, int k, cudaStream_t s) {
-  if (w.ntiles <= 0) return HIF_OK;
+MArgs phase_args(Handle *h, MultiState *M, int level, const PhaseWork &w, int k) {
   const LevelDev *lv = level >= 0 ? &h->lv[level] : nullptr;
   MArgs a{};
   a.tiles = w.tiles;
@@ -603,6 +838,7 @@ int launch_mma(Handle *h, MultiState *M, int ph, int level, const PhaseWork &w, 
   a.groups = lv ? lv->groups : nullptr;
   a.idx = h->idx;
   a.v16 = static_cast<const bf16 *>(h->bf16_vals);
+  a.v32 = h->f32.vals;
   a.gs_off = level >= 0 ? M->goff[level] : nullptr;
   a.root_G_off = h->root_G_off;
   a.ridx = h->idx + h->root_idx_off;
@@ -619,6 +855,45 @@ int launch_mma(Handle *h, MultiState *M, int ph, int level, const PhaseWork &w, 
   a.ldg = M->ldg;
   a.ldr = M->ldr;
   a.err = h->scal + kScalErr;
+  return a;
+}
+
+// the FP32 levels: column tiles of 8, 16 or 32
+template <int NC, bool kTrans, bool kComp>
+int launch_f32_nc(const MArgs &a, int ph, int ntiles, int k, cudaStream_t s) {
+  const size_t sm = kFStages * f32_stage_floats<NC>() * sizeof(float);
+  HIF_CUDA_TRY(cudaFuncSetAttribute(k_box_f32<NC, kTrans, kComp>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)sm));
+  k_box_f32<NC, kTrans, kComp><<<dim3(ntiles, (k + NC - 1) / NC), kFThreads, sm, s>>>(a, ph);
+  return HIF_OK;
+}
+template <bool kTrans, bool kComp>
+int launch_f32_cols(const MArgs &a, int ph, int ntiles, int k, cudaStream_t s) {
+  if (k <= 8) return launch_f32_nc<8, kTrans, kComp>(a, ph, ntiles, k, s);
+  if (k <= 16) return launch_f32_nc<16, kTrans, kComp>(a, ph, ntiles, k, s);
+  return launch_f32_nc<32, kTrans, kComp>(a, ph, ntiles, k, s);
+}
+
+int launch_f32(Handle *h, MultiState *M, int ph, int level, const PhaseWork &w, int k, cudaStream_t s) {
+  if (w.ntiles <= 0) return HIF_OK;
+  const MArgs a = phase_args(h, M, level, w, k);
+  StatScope sc(h, ph == kMCellFwd ? "multi_cell_fwd" : ph == kMCellBwd ? "multi_cell_bwd"
+                  : ph == kMGroupFwd ? "multi_group_fwd" : "multi_group_bwd", level, 0.0, s);
+  if (ph == kMCellBwd && level_uses_sform(h, level)) HIF_TRY((launch_f32_cols<true, true>(a, ph, w.ntiles, k, s)));
+  else if (ph == kMCellBwd || ph == kMGroupBwd) HIF_TRY((launch_f32_cols<true, false>(a, ph, w.ntiles, k, s)));
+  else HIF_TRY((launch_f32_cols<false, false>(a, ph, w.ntiles, k, s)));
+  note_launch();
+  if (w.nrtiles > 0) {
+    k_box_reduce<<<w.nrtiles, kTM, 0, s>>>(a, ph, w.rtiles);
+    note_launch();
+  }
+  HIF_CUDA_TRY(cudaGetLastError());
+  return HIF_OK;
+}
+
+int launch_mma(Handle *h, MultiState *M, int ph, int level, const PhaseWork &w, int k, cudaStream_t s) {
+  if (w.ntiles <= 0) return HIF_OK;
+  const MArgs a = phase_args(h, M, level, w, k);
   const size_t sm = mma_smem_bytes(a.npad);
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_box_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   StatScope sc(h, ph == kMCellFwd ? "mma_cell_fwd" : ph == kMCellBwd ? "mma_cell_bwd"
@@ -677,31 +952,28 @@ int multi_cg_buffers(Handle *h, int k, MultiCG *out) {
   return HIF_OK;
 }
 
-// X (N x k FP32, column-major) <- F^{-1} X: levels below bf16_lb column by
-// column with the single-column FP32 kernels, the BF16 levels and the root
-// for all columns at once on the tensor cores.
+// X (N x k FP32, column-major) <- F^{-1} X for all columns at once: the FP32
+// levels on the FP32 cores, the BF16 levels and the root on the tensor cores.
 int apply_multi_f32(Handle *h, int k, cudaStream_t s) {
   MultiState *M = static_cast<MultiState *>(h->multi);
   const int L = h->L, lb = std::min(h->bf16_lb, L);
-  const long long N = h->N;
-  for (int c = 0; c < k; ++c)
-    HIF_TRY(apply_levels_f32_range(h, h->f32.contrib, M->xI + c * N, M->x + c * N, 0, lb, true, s));
-  for (int l = lb; l < L; ++l) {
-    HIF_TRY(launch_mma(h, M, kMCellFwd, l, M->cf[l], k, s));
+  auto launch_box = [&](int ph, int l, const PhaseWork &w) {
+    return l < lb ? launch_f32(h, M, ph, l, w, k, s) : launch_mma(h, M, ph, l, w, k, s);
+  };
+  for (int l = 0; l < L; ++l) {
+    HIF_TRY(launch_box(kMCellFwd, l, M->cf[l]));
     HIF_TRY(launch_gather(h, M, l, true, k, s));
-    HIF_TRY(launch_mma(h, M, kMGroupFwd, l, M->grp[l], k, s));
+    HIF_TRY(launch_box(kMGroupFwd, l, M->grp[l]));
   }
   if (h->root_n > 0) {
     HIF_TRY(launch_mma(h, M, kMRootRows, -1, M->root, k, s));
     HIF_TRY(launch_mma(h, M, kMRootCols, -1, M->root, k, s));
   }
-  for (int l = L - 1; l >= lb; --l) {
+  for (int l = L - 1; l >= 0; --l) {
     HIF_TRY(launch_gather(h, M, l, false, k, s));
-    HIF_TRY(launch_mma(h, M, kMGroupBwd, l, M->grp[l], k, s));
-    HIF_TRY(launch_mma(h, M, kMCellBwd, l, M->cb[l], k, s));
+    HIF_TRY(launch_box(kMGroupBwd, l, M->grp[l]));
+    HIF_TRY(launch_box(kMCellBwd, l, M->cb[l]));
   }
-  for (int c = 0; c < k; ++c)
-    HIF_TRY(apply_levels_f32_range(h, h->f32.contrib, M->xI + c * N, M->x + c * N, 0, lb, false, s));
   return HIF_OK;
 }
 
