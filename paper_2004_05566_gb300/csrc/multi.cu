@@ -21,7 +21,11 @@
 // issues tcgen05.mma (M = 128, N = k rounded up to 16, K = 16 per
 // instruction, kind::f16 with BF16 operands and FP32 accumulation) and
 // commits each chunk to an mbarrier, so the staging of chunk c + 1 overlaps the
-// products of chunk c.  The accumulator lives in tensor memory (128 lanes x N
+// products of chunk c.  What bounds it is the latency of the staging loads and
+// the stores into the layout: the operands of chunk c + 1 are in registers
+// before chunk c is stored, and a transposed block goes out as 16-byte rows
+// (63^3, 16 columns: level-1 cells backward 283 -> 171 us, forward 154 -> 73 us;
+// root 54 + 52 -> 29 + 37 us).  The accumulator lives in tensor memory (128 lanes x N
 // columns, allocated per CTA) and is read back with tcgen05.ld by the four
 // warps, one 32-lane quarter each.  Every mbarrier wait is bounded; on expiry
 // the CTA records the failure in the handle's error slot and skips its
@@ -140,30 +144,24 @@ __device__ __forceinline__ Box box_of(const MArgs &a, int ph, int unit) {
 }
 
 // Stored row `row` of the block a product reads (A's row for the forward
-// phases, A's column for the transposed ones): its BF16 pointer, the padded
-// length that may be read (zeros beyond the row's own entries), and whether
-// it enters negated.
+// phases, A's column for the transposed ones): its BF16 pointer and the padded
+// length that may be read (zeros beyond the row's own entries).
 struct SRow {
   const bf16 *p;
   int len;
-  bool neg;
 };
 
-__device__ __forceinline__ SRow stored_row(const MArgs &a, int ph, int unit, int row) {
+__device__ __forceinline__ SRow stored_row(const MArgs &a, int ph, const CellDesc &c, const GroupDesc &g, int row) {
   switch (ph) {
     case kMCellFwd:
-    case kMCellBwd: {
-      const CellDesc &c = a.cells[unit];
-      if (row < c.nI) return {a.v16 + c.G_off + tri_off(row), (int)pad4(row + 1), false};
-      return {a.v16 + c.V_off + (long long)(row - c.nI) * pad4(c.nI), (int)pad4(c.nI), ph == kMCellBwd};
-    }
+    case kMCellBwd:
+      if (row < c.nI) return {a.v16 + c.G_off + tri_off(row), (int)pad4(row + 1)};
+      return {a.v16 + c.V_off + (long long)(row - c.nI) * pad4(c.nI), (int)pad4(c.nI)};
     case kMGroupFwd:
-    case kMGroupBwd: {
-      const GroupDesc &g = a.groups[unit];
-      return {a.v16 + g.H_off + (long long)row * pad4(g.n), (int)pad4(g.n), false};
-    }
+    case kMGroupBwd:
+      return {a.v16 + g.H_off + (long long)row * pad4(g.n), (int)pad4(g.n)};
     default:
-      return {a.v16 + a.root_G_off + tri_off(row), (int)pad4(row + 1), false};
+      return {a.v16 + a.root_G_off + tri_off(row), (int)pad4(row + 1)};
   }
 }
 
@@ -171,80 +169,117 @@ __device__ __forceinline__ uint32_t a_off(int i, int kk) {  // i in [0,128), kk 
   return (uint32_t)(kk >> 3) * kLboA + (uint32_t)(i >> 3) * kSbo + (uint32_t)(i & 7) * 16 + (uint32_t)(kk & 7) * 2;
 }
 
-// stage A (tile rows r0.., chunk columns k0..k0+63) into sA
-__device__ __forceinline__ void stage_a(const MArgs &a, int ph, int unit, const Box &bx, int r0, int k0,
-                                        unsigned char *sA) {
+// The thread's share of a chunk of A (tile rows r0.., K k0..k0+63) in
+// registers.  Forward: quads (row t / 16 + 16 j, K 4 (t % 16)).  Transposed:
+// rows i = 4 (t % 32).. of the stored rows k0 + 8 (t / 32) + j, i.e. an
+// 8 (K) x 4 (M) block.
+__device__ __forceinline__ void load_a(const MArgs &a, int ph, bool transposed, const CellDesc &c,
+                                       const GroupDesc &g, const Box &bx, int r0, int k0, uint2 (&v)[8]) {
   const int t = threadIdx.x;
-  const bool transposed = ph == kMCellBwd || ph == kMGroupBwd || ph == kMRootCols;
-  if (!transposed) {
-    // 16 threads per row, 4 elements each (8-byte loads); 8 rows per pass
-    const int q = t & 15, kk = 4 * q;
-    for (int i = t >> 4; i < kTM; i += kMThreads / 16) {
-      const int row = r0 + i;
-      uint2 v = make_uint2(0u, 0u);
-      if (row < bx.m) {
-        const SRow sr = stored_row(a, ph, unit, row);
-        if (k0 + kk < sr.len) v = *reinterpret_cast<const uint2 *>(sr.p + k0 + kk);
-      }
-      *reinterpret_cast<uint2 *>(sA + a_off(i, kk)) = v;
-    }
-  } else {
-    // A(i, kk) = stored row (k0 + kk), element r0 + i: 32 threads per stored
-    // row, 4 consecutive i each; 4 stored rows per pass
-    const int q = t & 31, ii = 4 * q;
-    for (int kk = t >> 5; kk < kKC; kk += kMThreads / 32) {
-      const int srow = k0 + kk;
-      uint2 v = make_uint2(0u, 0u);
-      bool neg = false;
-      if (srow < bx.K) {
-        const SRow sr = stored_row(a, ph, unit, srow);
-        if (r0 + ii < sr.len) v = *reinterpret_cast<const uint2 *>(sr.p + r0 + ii);
-        neg = sr.neg;
-      }
-      if (neg) {
-        v.x ^= 0x80008000u;
-        v.y ^= 0x80008000u;
-      }
-      const unsigned short e[4] = {(unsigned short)(v.x & 0xffffu), (unsigned short)(v.x >> 16),
-                                   (unsigned short)(v.y & 0xffffu), (unsigned short)(v.y >> 16)};
 #pragma unroll
-      for (int u = 0; u < 4; ++u) *reinterpret_cast<unsigned short *>(sA + a_off(ii + u, kk)) = e[u];
+  for (int j = 0; j < 8; ++j) {
+    v[j] = make_uint2(0u, 0u);
+    if (!transposed) {
+      const int row = r0 + (t >> 4) + 16 * j, k = k0 + 4 * (t & 15);
+      if (row < bx.m) {
+        const SRow sr = stored_row(a, ph, c, g, row);
+        if (k < sr.len) v[j] = *reinterpret_cast<const uint2 *>(sr.p + k);
+      }
+    } else {
+      const int row = k0 + 8 * (t >> 5) + j, i = r0 + 4 * (t & 31);
+      if (row < bx.K) {
+        const SRow sr = stored_row(a, ph, c, g, row);
+        if (i < sr.len) v[j] = *reinterpret_cast<const uint2 *>(sr.p + i);
+        if (ph == kMCellBwd && row >= c.nI) {  // -V^T
+          v[j].x ^= 0x80008000u;
+          v[j].y ^= 0x80008000u;
+        }
+      }
     }
   }
 }
 
-// input (row kk of X, column n) of a box
-__device__ __forceinline__ float input_of(const MArgs &a, int ph, int unit, const Box &bx, int kk, int n) {
-  if (kk >= bx.K) return 0.f;
-  switch (ph) {
-    case kMCellFwd: {
-      const CellDesc &c = a.cells[unit];
-      return a.x[n * a.ldx + a.idx[c.I_off + kk]];
-    }
-    case kMCellBwd: {
-      const CellDesc &c = a.cells[unit];
-      if (kk < c.nI) return a.xI[n * a.ldx + a.idx[c.I_off + kk]];
-      return a.x[n * a.ldx + a.idx[c.B_off + kk - c.nI]];
-    }
-    case kMGroupFwd:
-    case kMGroupBwd:
-      return a.gs[n * a.ldg + a.gs_off[unit] + kk];
-    case kMRootRows:
-      return a.x[n * a.ldx + a.ridx[kk]];
-    default:
-      return a.rt[n * a.ldr + kk];
-  }
-}
-
-// stage X_hi and X_lo (chunk rows k0..k0+63, all columns) into sB[0], sB[1]
-__device__ __forceinline__ void stage_b(const MArgs &a, int ph, int unit, const Box &bx, int k0,
-                                       unsigned char *sBh, unsigned char *sBl, uint32_t lboB) {
+// ... and into shared memory.  The transposed block becomes four 16-byte core
+// matrix rows (8 K of one M each); the four go out in an order rotated by lane so
+// that a quarter warp covers all banks (2-byte stores at a stride of 64 bytes
+// were 16-way conflicts, most of the kernel's time).
+__device__ __forceinline__ void store_a(bool transposed, const uint2 (&v)[8], unsigned char *sA) {
   const int t = threadIdx.x;
-  const int kk = t & (kKC - 1);
-  for (int n = t >> 6; n < a.npad; n += kMThreads / kKC) {
-    const float v = n < a.ncols ? input_of(a, ph, unit, bx, k0 + kk, n) : 0.f;
-    const bf16 hi = __float2bfloat16_rn(v);
-    const bf16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
+  if (!transposed) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) *reinterpret_cast<uint2 *>(sA + a_off((t >> 4) + 16 * j, 4 * (t & 15))) = v[j];
+    return;
+  }
+  uint4 o[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const uint32_t lo = u < 2 ? v[2 * e].x : v[2 * e].y, hi = u < 2 ? v[2 * e + 1].x : v[2 * e + 1].y;
+      w[e] = __byte_perm(lo, hi, (u & 1) ? 0x7632 : 0x5410);
+    }
+    o[u] = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  const int q = t & 31, rot = (q >> 1) & 3;
+  if (rot & 1) {
+    const uint4 x = o[0];
+    o[0] = o[1]; o[1] = o[2]; o[2] = o[3]; o[3] = x;
+  }
+  if (rot & 2) {
+    uint4 x = o[0];
+    o[0] = o[2]; o[2] = x;
+    x = o[1];
+    o[1] = o[3]; o[3] = x;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    *reinterpret_cast<uint4 *>(sA + a_off(4 * q + ((u + rot) & 3), 8 * (t >> 5))) = o[u];
+}
+
+// The thread's share of a chunk of X: K index k (-1 row index: absent),
+// columns t / 64 + 4 j.  x_row gives the row of the source vector, load_b the values.
+__device__ __forceinline__ int x_row(const MArgs &a, int ph, const CellDesc &c, const Box &bx, int k) {
+  if (k >= bx.K) return -1;
+  switch (ph) {
+    case kMCellFwd: return a.idx[c.I_off + k];
+    case kMCellBwd: return k < c.nI ? a.idx[c.I_off + k] : a.idx[c.B_off + k - c.nI];
+    case kMRootRows: return a.ridx[k];
+    default: return k;
+  }
+}
+
+template <int NQ>
+__device__ __forceinline__ void load_b(const MArgs &a, int ph, const CellDesc &c, const float *gsrc, int k, int xi,
+                                       float (&v)[NQ]) {
+  const float *src = a.x;
+  long long ld = a.ldx;
+  if (ph == kMCellBwd && k < c.nI) src = a.xI;
+  if (ph == kMGroupFwd || ph == kMGroupBwd) {
+    src = gsrc;
+    ld = a.ldg;
+  }
+  if (ph == kMRootCols) {
+    src = a.rt;
+    ld = a.ldr;
+  }
+#pragma unroll
+  for (int j = 0; j < NQ; ++j) {
+    const int n = ((int)threadIdx.x >> 6) + 4 * j;
+    v[j] = xi >= 0 && n < a.ncols ? src[n * ld + xi] : 0.f;
+  }
+}
+
+// X_hi and X_lo into the canonical layout (K-direction stride padded by 16
+// bytes, as A's)
+template <int NQ>
+__device__ __forceinline__ void store_b(const float (&v)[NQ], unsigned char *sBh, unsigned char *sBl, uint32_t lboB) {
+  const int kk = threadIdx.x & (kKC - 1);
+#pragma unroll
+  for (int j = 0; j < NQ; ++j) {
+    const int n = ((int)threadIdx.x >> 6) + 4 * j;
+    const bf16 hi = __float2bfloat16_rn(v[j]);
+    const bf16 lo = __float2bfloat16_rn(v[j] - __bfloat162float(hi));
     const uint32_t off = (uint32_t)(kk >> 3) * lboB + (uint32_t)(n >> 3) * kSbo + (uint32_t)(n & 7) * 16 +
                          (uint32_t)(kk & 7) * 2;
     *reinterpret_cast<bf16 *>(sBh + off) = hi;
@@ -283,11 +318,12 @@ __device__ __forceinline__ void store_out(const MArgs &a, int ph, int unit, cons
 
 // Dynamic shared memory: kMStages x (A chunk, X_hi chunk, X_lo chunk).
 __host__ __device__ constexpr size_t a_chunk_bytes() { return (size_t)(kKC / 8) * kLboA; }
-__host__ __device__ inline uint32_t b_lbo(int npad) { return (uint32_t)(npad / 8) * kSbo; }
+__host__ __device__ inline uint32_t b_lbo(int npad) { return (uint32_t)(npad / 8) * kSbo + 16; }
 __host__ __device__ inline size_t b_chunk_bytes(int npad) { return (size_t)(kKC / 8) * b_lbo(npad); }
 inline size_t mma_smem_bytes(int npad) { return kMStages * (a_chunk_bytes() + 2 * b_chunk_bytes(npad)); }
 
-__global__ void __launch_bounds__(kMThreads, 2) k_box_mma(MArgs a, int ph) {
+template <int NQ>  // columns padded to 4 NQ
+__global__ void __launch_bounds__(kMThreads, NQ <= 8 ? 3 : 2) k_box_mma(MArgs a, int ph) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint32_t s_tmem;
   __shared__ __align__(8) unsigned long long s_bar[kMStages];
@@ -295,7 +331,14 @@ __global__ void __launch_bounds__(kMThreads, 2) k_box_mma(MArgs a, int ph) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const MTile tile = a.tiles[blockIdx.x];
   const Box bx = box_of(a, ph, tile.unit);
-  const int npad = a.npad;
+  const bool transposed = ph == kMCellBwd || ph == kMGroupBwd || ph == kMRootCols;
+  const bool group = ph == kMGroupFwd || ph == kMGroupBwd;
+  CellDesc cd{};
+  GroupDesc gd{};
+  if (ph == kMCellFwd || ph == kMCellBwd) cd = a.cells[tile.unit];
+  if (group) gd = a.groups[tile.unit];
+  const float *gsrc = group ? a.gs + a.gs_off[tile.unit] : nullptr;
+  constexpr int npad = 4 * NQ;
   const uint32_t ncol_alloc = npad <= 32 ? 32u : (npad <= 64 ? 64u : 128u);
   const uint32_t lboB = b_lbo(npad);
   const size_t stage_bytes = a_chunk_bytes() + 2 * b_chunk_bytes(npad);
@@ -318,6 +361,19 @@ __global__ void __launch_bounds__(kMThreads, 2) k_box_mma(MArgs a, int ph) {
   const int nch = tile.c1 - tile.c0;  // chunks of this CTA (K chunks [c0, c1))
   const uint32_t idesc = mma_idesc(kTM, npad);
   bool ok = true;
+  // chunk c + 1 is loaded into registers while chunk c is stored and multiplied,
+  // and the rows of X it needs are looked up one chunk earlier still: the
+  // loads' latency was what bound the kernel
+  const int kx = t & (kKC - 1);
+  uint2 av[8];
+  float bv[NQ];
+  int xi = -1;
+  if (nch > 0) {
+    const int k0 = tile.c0 * kKC;
+    load_b<NQ>(a, ph, cd, gsrc, k0 + kx, x_row(a, ph, cd, bx, k0 + kx), bv);
+    load_a(a, ph, transposed, cd, gd, bx, tile.r0, k0, av);
+    xi = x_row(a, ph, cd, bx, k0 + kKC + kx);
+  }
   for (int c = 0; c < nch; ++c) {
     const int b = c % kMStages;
     unsigned char *sA = smem + b * stage_bytes;
@@ -328,9 +384,14 @@ __global__ void __launch_bounds__(kMThreads, 2) k_box_mma(MArgs a, int ph) {
       ok = false;
     if (!ok) s_fail = 1;  // benign race: every writer stores 1
     if (ok) {
-      const int k0 = (tile.c0 + c) * kKC;
-      stage_a(a, ph, tile.unit, bx, tile.r0, k0, sA);
-      stage_b(a, ph, tile.unit, bx, k0, sBh, sBl, lboB);
+      store_a(transposed, av, sA);
+      store_b<NQ>(bv, sBh, sBl, lboB);
+      if (c + 1 < nch) {
+        const int k1 = (tile.c0 + c + 1) * kKC;
+        load_b<NQ>(a, ph, cd, gsrc, k1 + kx, xi, bv);
+        load_a(a, ph, transposed, cd, gd, bx, tile.r0, k1, av);
+        xi = x_row(a, ph, cd, bx, k1 + kKC + kx);
+      }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -424,15 +485,18 @@ __global__ void __launch_bounds__(kMThreads, 2) k_box_mma(MArgs a, int ph) {
 // total by Kahan's summation.  Backward cells: the K index runs over the G
 // rows padded to a multiple of 64, then the V rows, whose chunks are
 // subtracted.
-// Measured at 63^3 with 16 columns (level 0, 353 MB of blocks): forward 1720 ->
-// 206 us, backward 1568 -> 263 us per apply.
+// Bound by shared-memory latency at 12 warps an SM, so four CTAs fit an SM
+// (quads of a staged row swizzled instead of padded), and tiles skip the chunks
+// that are zero by the triangle of G.
+// Measured at 63^3 with 16 columns (level 0, 353 MB of blocks), per apply:
+// forward 1720 us column by column, 206 at three CTAs, 165 now; backward 1568,
+// 263, 227.
 constexpr int kFThreads = 128;
 constexpr int kFC = 32;          // K of a staged chunk
 constexpr int kFStages = 3;
-constexpr int kFLdA = kFC + 4;   // floats per staged row of A (conflict-free quads)
 
 template <int NC>
-__host__ __device__ constexpr size_t f32_stage_floats() { return (size_t)kTM * kFLdA + (size_t)kFC * NC; }
+__host__ __device__ constexpr size_t f32_stage_floats() { return (size_t)kTM * kFC + (size_t)kFC * NC; }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool ok) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(su32(dst)), "l"(src), "r"(ok ? 16 : 0)
@@ -455,7 +519,7 @@ __device__ __forceinline__ FRow f32_row(const float *v, const CellDesc &c, const
 }
 
 template <int NC, bool kTrans, bool kComp>
-__global__ void __launch_bounds__(kFThreads) k_box_f32(MArgs a, int ph) {
+__global__ void __launch_bounds__(kFThreads, NC <= 16 ? 4 : 3) k_box_f32(MArgs a, int ph) {
   extern __shared__ __align__(16) float fsm[];
   constexpr int CP = NC / 4;  // columns per thread
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -498,7 +562,7 @@ __global__ void __launch_bounds__(kFThreads) k_box_f32(MArgs a, int ph) {
   auto stage = [&](int c) {
     if (c < c_end) {
       float *sA = fsm + (size_t)((c - c_begin) % kFStages) * f32_stage_floats<NC>();
-      float *sX = sA + (size_t)kTM * kFLdA;
+      float *sX = sA + (size_t)kTM * kFC;
       const int k0 = c * kFC;
       if constexpr (kTrans) {
 #pragma unroll
@@ -516,7 +580,8 @@ __global__ void __launch_bounds__(kFThreads) k_box_f32(MArgs a, int ph) {
         for (int j = 0; j < kSRows; ++j) {
           const int k = k0 + 4 * sq;
           const bool ok = k < fr[j].len;
-          cp_async16(sA + (srow + kSStep * j) * kFLdA + 4 * sq, fr[j].p + (ok ? k : 0), ok);
+          const int r = srow + kSStep * j;  // quads of a row swizzled against bank conflicts
+          cp_async16(sA + r * kFC + 4 * (sq ^ (r & 7)), fr[j].p + (ok ? k : 0), ok);
         }
       }
       const float *src;
@@ -554,7 +619,7 @@ __global__ void __launch_bounds__(kFThreads) k_box_f32(MArgs a, int ph) {
     __syncthreads();
     stage(c + kFStages - 1);
     const float *sA = fsm + (size_t)((c - c_begin) % kFStages) * f32_stage_floats<NC>();
-    const float *sX = sA + (size_t)kTM * kFLdA;
+    const float *sX = sA + (size_t)kTM * kFC;
     const bool neg = c * kFC >= kV;
     float acc[4][CP];
 #pragma unroll
@@ -567,7 +632,7 @@ __global__ void __launch_bounds__(kFThreads) k_box_f32(MArgs a, int ph) {
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const float4 v = *reinterpret_cast<const float4 *>(kTrans ? sA + (kk + u) * kTM + 4 * rg
-                                                                  : sA + (rg + 32 * u) * kFLdA + kk);
+                                                                  : sA + (rg + 32 * u) * kFC + (kk ^ (4 * (rg & 7))));
         av[u][0] = v.x; av[u][1] = v.y; av[u][2] = v.z; av[u][3] = v.w;
       }
 #pragma unroll
@@ -715,10 +780,10 @@ struct MultiState {
   long long ldc = 0, ldg = 0, ldr = 0;
   // per top level: the work of the cell forward, cell backward and entity
   // phases (the entity forward and backward share theirs), per-entity gs
-  // offsets; the root's (rows and columns share it)
+  // offsets; the root's rows and columns
   std::vector<PhaseWork> cf, cb, grp;
   std::vector<long long *> goff;
-  PhaseWork root;
+  PhaseWork root, root_t;
   float *tpart = nullptr;  // partial tiles of split boxes (largest phase)
 };
 
@@ -739,31 +804,41 @@ int upload_vec(Handle *h, const std::vector<T> &v, T **out) {
   return HIF_OK;
 }
 
-// CTAs of a phase whose boxes have (m, K) = sizes[u]: every 128-row tile; a
-// phase with few tiles splits K so that about kTargetCtas CTAs run (at least
-// 4 chunks per split), the splits of a tile adding up in k_box_reduce.
-int build_phase(Handle *h, const std::vector<int2> &sizes, PhaseWork *w) {
+// A box's operator: m rows, K; tri > 0: its first tri rows are lower
+// triangular (row r ends at K index r), tri < 0: its columns start at the
+// diagonal (row r begins at K index r).
+struct BoxSize {
+  int m, K, tri;
+};
+
+// CTAs of a phase: every 128-row tile of every box, over the K chunks that are
+// not zero by the triangle; a phase with few tiles splits K so that about
+// kTargetCtas CTAs run (at least 4 chunks per split), the splits of a tile
+// adding up in k_box_reduce.
+int build_phase(Handle *h, const std::vector<BoxSize> &sizes, PhaseWork *w) {
   constexpr int kTargetCtas = 3 * 152;
   long long T = 0;
-  for (const int2 &mk : sizes) T += (mk.x + kTM - 1) / kTM;
+  for (const BoxSize &b : sizes) T += (b.m + kTM - 1) / kTM;
   const int ks = (int)std::max<long long>(1, std::min<long long>(16, (kTargetCtas + T - 1) / std::max<long long>(T, 1)));
   std::vector<MTile> tiles;
   std::vector<RTile> rts;
   long long poff = 0;
   for (int u = 0; u < (int)sizes.size(); ++u) {
-    const int m = sizes[u].x, K = sizes[u].y;
-    const int nch = (K + kKC - 1) / kKC;
-    int nks = std::max(1, std::min(ks, nch / 4));
-    const int cps = nks > 1 ? (nch + nks - 1) / nks : nch;
-    nks = nks > 1 ? (nch + cps - 1) / cps : 1;
+    const int m = sizes[u].m, K = sizes[u].K, tri = sizes[u].tri;
     for (int r = 0; r < m; r += kTM) {
+      const int lo = tri < 0 ? r / kKC : 0;
+      const int hi = tri > 0 && r + kTM <= tri ? (r + kTM + kKC - 1) / kKC : (K + kKC - 1) / kKC;
+      const int nch = hi - lo;
+      int nks = std::max(1, std::min(ks, nch / 4));
+      const int cps = nks > 1 ? (nch + nks - 1) / nks : nch;
+      nks = nks > 1 ? (nch + cps - 1) / cps : 1;
       if (nks == 1) {
-        tiles.push_back({u, r, 0, nch, -1});
+        tiles.push_back({u, r, lo, hi, -1});
         continue;
       }
       rts.push_back({u, r, nks, 0, poff});
       for (int k = 0; k < nks; ++k) {
-        tiles.push_back({u, r, k * cps, std::min(nch, (k + 1) * cps), poff});
+        tiles.push_back({u, r, lo + k * cps, lo + std::min(nch, (k + 1) * cps), poff});
         poff += kPartTile;
       }
     }
@@ -791,18 +866,18 @@ int build_multi_state(Handle *h, int k) {
     long long gsz = 0, part = 0;
     for (int l = 0; l < L; ++l) {
       const LevelHost &H = h->lv_host[l];
-      std::vector<int2> cf, cb, gr;
+      std::vector<BoxSize> cf, cb, gr;
       for (const CellDesc &d : H.cells) {
-        cf.push_back(make_int2(d.nI + d.nB, d.nI));
+        cf.push_back({d.nI + d.nB, d.nI, d.nI});
         // the FP32 kernel starts the V rows on a chunk of their own
-        cb.push_back(make_int2(d.nI, (l < lb ? (d.nI + kKC - 1) / kKC * kKC : d.nI) + d.nB));
+        cb.push_back({d.nI, (l < lb ? (d.nI + kKC - 1) / kKC * kKC : d.nI) + d.nB, -1});
       }
       std::vector<long long> off(std::max<size_t>(1, H.groups.size()), 0);
       long long o = 0;
       for (int g = 0; g < (int)H.groups.size(); ++g) {
         off[g] = o;
         o += pad4(H.groups[g].n);
-        gr.push_back(make_int2(H.groups[g].n, H.groups[g].n));
+        gr.push_back({H.groups[g].n, H.groups[g].n, 0});
       }
       gsz = std::max(gsz, o);
       HIF_TRY(build_phase(h, cf, &M->cf[l]));
@@ -812,8 +887,11 @@ int build_multi_state(Handle *h, int k) {
       HIF_TRY(dev_alloc(h, (void **)&M->goff[l], off.size() * sizeof(long long)));
       HIF_CUDA_TRY(cudaMemcpy(M->goff[l], off.data(), off.size() * sizeof(long long), cudaMemcpyHostToDevice));
     }
-    if (h->root_n > 0) HIF_TRY(build_phase(h, {make_int2(h->root_n, h->root_n)}, &M->root));
-    part = std::max(part, M->root.part_floats);
+    if (h->root_n > 0) {
+      HIF_TRY(build_phase(h, {{h->root_n, h->root_n, h->root_n}}, &M->root));
+      HIF_TRY(build_phase(h, {{h->root_n, h->root_n, -1}}, &M->root_t));
+    }
+    part = std::max({part, M->root.part_floats, M->root_t.part_floats});
     HIF_TRY(dev_alloc(h, (void **)&M->tpart, (size_t)std::max<long long>(part, 4) * sizeof(float)));
     M->ldg = std::max<long long>(gsz, 4);
   }
@@ -895,12 +973,13 @@ int launch_mma(Handle *h, MultiState *M, int ph, int level, const PhaseWork &w, 
   if (w.ntiles <= 0) return HIF_OK;
   const MArgs a = phase_args(h, M, level, w, k);
   const size_t sm = mma_smem_bytes(a.npad);
-  HIF_CUDA_TRY(cudaFuncSetAttribute(k_box_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  auto kern = a.npad == 16 ? k_box_mma<4> : a.npad == 32 ? k_box_mma<8> : a.npad == 48 ? k_box_mma<12> : k_box_mma<16>;
+  HIF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   StatScope sc(h, ph == kMCellFwd ? "mma_cell_fwd" : ph == kMCellBwd ? "mma_cell_bwd"
                   : ph == kMGroupFwd ? "mma_group_fwd" : ph == kMGroupBwd ? "mma_group_bwd"
                   : ph == kMRootRows ? "mma_root_rows" : "mma_root_cols",
                level, 0.0, s);
-  k_box_mma<<<w.ntiles, kMThreads, sm, s>>>(a, ph);
+  kern<<<w.ntiles, kMThreads, sm, s>>>(a, ph);
   note_launch();
   if (w.nrtiles > 0) {
     k_box_reduce<<<w.nrtiles, kTM, 0, s>>>(a, ph, w.rtiles);
@@ -967,7 +1046,7 @@ int apply_multi_f32(Handle *h, int k, cudaStream_t s) {
   }
   if (h->root_n > 0) {
     HIF_TRY(launch_mma(h, M, kMRootRows, -1, M->root, k, s));
-    HIF_TRY(launch_mma(h, M, kMRootCols, -1, M->root, k, s));
+    HIF_TRY(launch_mma(h, M, kMRootCols, -1, M->root_t, k, s));
   }
   for (int l = L - 1; l >= 0; --l) {
     HIF_TRY(launch_gather(h, M, l, false, k, s));
