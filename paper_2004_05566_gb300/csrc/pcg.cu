@@ -17,7 +17,7 @@
 
 namespace hifcn {
 
-int cn_rhs(Handle *h, const double *u, const double *r, double *g, cudaStream_t s);
+int cn_rhs(Handle *h, const double *u, const double *r, double *g, cudaStream_t s, int ncols = 1);
 int apply_inplace_f64(Handle *h, double *x, cudaStream_t s);
 extern "C" int64_t hif_launch_count(void);
 int apply_inplace_f32(Handle *h, float *x, cudaStream_t s);
@@ -158,12 +158,27 @@ __global__ void __launch_bounds__(NT) k_resid_norm(const double *__restrict__ b,
   if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
+// The vector kernels of a solve also run for the columns of cn_step_multi in
+// one launch (kCols): grid.y = column, vectors N apart, scalars 16, tickets 4,
+// partials pstride; a converged column returns at once.  One launch per column
+// and kernel left a small operator waiting on launches (cn_step_multi at 63^3,
+// 16 states: 8.81 ms, 7.21 in one launch).
+constexpr int kColScal = 16, kColTickets = 4;
+
 // start: x = 0, r = b, zin = b, partial b.b
-template <typename TZ>
+template <typename TZ, bool kCols = false>
 __global__ void __launch_bounds__(NT) k_start(const double *__restrict__ b, double *__restrict__ x,
                                               double *__restrict__ r, TZ *__restrict__ zin, long long N,
-                                              double *__restrict__ part) {
+                                              double *__restrict__ part, int pstride) {
   __shared__ double sm[NT / 32];
+  if constexpr (kCols) {
+    const long long o = blockIdx.y * N;
+    b += o;
+    x += o;
+    r += o;
+    zin += o;
+    part += (long long)blockIdx.y * pstride;
+  }
   double acc = 0.0;
   for (long long j = blockIdx.x * (long long)NT + threadIdx.x; j < N; j += (long long)gridDim.x * NT) {
     double bj = b[j];
@@ -187,9 +202,13 @@ __global__ void __launch_bounds__(NT) k_start(const double *__restrict__ b, doub
 // loop runs the same kernels.
 
 // prologue scalar phase: b.b, counters, and the loop condition (b != 0)
-template <bool kGraph>
+template <bool kGraph, bool kCols = false>
 __global__ void k_scalar_start(double *__restrict__ s, const double *__restrict__ part, int np,
-                               cudaGraphConditionalHandle cond) {
+                               cudaGraphConditionalHandle cond, int pstride) {
+  if constexpr (kCols) {
+    s += blockIdx.x * kColScal;
+    part += (long long)blockIdx.x * pstride;
+  }
   double v = warp_sum_partials(part, np);
   if (threadIdx.x != 0) return;
   s[S_BB] = v;
@@ -404,13 +423,24 @@ __device__ __forceinline__ void wz_load(int j, int N, int S, int S2, const GridW
 
 // first kernel: w = A z, partials of r.z, w.z and q.z; the last block forms
 // beta, sigma and alpha
-template <typename TZ, bool D3>
+template <typename TZ, bool D3, bool kCols = false>
 __global__ void __launch_bounds__(NT) k_cg_wz(const double *__restrict__ r, const TZ *__restrict__ z,
                                               double *__restrict__ w, const double *__restrict__ q,
                                               StencilArgs st, double *__restrict__ part,
-                                              double *__restrict__ s, unsigned *__restrict__ ticket) {
+                                              double *__restrict__ s, unsigned *__restrict__ ticket, int pstride) {
   __shared__ double sm[3 * NT];
   cg_pdl_enter();
+  if constexpr (kCols) {
+    s += blockIdx.y * kColScal;
+    if (s[S_CONV] != 0.0) return;
+    const long long o = blockIdx.y * st.N;
+    r += o;
+    z += o;
+    w += o;
+    q += o;
+    part += (long long)blockIdx.y * pstride;
+    ticket += blockIdx.y * kColTickets;
+  }
   double arz = 0.0, awz = 0.0, aqz = 0.0;
   const bool first = s[S_IT] == 0.0;  // q holds no direction yet
   const int N = (int)st.N, S = st.n - 1, S2 = S * S;
@@ -502,17 +532,30 @@ __device__ __forceinline__ void upd_load(int j, int n, bool first, const TZ *zin
 // unless this iteration recomputes the true residual) the end-of-iteration
 // scalar phase.  z and zin are the same buffer: each element is read (one
 // element ahead, by the same thread) before it is overwritten.
-template <typename TZ, bool kGraph>
+template <typename TZ, bool kGraph, bool kCols = false>
 __global__ void __launch_bounds__(NT) k_cg_update(double *__restrict__ x, double *__restrict__ r,
                                                   double *__restrict__ p, double *__restrict__ q,
                                                   const double *__restrict__ w, TZ *zin,
                                                   double *__restrict__ s, long long N,
                                                   double *__restrict__ part, unsigned *__restrict__ ticket,
                                                   int period, double tol2, int maxit,
-                                                  cudaGraphConditionalHandle cond) {
+                                                  cudaGraphConditionalHandle cond, int pstride) {
   __shared__ double sm[NT];
   __shared__ int s_flags;  // bit 0: first iteration, bit 1: the true residual follows
   cg_pdl_enter();
+  if constexpr (kCols) {
+    s += blockIdx.y * kColScal;
+    if (s[S_CONV] != 0.0) return;
+    const long long o = blockIdx.y * N;
+    x += o;
+    r += o;
+    p += o;
+    q += o;
+    w += o;
+    zin += o;
+    part += (long long)blockIdx.y * pstride;
+    ticket += blockIdx.y * kColTickets;
+  }
   if (threadIdx.x == 0) {
     const int it1 = (int)s[S_IT] + 1;  // iteration that updates x now
     s_flags = (it1 == 1 ? 1 : 0) | ((period > 0 && it1 % period == 0) ? 2 : 0);
@@ -559,18 +602,18 @@ template <typename TZ>
 cudaError_t launch_cg_wz(bool pdl, int nb, cudaStream_t s, const double *r, const TZ *z, double *w,
                          const double *q, const StencilArgs &st, double *part, double *sc, unsigned *tk) {
   if (st.dim == 3) {
-    if (pdl) return launch_cg(k_cg_wz<TZ, true>, nb, NT, s, r, z, w, q, st, part, sc, tk);
-    k_cg_wz<TZ, true><<<nb, NT, 0, s>>>(r, z, w, q, st, part, sc, tk);
+    if (pdl) return launch_cg(k_cg_wz<TZ, true>, nb, NT, s, r, z, w, q, st, part, sc, tk, 0);
+    k_cg_wz<TZ, true><<<nb, NT, 0, s>>>(r, z, w, q, st, part, sc, tk, 0);
   } else {
-    if (pdl) return launch_cg(k_cg_wz<TZ, false>, nb, NT, s, r, z, w, q, st, part, sc, tk);
-    k_cg_wz<TZ, false><<<nb, NT, 0, s>>>(r, z, w, q, st, part, sc, tk);
+    if (pdl) return launch_cg(k_cg_wz<TZ, false>, nb, NT, s, r, z, w, q, st, part, sc, tk, 0);
+    k_cg_wz<TZ, false><<<nb, NT, 0, s>>>(r, z, w, q, st, part, sc, tk, 0);
   }
   return cudaGetLastError();
 }
 
 // every `period` iterations: r = b - A x, z-input = r, r.r and the
 // end-of-iteration scalar phase (a no-op launch otherwise)
-template <typename TZ, bool kGraph>
+template <typename TZ, bool kGraph, bool kCols = false>
 __global__ void __launch_bounds__(NT) k_true_residual_cond(const double *__restrict__ b,
                                                            const double *__restrict__ x,
                                                            double *__restrict__ r,
@@ -578,12 +621,23 @@ __global__ void __launch_bounds__(NT) k_true_residual_cond(const double *__restr
                                                            double *__restrict__ s, int period,
                                                            double *__restrict__ part,
                                                            unsigned *__restrict__ ticket, double tol2,
-                                                           int maxit, cudaGraphConditionalHandle cond) {
+                                                           int maxit, cudaGraphConditionalHandle cond,
+                                                           int pstride) {
   // only after an update kernel that left the iteration to this one (its
   // count is not advanced yet); every block reads the flag before the last
   // block clears it
   (void)period;
   cg_pdl_enter();
+  if constexpr (kCols) {
+    s += blockIdx.y * kColScal;
+    const long long o = blockIdx.y * st.N;
+    b += o;
+    x += o;
+    r += o;
+    zin += o;
+    part += (long long)blockIdx.y * pstride;
+    ticket += blockIdx.y * kColTickets;
+  }
   if (s[S_TRUE] == 0.0) return;
   __shared__ double sm[NT / 32];
   double acc = 0.0;
@@ -694,8 +748,8 @@ int build_pcg_graph(Handle *h, TZ *z, PcgGraph *G, bool warm) {
     k_start_warm<TZ><<<nb, NT, 0, cs>>>(h->g, h->xsol, h->r, z, st, part, part + nb);
     k_scalar_start_warm<true><<<1, 32, 0, cs>>>(sc, part, part + nb, nb, tol2, h->xsol, N, cond);
   } else {
-    k_start<TZ><<<nb, NT, 0, cs>>>(h->g, h->xsol, h->r, z, N, part);
-    k_scalar_start<true><<<1, 32, 0, cs>>>(sc, part, nb, cond);
+    k_start<TZ><<<nb, NT, 0, cs>>>(h->g, h->xsol, h->r, z, N, part, 0);
+    k_scalar_start<true><<<1, 32, 0, cs>>>(sc, part, nb, cond, 0);
   }
   HIF_CUDA_TRY(cudaStreamGetCaptureInfo(cs, &cst, nullptr, &graph, &deps, nullptr, &ndeps));
   cudaGraphNodeParams cp = {};
@@ -718,10 +772,10 @@ int build_pcg_graph(Handle *h, TZ *z, PcgGraph *G, bool warm) {
   const int nbc = h->nblocks_cg;
   HIF_CUDA_TRY(launch_cg_wz<TZ>(true, nbc, cs, h->r, z, h->w, h->q, st, part, sc, tk));
   HIF_CUDA_TRY(launch_cg(k_cg_update<TZ, true>, nbc, NT, cs, h->xsol, h->r, h->p, h->q, (const double *)h->w, z,
-                         sc, N, part, tk + 2, h->opt.true_res_period, tol2, h->opt.cg_maxit, cond));
+                         sc, N, part, tk + 2, h->opt.true_res_period, tol2, h->opt.cg_maxit, cond, 0));
   HIF_CUDA_TRY(launch_cg(k_true_residual_cond<TZ, true>, nb, NT, cs, (const double *)h->g,
                          (const double *)h->xsol, h->r, z, st, sc, h->opt.true_res_period, part, tk + 3, tol2,
-                         h->opt.cg_maxit, cond));
+                         h->opt.cg_maxit, cond, 0));
   note_launch(3);
   cudaGraph_t body_out = nullptr;
   cudaError_t e_end = cudaStreamEndCapture(cs, &body_out);
@@ -802,8 +856,8 @@ int pcg_impl(Handle *h, const double *b, double *x, TZ *z, int *iters_out, doubl
     k_start_warm<TZ><<<nb, NT, 0, s>>>(b, x, h->r, z, st, part, part + nb);
     k_scalar_start_warm<false><<<1, 32, 0, s>>>(sc, part, part + nb, nb, tol2, x, N, 0);
   } else {
-    k_start<TZ><<<nb, NT, 0, s>>>(b, x, h->r, z, N, part);
-    k_scalar_start<false><<<1, 32, 0, s>>>(sc, part, nb, 0);
+    k_start<TZ><<<nb, NT, 0, s>>>(b, x, h->r, z, N, part, 0);
+    k_scalar_start<false><<<1, 32, 0, s>>>(sc, part, nb, 0, 0);
   }
   note_launch(2);
   HIF_CUDA_TRY(cudaMemcpyAsync(h->host_scal, sc, 16 * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -827,9 +881,9 @@ int pcg_impl(Handle *h, const double *b, double *x, TZ *z, int *iters_out, doubl
     HIF_TRY(precond(z));
     HIF_CUDA_TRY(launch_cg_wz<TZ>(false, h->nblocks_cg, s, h->r, z, h->w, h->q, st, part, sc, tk));
     k_cg_update<TZ, false><<<h->nblocks_cg, NT, 0, s>>>(x, h->r, h->p, h->q, h->w, z, sc, N, part, tk + 2, period,
-                                            tol2, h->opt.cg_maxit, 0);
+                                            tol2, h->opt.cg_maxit, 0, 0);
     k_true_residual_cond<TZ, false><<<nb, NT, 0, s>>>(b, x, h->r, z, st, sc, period, part, tk + 3, tol2,
-                                                     h->opt.cg_maxit, 0);
+                                                     h->opt.cg_maxit, 0, 0);
     note_launch(3);
     ++it;
     HIF_CUDA_TRY(cudaGetLastError());
@@ -915,7 +969,7 @@ int cn(Handle *h, const double *u, const double *r, double *u1, int *iters, cuda
 // share every application of the preconditioner (one multi-column apply per
 // iteration, the BF16 top levels on the tensor cores).  A column that has
 // converged stops updating; the loop ends when none is active.  The vector
-// kernels are those of the single-column solve, launched per active column.
+// kernels are those of the single-column solve, launched over all columns.
 int cn_cols(Handle *h, const double *U, const double *R, double *U1, int k, int *iters, cudaStream_t s) {
   HIF_TRY(multi_check(h, k, "cn_step_multi"));
   if (h->opt.x0_mode != 0 || h->opt.solver != 0) {
@@ -929,24 +983,23 @@ int cn_cols(Handle *h, const double *U, const double *R, double *U1, int k, int 
   StencilArgs st{h->diag, h->wx, h->wy, h->wz, h->grid.dim, h->grid.n, N};
   const double tol2 = h->opt.cg_tol * h->opt.cg_tol;
   const int period = h->opt.true_res_period;
-  std::vector<double> sc((size_t)16 * k);
-  for (int c = 0; c < k; ++c) {
-    double *g = C.g + c * N;
-    HIF_TRY(cn_rhs(h, U + c * N, R ? R + c * N : nullptr, g, s));
-    k_start<float><<<nb, NT, 0, s>>>(g, C.x + c * N, C.r + c * N, C.z + c * N, N, C.part + 4LL * nb * c);
-    k_scalar_start<false><<<1, 32, 0, s>>>(C.scal + 16 * c, C.part + 4LL * nb * c, nb, 0);
-    note_launch(2);
-  }
+  const int pst = 4 * nb;
+  std::vector<double> sc((size_t)kColScal * k);
+  HIF_TRY(cn_rhs(h, U, R, C.g, s, k));
+  k_start<float, true><<<dim3(nb, k), NT, 0, s>>>(C.g, C.x, C.r, C.z, N, C.part, pst);
+  k_scalar_start<false, true><<<k, 32, 0, s>>>(C.scal, C.part, nb, 0, pst);
+  note_launch(2);
   HIF_CUDA_TRY(cudaGetLastError());
   HIF_CUDA_TRY(cudaMemcpyAsync(sc.data(), C.scal, sc.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   HIF_CUDA_TRY(cudaStreamSynchronize(s));
   std::vector<char> active(k);
   int nactive = 0;
   for (int c = 0; c < k; ++c) {
-    active[c] = sc[16 * c + S_BB] > 0.0;
+    active[c] = sc[kColScal * c + S_BB] > 0.0;
     nactive += active[c];
     if (iters) iters[c] = 0;
   }
+  const dim3 grid(h->nblocks_cg, k);
   int status = HIF_OK;
   for (int it = 0; nactive > 0; ++it) {
     if (it >= h->opt.cg_maxit) {
@@ -954,19 +1007,17 @@ int cn_cols(Handle *h, const double *U, const double *R, double *U1, int k, int 
       break;
     }
     HIF_TRY(apply_multi_f32(h, k, s));
-    for (int c = 0; c < k; ++c) {
-      if (!active[c]) continue;
-      double *sct = C.scal + 16 * c, *part = C.part + 4LL * nb * c;
-      unsigned *tk = C.tk + 4 * c;
-      float *z = C.z + c * N;
-      HIF_CUDA_TRY(launch_cg_wz<float>(false, h->nblocks_cg, s, C.r + c * N, z, C.w + c * N, C.q + c * N, st,
-                                       part, sct, tk));
-      k_cg_update<float, false><<<h->nblocks_cg, NT, 0, s>>>(C.x + c * N, C.r + c * N, C.p + c * N, C.q + c * N,
-                                                  C.w + c * N, z, sct, N, part, tk + 2, period, tol2,
-                                                  h->opt.cg_maxit, 0);
-      k_true_residual_cond<float, false><<<nb, NT, 0, s>>>(C.g + c * N, C.x + c * N, C.r + c * N, z, st, sct,
-                                                         period, part, tk + 3, tol2, h->opt.cg_maxit, 0);
-      note_launch(3);
+    if (st.dim == 3)
+      k_cg_wz<float, true, true><<<grid, NT, 0, s>>>(C.r, C.z, C.w, C.q, st, C.part, C.scal, C.tk, pst);
+    else
+      k_cg_wz<float, false, true><<<grid, NT, 0, s>>>(C.r, C.z, C.w, C.q, st, C.part, C.scal, C.tk, pst);
+    k_cg_update<float, false, true><<<grid, NT, 0, s>>>(C.x, C.r, C.p, C.q, C.w, C.z, C.scal, N, C.part, C.tk + 2,
+                                                        period, tol2, h->opt.cg_maxit, 0, pst);
+    note_launch(2);
+    if (period > 0 && (it + 1) % period == 0) {  // the active columns are all at this iteration
+      k_true_residual_cond<float, false, true><<<dim3(nb, k), NT, 0, s>>>(
+          C.g, C.x, C.r, C.z, st, C.scal, period, C.part, C.tk + 3, tol2, h->opt.cg_maxit, 0, pst);
+      note_launch();
     }
     HIF_CUDA_TRY(cudaGetLastError());
     HIF_CUDA_TRY(cudaMemcpyAsync(sc.data(), C.scal, sc.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -975,15 +1026,14 @@ int cn_cols(Handle *h, const double *U, const double *R, double *U1, int k, int 
     if (h->host_scal[kScalErr] != 0.0) return take_timeout(h);
     for (int c = 0; c < k; ++c) {
       if (!active[c]) continue;
-      if (iters) iters[c] = (int)sc[16 * c + S_IT];
-      if (sc[16 * c + S_CONV] != 0.0) {
+      if (iters) iters[c] = (int)sc[kColScal * c + S_IT];
+      if (sc[kColScal * c + S_CONV] != 0.0) {
         active[c] = 0;
         --nactive;
       }
     }
   }
-  for (int c = 0; c < k; ++c)
-    HIF_CUDA_TRY(cudaMemcpyAsync(U1 + c * N, C.x + c * N, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  HIF_CUDA_TRY(cudaMemcpyAsync(U1, C.x, (size_t)k * N * sizeof(double), cudaMemcpyDeviceToDevice, s));
   HIF_CUDA_TRY(cudaStreamSynchronize(s));
   return status;
 }

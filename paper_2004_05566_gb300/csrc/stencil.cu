@@ -58,6 +58,10 @@ __global__ void k_cn_rhs(const double *__restrict__ u, const double *__restrict_
                          const double *__restrict__ wx, const double *__restrict__ wy,
                          const double *__restrict__ wz, int dim, int n, long long N, double dt,
                          int kind, double k1, double inv_k2, double kappa) {
+  // grid.y: states N apart (cn_step_multi)
+  u += blockIdx.y * N;
+  g += blockIdx.y * N;
+  if (r) r += blockIdx.y * N;
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < N;
        j += (long long)gridDim.x * blockDim.x) {
     double uj = u[j];
@@ -103,10 +107,10 @@ int stencil_matvec(Handle *h, const double *x, double *y, cudaStream_t s) {
   return HIF_OK;
 }
 
-int cn_rhs(Handle *h, const double *u, const double *r, double *g, cudaStream_t s) {
+int cn_rhs(Handle *h, const double *u, const double *r, double *g, cudaStream_t s, int ncols) {
   double inv_k2 = h->react_k2 == 0.0 ? 0.0 : 1.0 / h->react_k2;
   const double kappa = (1.0 - h->opt.theta) / h->opt.theta;
-  k_cn_rhs<<<h->nblocks_vec, 256, 0, s>>>(u, r, g, h->diag, h->wx, h->wy, h->wz, h->grid.dim,
+  k_cn_rhs<<<dim3(h->nblocks_vec, ncols), 256, 0, s>>>(u, r, g, h->diag, h->wx, h->wy, h->wz, h->grid.dim,
                                           h->grid.n, h->N, h->dt, h->react_kind, h->react_k1,
                                           inv_k2, kappa);
   note_launch();
