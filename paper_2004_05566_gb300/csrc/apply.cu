@@ -3157,7 +3157,9 @@ int make_cell_inverses(Handle *h, cudaStream_t s) {
     bool stored = true;  // every cell of the level has room for S
     for (const CellDesc &c : h->lv_host[l].cells) stored = stored && c.S_off >= 0;
     if (!stored) continue;
-    if (!h->lean_setup) {  // a streaming setup formed S before dropping the FP64 values
+    // a streaming setup formed S before dropping the FP64 values, the leaf
+    // elimination forms its own
+    if (!h->lean_setup && !(l == 0 && h->leaf_S)) {
       k_make_S<<<lv.ncells, 256, 0, s>>>(lv.cells, h->f64.vals);
       note_launch();
     }

@@ -339,6 +339,7 @@ struct hif_handle {
   // (S formed first) and dropped the FP64 values: the handle is as after
   // hif_release_fp64 from the start
   bool lean_setup = false;
+  bool leaf_S = false;  // the setup's leaf elimination formed S of level 0
   long long device_bytes = 0;
   // allocations [factor_alloc_begin, end) belong to the factor (released by
   // hif_refactor); work_device_bytes is device_bytes without them

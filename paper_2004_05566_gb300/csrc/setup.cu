@@ -35,6 +35,7 @@
 #include "internal.h"
 #include "device_common.cuh"
 #include "dense_batched.cuh"
+#include "leaf_factor.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -832,12 +833,13 @@ int gpu_setup(Handle *h, const double *a_nodes, cudaStream_t s) {
   const char *lean_env = std::getenv("HIFCN_LEAN_SETUP");
   const int lean_mode = !reduced ? 0 : !lean_env ? -1 : (lean_env[0] == '1' ? 1 : 0);  // -1: by memory
   h->lean_setup = false;
+  h->leaf_S = false;
   bool lean = false;
   std::vector<float *> level_f32(L + 1, nullptr);
   std::vector<unsigned short *> level_b16(L + 1, nullptr);
   auto stream_level = [&](int k) -> int {
     if (!level_vals[k]) return HIF_OK;
-    if (k < L && !h->lv_host[k].cells.empty() && h->lv_host[k].cells[0].S_off >= 0) {
+    if (k < L && !(k == 0 && h->leaf_S) && !h->lv_host[k].cells.empty() && h->lv_host[k].cells[0].S_off >= 0) {
       Scratch tmp;
       CellDesc *dc = nullptr;
       HIF_TRY(tmp.upload(&dc, h->lv_host[k].cells, s));
@@ -1000,7 +1002,20 @@ int gpu_setup(Handle *h, const double *a_nodes, cudaStream_t s) {
     // assemble (level 0 from the stencil, above by extend-add of the children's
     // Schur complements), eliminate the interiors, keep X_BB
     std::vector<int> fchunk = {0};
-    {
+    // the leaf level straight from the stencil where its bands fit shared memory
+    int max_leaf_nB = 0, band = 0;
+    size_t leaf_smem = 0;
+    for (auto &C : cells) max_leaf_nB = std::max(max_leaf_nB, C.nB);
+    const bool leaf_direct = l == 0 && l < L && leaf::supported(dim, leaf, max_leaf_nB, &band, &leaf_smem);
+    if (leaf_direct) {
+      const long long stride = want_S ? 0 : tri_off(level_max_nI);
+      const long long cap = std::max(setup_budget("HIFCN_SETUP_FRONT_BYTES", 0.6) / (long long)sizeof(double), 1LL);
+      const int per = stride ? (int)std::max(1LL, std::min<long long>(ncells, cap / stride)) : ncells;
+      for (int c0 = per; c0 < ncells; c0 += per) fchunk.push_back(c0);
+      fchunk.push_back(ncells);
+      foff = stride * per;
+      h->leaf_S = want_S;
+    } else {
       const long long front_cap = setup_budget("HIFCN_SETUP_FRONT_BYTES", 0.6);
       long long run = 0, maxrun = 0, cap = std::max(front_cap / (long long)sizeof(double), 1LL);
       for (int c = 0; c < ncells; ++c) {
@@ -1024,6 +1039,11 @@ int gpu_setup(Handle *h, const double *a_nodes, cudaStream_t s) {
     for (auto &C : cells) max_np = std::max(max_np, C.nI + C.nB);
     for (size_t k = 0; k + 1 < fchunk.size(); ++k) {
       const int c0 = fchunk[k], nck = fchunk[k + 1] - c0;
+      if (leaf_direct) {
+        HIF_TRY(leaf::factor_cells(dcells, c0, nck, dcdofs, h->diag, h->wx, h->wy, h->wz, dim, n, P.s, P.nc, band,
+                                   leaf_smem, vals, Fc, want_S ? 0 : tri_off(level_max_nI), Fb, derr, s));
+        continue;
+      }
       if (l == 0) {
         const int box = P.s + 1;
         size_t sm = sizeof(int) * (dim == 3 ? (size_t)box * box * box : (size_t)box * box);
