@@ -84,9 +84,20 @@ struct SGroup {
 struct SSkel {        // one skeletonized group of a sub-step
   int g;              // group id
   int R;              // rows of A~_{R,g}
-  long long row_off;  // into rowptr (R + 1 entries)
+  int rg0, nrg;       // its row groups
   long long ws_off;   // workspace (doubles)
   long long perm_off; // output pivot order (n ints)
+};
+
+// The rows of A~_{R,g} are the surviving DOFs of the other entities on the
+// boundaries of g's cells, entity by entity: rows [row0, row0 + n) are the DOFs
+// pos[pos_off + i] of one entity, which sits at offset occ.y in the boundary of
+// the occ.x-th of g's cells for each of its nocc occurrences (the entries of
+// shared rows are summed).
+struct SRowGroup {
+  int row0, n;
+  int pos_off;
+  int occ0, nocc;
 };
 
 __device__ __forceinline__ bool owner_axis(int a, int b, int s, int nc, int c) {
@@ -387,11 +398,49 @@ __global__ void __launch_bounds__(NT) k_group_h_jacobi(const SGroup *__restrict_
 
 // -------------------------------------------------------------- skeletonization
 
+// Rows r0, r0 + step, ... < r1 of A~_{R,g} into M (R x n column major).
+__device__ __forceinline__ void skel_gather_rows(const SSkel &S, const SGroup &g, const int2 *__restrict__ gcells,
+                                                 const SCell *__restrict__ cells,
+                                                 const SRowGroup *__restrict__ rgroups,
+                                                 const int2 *__restrict__ occs, const int *__restrict__ pos,
+                                                 const double *__restrict__ F, double *__restrict__ M, int r0,
+                                                 int r1, int step) {
+  constexpr int kOcc = 4;  // cells around an edge
+  for (int r = r0; r < r1; r += step) {
+    int lo = S.rg0, hi = S.rg0 + S.nrg;  // the row's group
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (rgroups[mid].row0 <= r) lo = mid;
+      else hi = mid;
+    }
+    const SRowGroup rg = rgroups[lo];
+    const int a = pos[rg.pos_off + r - rg.row0];
+    const double *src[kOcc];
+    long long ld[kOcc];
+#pragma unroll
+    for (int q = 0; q < kOcc; ++q)
+      if (q < rg.nocc) {
+        const int2 oc = occs[rg.occ0 + q];
+        const int2 cl = gcells[g.gc_off + oc.x];
+        const SCell c = cells[cl.x];
+        ld[q] = c.nI + c.nB;
+        src[q] = F + c.F_off + (c.nI + oc.y + a) + (long long)(c.nI + cl.y) * ld[q];
+      }
+    for (int j = 0; j < g.n; ++j) {
+      double acc = 0.0;
+#pragma unroll
+      for (int q = 0; q < kOcc; ++q)
+        if (q < rg.nocc) acc += src[q][j * ld[q]];
+      M[r + (long long)j * S.R] = acc;
+    }
+  }
+}
+
 __global__ void __launch_bounds__(NT) k_skel(const SSkel *__restrict__ sk, const SGroup *__restrict__ groups,
                                              const int2 *__restrict__ gcells,
                                              const SCell *__restrict__ cells,
-                                             const long long *__restrict__ rowptr,
-                                             const int2 *__restrict__ rowent,
+                                             const SRowGroup *__restrict__ rgroups,
+                                             const int2 *__restrict__ occs, const int *__restrict__ pos,
                                              const double *__restrict__ Linv, double *__restrict__ F,
                                              double *__restrict__ ws_all, double *__restrict__ vals,
                                              int *__restrict__ kout, int *__restrict__ perm_all,
@@ -413,18 +462,7 @@ __global__ void __launch_bounds__(NT) k_skel(const SSkel *__restrict__ sk, const
   double *vh = Kq + (long long)n * n;          // Householder vector (R)
 
   // (a) gather A~_{R,g}
-  for (long long t = threadIdx.x; t < (long long)R * n; t += NT) {
-    int r = (int)(t % R), j = (int)(t / R);
-    double acc = 0.0;
-    for (long long e = rowptr[S.row_off + r]; e < rowptr[S.row_off + r + 1]; ++e) {
-      int2 en = rowent[e];  // (slot in the group's cell list, B position of the row DOF)
-      int2 cl = gcells[g.gc_off + en.x];
-      const SCell c = cells[cl.x];
-      const int nn = c.nI + c.nB;
-      acc += F[c.F_off + (c.nI + en.y) + (long long)(c.nI + cl.y + j) * nn];
-    }
-    M[r + (long long)j * R] = acc;
-  }
+  skel_gather_rows(S, g, gcells, cells, rgroups, occs, pos, F, M, threadIdx.x, R, NT);
   for (int j = threadIdx.x; j < n; j += NT) perm[j] = j;
   if (threadIdx.x == 0) {
     s_k = 0;
@@ -585,6 +623,385 @@ __global__ void __launch_bounds__(NT) k_skel(const SSkel *__restrict__ sk, const
   }
   if (threadIdx.x == 0) kout[blockIdx.x] = k;
   for (int j = threadIdx.x; j < n; j += NT) perm_all[S.perm_off + j] = perm[j];
+}
+
+// ------------------------------------------------ skeletonization, large entities
+//
+// One CTA per entity leaves a large one waiting on a single SM: at 3D 63^3 the 12
+// level-2 faces (597 DOFs, some 4500 rows) took 829 ms.  Sub-steps whose largest
+// entity is above kSkelCtaDofs DOFs run these kernels instead, each spread over
+// the chip: the gather by row chunks, the pivoted QR by a thread-block cluster
+// per entity, everything after it (n^3 products an entity) as 64 x 64 tiles, the
+// Cholesky of I + T^T T through the batched kernels of the fronts.  Below it (all
+// of 2D, the 3D leaf faces) an entity's work is too small to split (1344 leaf faces
+// of 49 DOFs: 7.9 ms in one launch).
+// Measured, face sub-steps: 63^3 level 2 (597 DOFs) 829 -> 48 ms, level 1 (225) 162
+// -> 55 ms; 47^3 level 2 (405) 183 -> 19 ms, level 1 (121) 21 -> 12 ms.
+constexpr int kSkelCtaDofs = 64;
+constexpr int kQrThreads = 512;
+constexpr int kQrMaxCluster = 16;
+constexpr size_t kQrMaxSmem = 200 * 1024;
+
+// shared memory of the QR: the pivot column, the pivots, the columns' flags
+size_t qr_smem(int R, int n) { return (size_t)R * sizeof(double) + (size_t)n * (sizeof(int) + 1) + 16; }
+
+// workspace of one entity (doubles): M | T | Sm | Gp | U | TS | X | rdiag and the
+// single-CTA kernel's M | T | Sm | Lsi | TSi | Kq | vh
+long long skel_workspace(long long R, long long n) { return R * n + 6 * n * n + 8 * n + std::max<long long>(R, 1); }
+
+struct SkelWs {
+  double *M, *T, *Sm, *Gp, *U, *TS, *X, *rd;
+};
+__host__ __device__ inline SkelWs skel_ws(double *base, long long R, long long n) {
+  SkelWs w;
+  w.M = base;                 // R x n column major (columns stay in place)
+  w.T = w.M + R * n;          // k x nr row major
+  w.Sm = w.T + n * n;         // nr x nr column major, lower
+  w.Gp = w.Sm + n * n;        // inverse factor of Sm, packed lower (tri_off)
+  w.U = w.Gp + n * n + 4 * n; // k x nr row major: T Ls^{-T}
+  w.TS = w.U + n * n;         // k x nr row major: T S^{-1}
+  w.X = w.TS + n * n;         // k x k row major
+  w.rd = w.X + n * n;         // n: diagonal of R
+  return w;
+}
+
+// grid = (entities, row chunks of NT)
+__global__ void __launch_bounds__(NT) k_skel_gather(const SSkel *__restrict__ sk, const SGroup *__restrict__ groups,
+                                                    const int2 *__restrict__ gcells,
+                                                    const SCell *__restrict__ cells,
+                                                    const SRowGroup *__restrict__ rgroups,
+                                                    const int2 *__restrict__ occs, const int *__restrict__ pos,
+                                                    const double *__restrict__ F, double *__restrict__ ws) {
+  const SSkel S = sk[blockIdx.x];
+  const SGroup g = groups[S.g];
+  skel_gather_rows(S, g, gcells, cells, rgroups, occs, pos, F, skel_ws(ws + S.ws_off, S.R, g.n).M,
+                   blockIdx.y * NT + threadIdx.x, S.R, gridDim.y * NT);
+}
+
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_store(void *p, unsigned rank, double v) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(p), b;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(a), "r"(rank));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(b), "d"(v) : "memory");
+}
+
+// Column-pivoted Householder QR of M, stopped at the first |R_tt| <= eps |R_00|.
+// One cluster per entity; CTA c owns the columns j = c (mod size), a warp takes a
+// column at a time.  Columns are not swapped: a chosen column keeps its place and
+// is left alone, so a step needs one cluster barrier: every CTA publishes its best
+// remaining column norm (of the update before) to all, and after the barrier each
+// reads the pivot column from memory and applies the reflector to its own columns,
+// summing their new norms on the way (three products an element: the FP64 pipe's
+// bound).  Ties go to the smaller column.
+__global__ void __launch_bounds__(kQrThreads) k_skel_qr(const SSkel *__restrict__ sk,
+                                                        const SGroup *__restrict__ groups, double *__restrict__ ws,
+                                                        int *__restrict__ kout, int *__restrict__ perm_all,
+                                                        double eps) {
+  extern __shared__ __align__(16) double qsm[];
+  __shared__ double s_best[2][kQrMaxCluster][2];  // (norm^2, column) of each CTA, by step parity
+  __shared__ double s_wb[kQrThreads / 32][2];
+  const unsigned cr = cluster_rank(), cs = cluster_size();
+  const SSkel S = sk[blockIdx.x / cs];
+  const SGroup g = groups[S.g];
+  const int n = g.n, R = S.R;
+  const SkelWs w = skel_ws(ws + S.ws_off, R, n);
+  double *vh = qsm;                                    // pivot column, R
+  int *perm = reinterpret_cast<int *>(vh + R);         // chosen columns in order
+  unsigned char *used = reinterpret_cast<unsigned char *>(perm + n);
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  constexpr int NW = kQrThreads / 32;
+  for (int j = t; j < n; j += kQrThreads) used[j] = 0;
+  double best = -1.0;  // this warp's best remaining column
+  int best_j = n;
+  for (int j = cr + cs * warp; j < n; j += cs * NW) {
+    const double *col = w.M + (long long)j * R;
+    double a = 0.0;
+#pragma unroll 4
+    for (int r = lane; r < R; r += 32) a += col[r] * col[r];
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (a > best) {
+      best = a;
+      best_j = j;
+    }
+  }
+  const int tmax = R < n ? R : n;
+  double r00 = 0.0;
+  int k = 0;
+  for (int step = 0; step < tmax; ++step) {
+    if (lane == 0) {
+      s_wb[warp][0] = best;
+      s_wb[warp][1] = (double)best_j;
+    }
+    __syncthreads();
+    if (t < (int)cs) {  // the CTA's best to CTA t
+      double b = -1.0, bj = (double)n;
+      for (int v = 0; v < NW; ++v)
+        if (s_wb[v][0] > b || (s_wb[v][0] == b && s_wb[v][1] < bj)) {
+          b = s_wb[v][0];
+          bj = s_wb[v][1];
+        }
+      cluster_store(&s_best[step & 1][cr][0], t, b);
+      cluster_store(&s_best[step & 1][cr][1], t, bj);
+    }
+    cluster_sync();
+    double nb = -1.0, nj = (double)n;
+    for (unsigned c = 0; c < cs; ++c) {
+      const double b = s_best[step & 1][c][0], bj = s_best[step & 1][c][1];
+      if (b > nb || (b == nb && bj < nj)) {
+        nb = b;
+        nj = bj;
+      }
+    }
+    const int p = (int)nj;
+    const double r = nb > 0.0 ? sqrt(nb) : 0.0;  // (no column left: nb = -1)
+    if (step == 0) r00 = r;
+    if (!(r > 0.0) || r <= eps * r00) break;  // the same decision in every CTA
+    k = step + 1;
+    const double *pc = w.M + (long long)p * R;
+    const double x0 = __ldcg(pc + step);
+    const double alpha = x0 >= 0.0 ? -r : r;
+    const double v0 = x0 - alpha;
+    const double vn2 = r * r - x0 * x0 + v0 * v0;
+    const double sc = vn2 > 0.0 ? 2.0 / vn2 : 0.0;
+    for (int q = step + 1 + t; q < R; q += kQrThreads) vh[q] = __ldcg(pc + q);
+    if (t == 0) {
+      vh[step] = v0;
+      perm[step] = p;
+      used[p] = 1;
+      if (cr == 0) w.rd[step] = alpha;
+    }
+    __syncthreads();
+    best = -1.0;
+    best_j = n;
+    for (int j = cr + cs * warp; j < n; j += cs * NW) {
+      if (used[j]) continue;
+      double *col = w.M + (long long)j * R;
+      double a = 0.0, a2 = 0.0;
+      int q = step + lane;
+      for (; q + 96 < R; q += 128) {
+        double m[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) m[u] = col[q + 32 * u];
+        a += vh[q] * m[0];
+        a2 += vh[q + 32] * m[1];
+        a += vh[q + 64] * m[2];
+        a2 += vh[q + 96] * m[3];
+      }
+      for (; q < R; q += 32) a += vh[q] * col[q];
+      a += a2;
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      const double f = a * sc;
+      double s0 = 0.0, s1 = 0.0;
+      // row `step` becomes the column's entry of R and leaves the norm
+      if (lane == 0) col[step] -= f * v0;
+      q = step + 1 + lane;
+      for (; q + 96 < R; q += 128) {
+        double m[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) m[u] = col[q + 32 * u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          m[u] -= f * vh[q + 32 * u];
+          col[q + 32 * u] = m[u];
+        }
+        s0 += m[0] * m[0];
+        s1 += m[1] * m[1];
+        s0 += m[2] * m[2];
+        s1 += m[3] * m[3];
+      }
+      for (; q < R; q += 32) {
+        const double m = col[q] - f * vh[q];
+        col[q] = m;
+        s0 += m * m;
+      }
+      s0 += s1;
+      for (int o = 16; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+      if (s0 > best) {
+        best = s0;
+        best_j = j;
+      }
+    }
+  }
+  cluster_sync();  // no CTA leaves while another may still store into it
+  if (cr == 0) {
+    int *out = perm_all + S.perm_off;
+    for (int j = t; j < k; j += kQrThreads) out[j] = perm[j];
+    if (t == 0) {
+      kout[blockIdx.x / cs] = k;
+      int o = k;
+      for (int j = 0; j < n; ++j)
+        if (!used[j]) out[o++] = j;
+    }
+  }
+}
+
+// T = R11^{-1} R12 by blocks of 32 rows from the last: grid = (entities, blocks of
+// 32 columns of T)
+__global__ void __launch_bounds__(NT) k_skel_T(const SSkel *__restrict__ sk, const SGroup *__restrict__ groups,
+                                               double *__restrict__ ws, const int *__restrict__ kin,
+                                               const int *__restrict__ perm_all) {
+  __shared__ double Rs[32][33], Xs[32][33];
+  const SSkel S = sk[blockIdx.x];
+  const int n = groups[S.g].n, R = S.R, k = kin[blockIdx.x], nr = n - k;
+  const int c0 = blockIdx.y * 32;
+  if (c0 >= nr) return;
+  const SkelWs w = skel_ws(ws + S.ws_off, R, n);
+  const int *perm = perm_all + S.perm_off;
+  const int tr = threadIdx.x % 32, tc = threadIdx.x / 32;  // row of the block; columns tc + 8 v
+  for (int i0 = (k - 1) / 32 * 32; i0 >= 0 && k > 0; i0 -= 32) {
+    double acc[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      const int c = c0 + tc + 8 * v;
+      acc[v] = i0 + tr < k && c < nr ? w.M[i0 + tr + (long long)perm[k + c] * R] : 0.0;
+    }
+    for (int j0 = i0 + 32; j0 < k; j0 += 32) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < 1024; e += NT) {
+        const int a = e % 32, b = e / 32;
+        Rs[b][a] = i0 + a < k && j0 + b < k ? w.M[i0 + a + (long long)perm[j0 + b] * R] : 0.0;
+        Xs[b][a] = j0 + b < k && c0 + a < nr ? w.T[(long long)(j0 + b) * nr + c0 + a] : 0.0;
+      }
+      __syncthreads();
+#pragma unroll 8
+      for (int b = 0; b < 32; ++b) {
+        const double l = Rs[b][tr];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[v] -= l * Xs[b][tc + 8 * v];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < 4; ++v) Xs[tr][tc + 8 * v] = acc[v];
+    for (int e = threadIdx.x; e < 1024; e += NT) {
+      const int a = e % 32, b = e / 32;
+      Rs[b][a] = i0 + a < k && i0 + b < k && a < b ? w.M[i0 + a + (long long)perm[i0 + b] * R] : 0.0;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {  // a column per thread
+      const int c = threadIdx.x;
+      for (int a = min(31, k - 1 - i0); a >= 0; --a) {
+        double v = Xs[a][c];
+        for (int b = a + 1; b < 32 && i0 + b < k; ++b) v -= Rs[b][a] * Xs[b][c];
+        v /= w.rd[i0 + a];
+        Xs[a][c] = v;
+        if (c0 + c < nr) w.T[(long long)(i0 + a) * nr + c0 + c] = v;
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Products after the QR, 64 x 64 tiles with 4 x 4 results a thread; grid =
+// (entities, tiles).
+//   kMulS: Sm = I + T^T T (lower)            kMulU: U = T Ls^{-T}
+//   kMulTS: TS = U Ls^{-1} (= T S^{-1})      kMulX: X = I - U U^T, also into the owner
+//   kMulH: H = K^T Linv with rows and columns in DOF order, K^T in (redundant,
+//          skeleton) order [[Ls^{-1}, -U^T], [TS, X]]
+enum SkelMul { kMulS = 0, kMulU, kMulTS, kMulX, kMulH };
+
+template <int OP>
+__global__ void __launch_bounds__(NT) k_skel_mul(const SSkel *__restrict__ sk, const SGroup *__restrict__ groups,
+                                                 const int2 *__restrict__ gcells, const SCell *__restrict__ cells,
+                                                 double *__restrict__ ws, const int *__restrict__ kin,
+                                                 const int *__restrict__ perm_all, const double *__restrict__ Linv,
+                                                 double *__restrict__ F, double *__restrict__ vals) {
+  constexpr int TB = 64, KC = 32;
+  __shared__ double As[KC][TB + 1], Bs[KC][TB + 1];
+  const SSkel S = sk[blockIdx.x];
+  const SGroup g = groups[S.g];
+  const int n = g.n, k = kin[blockIdx.x], nr = n - k;
+  const SkelWs w = skel_ws(ws + S.ws_off, S.R, n);
+  const int *perm = perm_all + S.perm_off;
+  const int m = OP == kMulS ? nr : OP == kMulH ? n : k;                      // rows
+  const int nc = OP == kMulX ? k : OP == kMulH ? n : nr;                     // columns
+  const int K = OP == kMulS ? k : OP == kMulH ? n : nr;
+  const int tm = (m + TB - 1) / TB, tn = (nc + TB - 1) / TB;
+  const double *Li = Linv + g.Linv_off;
+  auto q_of = [&](int b) { return b < nr ? perm[k + b] : perm[b - nr]; };
+  auto lsi = [&](int i, int j) { return j <= i ? w.Gp[tri_off(i) + j] : 0.0; };
+  auto Aval = [&](int i, int q) -> double {  // row i, K index q
+    if (OP == kMulS) return w.T[(long long)q * nr + i];
+    if (OP == kMulU) return w.T[(long long)i * nr + q];
+    if (OP == kMulTS || OP == kMulX) return w.U[(long long)i * nr + q];
+    if (i < nr) return q < nr ? lsi(i, q) : -w.U[(long long)(q - nr) * nr + i];
+    return q < nr ? w.TS[(long long)(i - nr) * nr + q] : w.X[(long long)(i - nr) * k + q - nr];
+  };
+  auto Bval = [&](int q, int j) -> double {
+    if (OP == kMulS) return w.T[(long long)q * nr + j];
+    if (OP == kMulU) return lsi(j, q);
+    if (OP == kMulTS) return lsi(q, j);
+    if (OP == kMulX) return w.U[(long long)j * nr + q];
+    return Li[(long long)q_of(q) * n + j];
+  };
+  // the K index runs along consecutive addresses for these operands
+  constexpr bool kAk = OP != kMulS, kBk = OP == kMulU || OP == kMulX;
+  for (int y = blockIdx.y; y < tm * tn; y += gridDim.y) {
+    const int i0 = (y % tm) * TB, j0 = (y / tm) * TB;
+    if (OP == kMulS && j0 > i0) continue;  // lower triangle
+    double acc[4][4] = {};
+    // consecutive threads along the results' contiguous index
+    const int ta = OP == kMulS ? threadIdx.x % 16 : threadIdx.x / 16;
+    const int tb = OP == kMulS ? threadIdx.x / 16 : threadIdx.x % 16;
+    for (int q0 = 0; q0 < K; q0 += KC) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < KC * TB; e += NT) {
+        const int ka = kAk ? e % KC : e / TB, ia = kAk ? e / KC : e % TB;
+        As[ka][ia] = i0 + ia < m && q0 + ka < K ? Aval(i0 + ia, q0 + ka) : 0.0;
+        const int kb = kBk ? e % KC : e / TB, jb = kBk ? e / KC : e % TB;
+        Bs[kb][jb] = j0 + jb < nc && q0 + kb < K ? Bval(q0 + kb, j0 + jb) : 0.0;
+      }
+      __syncthreads();
+#pragma unroll 8
+      for (int q = 0; q < KC; ++q) {
+        double a[4], b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          a[u] = As[q][ta + 16 * u];
+          b[u] = Bs[q][tb + 16 * u];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) acc[u][v] += a[u] * b[v];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int i = i0 + ta + 16 * u, j = j0 + tb + 16 * v;
+        if (i >= m || j >= nc) continue;
+        const double x = acc[u][v];
+        if (OP == kMulS) {
+          w.Sm[i + (long long)j * nr] = (i == j ? 1.0 : 0.0) + x;
+        } else if (OP == kMulU) {
+          w.U[(long long)i * nr + j] = x;
+        } else if (OP == kMulTS) {
+          w.TS[(long long)i * nr + j] = x;
+        } else if (OP == kMulX) {
+          const double xv = (i == j ? 1.0 : 0.0) - x;
+          w.X[(long long)i * k + j] = xv;
+          const int2 cl = gcells[g.gc_off];
+          const SCell c = cells[cl.x];
+          F[c.F_off + (c.nI + cl.y + perm[i]) + (long long)(c.nI + cl.y + perm[j]) * (c.nI + c.nB)] = xv;
+        } else {
+          vals[g.H_off + (long long)q_of(i) * pad4(n) + j] = x;
+        }
+      }
+  }
 }
 
 // ------------------------------------------------------------------ host planning
@@ -762,6 +1179,97 @@ long long setup_budget(const char *env, double frac) {
 int set_smem(const void *fn, size_t bytes) {
   if (bytes > 48 * 1024)
     HIF_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  return HIF_OK;
+}
+
+// The skeletonization of one launch's entities through the kernels for large ones.
+int skeletonize_large(const std::vector<SSkel> &sk, const std::vector<SGroup> &groups, const SSkel *dsk,
+                      const SGroup *dgroups, const int2 *dgcells, const SCell *dcells, const SRowGroup *drg,
+                      const int2 *docc, const int *dpos, const double *Linv, double *F, double *ws, double *vals,
+                      int *dk, int *dperm, double eps, int *derr, cudaStream_t s) {
+  const int nt = (int)sk.size();
+  int max_n = 1, max_R = 1;
+  for (const SSkel &x : sk) {
+    max_n = std::max(max_n, groups[x.g].n);
+    max_R = std::max(max_R, x.R);
+  }
+  k_skel_gather<<<dim3(nt, std::min((max_R + NT - 1) / NT, 65535)), NT, 0, s>>>(dsk, dgroups, dgcells, dcells, drg,
+                                                                                docc, dpos, F, ws);
+  note_launch();
+  HIF_CUDA_TRY(cudaGetLastError());
+  // pivoted QR: the largest cluster that keeps about two CTAs an SM, at most 16
+  // (8 is the portable limit; 16 only when the device takes it)
+  const size_t qsm = qr_smem(max_R, max_n);
+  HIF_TRY(set_smem((const void *)k_skel_qr, qsm));
+  HIF_CUDA_TRY(cudaFuncSetAttribute((const void *)k_skel_qr, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  int cs = 1;
+  while (cs < kQrMaxCluster && nt * cs * 2 <= 2 * 152) cs *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kQrThreads);
+  cfg.dynamicSmemBytes = qsm;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  for (;; cs /= 2) {
+    cfg.gridDim = dim3(nt * cs);
+    attr[0].val.clusterDim.x = cs;
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, k_skel_qr, &cfg) != cudaSuccess) cudaGetLastError();
+    if (fit >= 1 || cs == 1) break;
+  }
+  HIF_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_skel_qr, dsk, dgroups, ws, dk, dperm, eps));
+  note_launch();
+  // ranks: the sizes of what follows
+  std::vector<int> kh(nt);
+  HIF_CUDA_TRY(cudaMemcpyAsync(kh.data(), dk, nt * sizeof(int), cudaMemcpyDeviceToHost, s));
+  HIF_CUDA_TRY(cudaStreamSynchronize(s));
+  int max_nr = 0, max_k = 0;
+  std::vector<JBlock> jb(nt);
+  for (int t = 0; t < nt; ++t) {
+    const int n = groups[sk[t].g].n;
+    max_nr = std::max(max_nr, n - kh[t]);
+    max_k = std::max(max_k, kh[t]);
+    const SkelWs w = skel_ws(ws + sk[t].ws_off, sk[t].R, n);
+    jb[t].nI = n - kh[t];
+    jb[t].nB = 0;
+    jb[t].F_off = w.Sm - ws;
+    jb[t].G_off = w.Gp - ws;
+    jb[t].V_off = 0;
+  }
+  auto tiles = [](int a, int b) { return std::max(1, std::min(((a + 63) / 64) * ((b + 63) / 64), 65535)); };
+  Scratch tmp;
+  JBlock *djb = nullptr;
+  if (max_nr > 0) {
+    if (max_k > 0) {
+      k_skel_T<<<dim3(nt, (max_nr + 31) / 32), NT, 0, s>>>(dsk, dgroups, ws, dk, dperm);
+      note_launch();
+    }
+    k_skel_mul<kMulS><<<dim3(nt, tiles(max_nr, max_nr)), NT, 0, s>>>(dsk, dgroups, dgcells, dcells, ws, dk, dperm,
+                                                                     Linv, F, vals);
+    note_launch();
+    HIF_TRY(tmp.upload(&djb, jb, s));
+    HIF_TRY(dense::eliminate_cells<JBlock>(jb, djb, ws, ws, derr, s));
+    if (max_k > 0) {
+      k_skel_mul<kMulU><<<dim3(nt, tiles(max_k, max_nr)), NT, 0, s>>>(dsk, dgroups, dgcells, dcells, ws, dk, dperm,
+                                                                      Linv, F, vals);
+      k_skel_mul<kMulTS><<<dim3(nt, tiles(max_k, max_nr)), NT, 0, s>>>(dsk, dgroups, dgcells, dcells, ws, dk, dperm,
+                                                                       Linv, F, vals);
+      note_launch(2);
+    }
+  }
+  if (max_k > 0) {
+    k_skel_mul<kMulX><<<dim3(nt, tiles(max_k, max_k)), NT, 0, s>>>(dsk, dgroups, dgcells, dcells, ws, dk, dperm,
+                                                                   Linv, F, vals);
+    note_launch();
+  }
+  k_skel_mul<kMulH><<<dim3(nt, tiles(max_n, max_n)), NT, 0, s>>>(dsk, dgroups, dgcells, dcells, ws, dk, dperm, Linv,
+                                                                 F, vals);
+  note_launch();
+  HIF_CUDA_TRY(cudaGetLastError());
+  HIF_CUDA_TRY(cudaStreamSynchronize(s));  // the descriptors of tmp are read by the kernels
   return HIF_OK;
 }
 
@@ -1207,47 +1715,59 @@ int gpu_setup(Handle *h, const double *a_nodes, cudaStream_t s) {
                                         (long long)sizeof(double), 1LL);
     for (int cd : codims) {
       std::vector<SSkel> sk;
-      std::vector<long long> rowptr;
-      std::vector<int2> rowent;
+      std::vector<SRowGroup> rgroups;
+      std::vector<int2> occs;
       std::vector<int> ws_at = {0};  // groups in launches whose workspaces fit the scratch
       long long wsoff = 0, wsmax = 0, poff = 0;
       int max_n = 1;
-      std::vector<int> rowid(N, -1);
+      // surviving DOFs of every entity (those of an earlier sub-step's redundant
+      // set are gone)
+      std::vector<int> pos, pos_off(ng + 1, 0);
+      for (int g = 0; g < ng; ++g) {
+        for (int a = 0; a < (int)P.g_dofs[g].size(); ++a)
+          if (alive[P.g_dofs[g][a]]) pos.push_back(a);
+        pos_off[g + 1] = (int)pos.size();
+      }
+      std::vector<int> rg_of(ng, -1);
+      std::vector<int2> seen;  // (entity, occurrence) of the current group, in order of first encounter
       for (int g = 0; g < ng; ++g) {
         if (P.g_codim[g] != cd) continue;
         SSkel x{};
         x.g = g;
-        x.row_off = (long long)rowptr.size();
-        // rows: boundary DOFs of the adjacent cells except g's own and those
-        // eliminated earlier in this level (redundant DOFs of a previous sub-step)
-        std::vector<int> rows;
-        std::vector<std::vector<int2>> rent;
+        x.rg0 = (int)rgroups.size();
+        std::vector<std::vector<int2>> oc;
         for (size_t q = 0; q < P.g_cells[g].size(); ++q) {
-          int c = P.g_cells[g][q];
           int p = 0;
-          for (int g2 : P.cG[c]) {
-            for (int a = 0; a < (int)P.g_dofs[g2].size(); ++a, ++p) {
-              if (g2 == g) continue;
-              int d = P.g_dofs[g2][a];
-              if (!alive[d]) continue;
-              if (rowid[d] < 0) {
-                rowid[d] = (int)rows.size();
-                rows.push_back(d);
-                rent.push_back({});
+          for (int g2 : P.cG[P.g_cells[g][q]]) {
+            const int n2 = (int)P.g_dofs[g2].size();
+            if (g2 != g && pos_off[g2 + 1] > pos_off[g2]) {
+              if (rg_of[g2] < 0) {
+                rg_of[g2] = (int)oc.size();
+                oc.push_back({});
+                SRowGroup rg{};
+                rg.row0 = x.R;
+                rg.n = pos_off[g2 + 1] - pos_off[g2];
+                rg.pos_off = pos_off[g2];
+                x.R += rg.n;
+                rgroups.push_back(rg);
+                seen.push_back(make_int2(g2, 0));
               }
-              rent[rowid[d]].push_back(make_int2((int)q, p));
+              oc[rg_of[g2]].push_back(make_int2((int)q, p));
             }
+            p += n2;
           }
         }
-        for (size_t r = 0; r < rows.size(); ++r) {
-          rowptr.push_back((long long)rowent.size());
-          for (auto e : rent[r]) rowent.push_back(e);
-          rowid[rows[r]] = -1;
+        for (size_t e = 0; e < oc.size(); ++e) {
+          SRowGroup &rg = rgroups[x.rg0 + e];
+          rg.occ0 = (int)occs.size();
+          rg.nocc = (int)oc[e].size();
+          occs.insert(occs.end(), oc[e].begin(), oc[e].end());
         }
-        rowptr.push_back((long long)rowent.size());
-        x.R = (int)rows.size();
+        for (const int2 &v : seen) rg_of[v.x] = -1;
+        seen.clear();
+        x.nrg = (int)oc.size();
         const long long nG = groups[g].n;
-        const long long need = (long long)x.R * nG + 5 * nG * nG + std::max<long long>(x.R, 1);
+        const long long need = skel_workspace(x.R, nG);
         if (wsoff > 0 && wsoff + need > wcap) {
           ws_at.push_back((int)sk.size());
           wsoff = 0;
@@ -1263,22 +1783,33 @@ int gpu_setup(Handle *h, const double *a_nodes, cudaStream_t s) {
       if (sk.empty()) continue;
       ws_at.push_back((int)sk.size());
       SSkel *dsk = nullptr;
-      long long *drowptr = nullptr;
-      int2 *drowent = nullptr;
+      SRowGroup *drg = nullptr;
+      int2 *docc = nullptr;
+      int *dpos = nullptr;
       double *ws = nullptr;
       int *dk = nullptr, *dperm = nullptr;
       Scratch sub;
       HIF_TRY(sub.upload(&dsk, sk, s));
-      HIF_TRY(sub.upload(&drowptr, rowptr, s));
-      HIF_TRY(sub.upload(&drowent, rowent, s));
+      HIF_TRY(sub.upload(&drg, rgroups, s));
+      HIF_TRY(sub.upload(&docc, occs, s));
+      HIF_TRY(sub.upload(&dpos, pos, s));
       HIF_TRY(sub.alloc(&ws, wsmax));
       HIF_TRY(sub.alloc(&dk, sk.size()));
       HIF_TRY(sub.alloc(&dperm, poff));
+      int max_R = 1;
+      for (const SSkel &x : sk) max_R = std::max(max_R, x.R);
+      const bool large = max_n > kSkelCtaDofs && qr_smem(max_R, max_n) <= kQrMaxSmem;
       size_t sm = (size_t)max_n * (sizeof(double) + sizeof(int)) + 16;
-      HIF_TRY(set_smem((const void *)k_skel, sm));
+      if (!large) HIF_TRY(set_smem((const void *)k_skel, sm));
       for (size_t k = 0; k + 1 < ws_at.size(); ++k) {
         const int t0 = ws_at[k], nt = ws_at[k + 1] - t0;
-        k_skel<<<nt, NT, sm, s>>>(dsk + t0, dgroups, dgcells, dbcells, drowptr, drowent, Linv, Fb, ws, vals,
+        if (large) {
+          HIF_TRY(skeletonize_large(std::vector<SSkel>(sk.begin() + t0, sk.begin() + t0 + nt), groups, dsk + t0,
+                                    dgroups, dgcells, dbcells, drg, docc, dpos, Linv, Fb, ws, vals, dk + t0, dperm,
+                                    eps, derr, s));
+          continue;
+        }
+        k_skel<<<nt, NT, sm, s>>>(dsk + t0, dgroups, dgcells, dbcells, drg, docc, dpos, Linv, Fb, ws, vals,
                                   dk + t0, dperm, eps, derr);
         note_launch();
         HIF_CUDA_TRY(cudaGetLastError());
