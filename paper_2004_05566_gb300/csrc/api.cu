@@ -133,6 +133,15 @@ int make_root_dense(Handle *h, cudaStream_t s);
 int build_items(Handle *h, LevelDev &D, const LevelHost &H, int target, cudaStream_t s) {
   std::vector<CellItem> fw, bw;
   const int ncell = (int)H.cells.size();
+  // cut cells so that an item holds at most kItemBytes of FP32 factor, where the
+  // default count would leave more (3D levels of a few hundred large cells: an SM
+  // with three such items waits on its loads; 63^3 cells forward, with twice the
+  // loads in flight: 108, 69 and 56 -> 69, 46 and 37 us at levels 0 to 2)
+  if (target == kDefaultItemTarget && ncell < target) {
+    double vals = 0;
+    for (const CellDesc &cd : H.cells) vals += (double)cd.nI * (cd.nI + 1) / 2 + (double)cd.nB * cd.nI;
+    target = (int)std::max<double>(target, std::min(4.0 * vals / kItemBytes, 152.0 * 32));
+  }
   for (int c = 0; c < ncell; ++c) {
     const CellDesc &cd = H.cells[c];
     const int rows = cd.nB + cd.nI;
@@ -303,6 +312,12 @@ int finish_device_factor(Handle *h, cudaStream_t s) {
   }
   if (h->root_n > 0) HIF_TRY(dev_alloc(h, &h->upper_rt, h->root_n * sizeof(double)));
   h->root_split = h->root_n > root_split;
+  if (h->root_split) {
+    const size_t nb = (h->root_n + 127) / 128, nch = (h->root_n + kRootRowChunk - 1) / kRootRowChunk;
+    HIF_TRY(dev_alloc(h, &h->root_part, nb * nch * 128 * sizeof(double)));
+    HIF_TRY(dev_alloc(h, (void **)&h->root_tk, nb * sizeof(unsigned)));
+    HIF_CUDA_TRY(cudaMemsetAsync(h->root_tk, 0, nb * sizeof(unsigned), s));
+  }
   HIF_TRY(make_cell_inverses(h, s));
   if (!lean) HIF_TRY(dev_alloc(h, (void **)&h->f64.contrib, h->max_contrib * sizeof(double)));
   if (h->opt.precision == HIF_FP32 || h->opt.precision == HIF_FP32_BF16TOP) {
@@ -477,6 +492,8 @@ void release_factor(Handle *h) {
   h->upper_phases = nullptr;
   h->upper_levels = nullptr;
   h->upper_rt = nullptr;
+  h->root_part = nullptr;
+  h->root_tk = nullptr;
   h->root_split = false;
   h->root_S = nullptr;
   h->root_S_ld = 0;

@@ -113,6 +113,51 @@ __device__ __forceinline__ void ld4(const __nv_bfloat16 *p, float (&o)[4]) {
   o[2] = __uint_as_float(v.y << 16);
   o[3] = __uint_as_float(v.y & 0xffff0000u);
 }
+// Factor values on their one pass through the chip: zero where !ok, not kept in
+// L1, and volatile, so that the compiler leaves a batch of them in flight (it
+// otherwise orders each load next to its use to save registers: 32 registers and
+// two or three loads in flight for a batch of eight).
+__device__ __forceinline__ void ld4_stream(const float *p, bool ok, float (&o)[4]) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %5, 0;\n\tmov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\t"
+      "mov.f32 %2, 0f00000000;\n\tmov.f32 %3, 0f00000000;\n\t"
+      "@p ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+      : "=&f"(o[0]), "=&f"(o[1]), "=&f"(o[2]), "=&f"(o[3])
+      : "l"(p), "r"((int)ok));
+}
+__device__ __forceinline__ void ld2_stream(const double *p, bool ok, double &a, double &b) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %3, 0;\n\tmov.f64 %0, 0d0000000000000000;\n\t"
+      "mov.f64 %1, 0d0000000000000000;\n\t"
+      "@p ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];\n\t}"
+      : "=&d"(a), "=&d"(b)
+      : "l"(p), "r"((int)ok));
+}
+__device__ __forceinline__ double ld1_stream(const double *p, bool ok) {
+  double a;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\tmov.f64 %0, 0d0000000000000000;\n\t"
+      "@p ld.global.nc.L1::no_allocate.f64 %0, [%1];\n\t}"
+      : "=&d"(a)
+      : "l"(p), "r"((int)ok));
+  return a;
+}
+__device__ __forceinline__ void ld4_stream(const double *p, bool ok, double (&o)[4]) {
+  ld2_stream(p, ok, o[0], o[1]);
+  ld2_stream(p + 2, ok, o[2], o[3]);
+}
+__device__ __forceinline__ void ld4_stream(const __nv_bfloat16 *p, bool ok, float (&o)[4]) {
+  unsigned a, b;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %3, 0;\n\tmov.u32 %0, 0;\n\tmov.u32 %1, 0;\n\t"
+      "@p ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];\n\t}"
+      : "=&r"(a), "=&r"(b)
+      : "l"(p), "r"((int)ok));
+  o[0] = __uint_as_float(a << 16);
+  o[1] = __uint_as_float(a & 0xffff0000u);
+  o[2] = __uint_as_float(b << 16);
+  o[3] = __uint_as_float(b & 0xffff0000u);
+}
 __device__ __forceinline__ void st4(float *p, const float (&v)[4]) {
   *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
@@ -147,7 +192,7 @@ __device__ __forceinline__ void warp_rows_dot4_f64(const double *const (&rp)[kRo
   for (; p + 24 < np2; p += 32) {
     double2 v[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = *reinterpret_cast<const double2 *>(row + 2 * (p + 8 * k));
+    for (int k = 0; k < 4; ++k) ld2_stream(row + 2 * (p + 8 * k), true, v[k].x, v[k].y);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const double2 xv = *reinterpret_cast<const double2 *>(xs + 2 * (p + 8 * k));
@@ -187,15 +232,32 @@ __device__ __forceinline__ void warp_rows_dot4(const TV *const (&rp)[kRows], con
     acc[u] = T(0);
     maxq = nq[u] > maxq ? nq[u] : maxq;
   }
-  for (int q = lane; q < maxq; q += 32) {
+  // kRows quads a lane in flight, 2 kRows where the rows are longer than 32
+  // quads: the rows of a big box come from HBM and its CTAs wait on them
+  int q = lane;
+  for (; q - lane + 32 < maxq; q += 64) {
+    T v[2][kRows][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int u = 0; u < kRows; ++u) {
+        ld4_stream(rp[u] + 4 * (q + 32 * h), q + 32 * h < nq[u], v[h][u]);
+      }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      T xv[4] = {T(0), T(0), T(0), T(0)};
+      if (q + 32 * h < maxq) ld4(xs + 4 * (q + 32 * h), xv);
+#pragma unroll
+      for (int u = 0; u < kRows; ++u)
+        acc[u] += v[h][u][0] * xv[0] + v[h][u][1] * xv[1] + v[h][u][2] * xv[2] + v[h][u][3] * xv[3];
+    }
+  }
+  if (q < maxq) {
     T v[kRows][4];
 #pragma unroll
-    for (int u = 0; u < kRows; ++u) {
-      if (q < nq[u]) ld4(rp[u] + 4 * q, v[u]);
-      else v[u][0] = v[u][1] = v[u][2] = v[u][3] = T(0);
-    }
+    for (int u = 0; u < kRows; ++u) ld4_stream(rp[u] + 4 * q, q < nq[u], v[u]);
     T xv[4];
-    xv[0] = xs[4 * q]; xv[1] = xs[4 * q + 1]; xv[2] = xs[4 * q + 2]; xv[3] = xs[4 * q + 3];
+    ld4(xs + 4 * q, xv);
 #pragma unroll
     for (int u = 0; u < kRows; ++u)
       acc[u] += v[u][0] * xv[0] + v[u][1] * xv[1] + v[u][2] * xv[2] + v[u][3] * xv[3];
@@ -267,7 +329,7 @@ __device__ __forceinline__ void cell_fwd_unit(const CellItem &it, const CellDesc
 }
 
 template <typename T, typename TV = T>
-__global__ void __launch_bounds__(kCellFwdThreads) k_cell_fwd(const CellItem *__restrict__ items,
+__global__ void __launch_bounds__(kCellFwdThreads, sizeof(T) == 4 ? 3 : 4) k_cell_fwd(const CellItem *__restrict__ items,
                                                               const CellDesc *__restrict__ cells,
                                                               const int *__restrict__ idx,
                                                               const TV *__restrict__ vals,
@@ -706,7 +768,7 @@ __device__ __forceinline__ void cell_bwd_cols_f64(const CellItem &it, const Cell
       for (; i + 3 * NW < c.nI; i += 4 * NW) {
         double v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = ok ? G[tri_off(i + k * NW) + col] : 0.0;
+        for (int k = 0; k < 4; ++k) v[k] = ld1_stream(G + tri_off(i + k * NW) + col, ok);
         acc += v[0] * xs[i];
         acc2 += v[1] * xs[i + NW];
         acc += v[2] * xs[i + 2 * NW];
@@ -717,7 +779,7 @@ __device__ __forceinline__ void cell_bwd_cols_f64(const CellItem &it, const Cell
       for (; q + 3 * NW < c.nB; q += 4 * NW) {
         double v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = ok ? V[(long long)(q + k * NW) * vstride + col] : 0.0;
+        for (int k = 0; k < 4; ++k) v[k] = ld1_stream(V + (long long)(q + k * NW) * vstride + col, ok);
         acc -= v[0] * xb[q];
         acc2 -= v[1] * xb[q + NW];
         acc -= v[2] * xb[q + 2 * NW];
@@ -737,12 +799,80 @@ __device__ __forceinline__ void cell_bwd_cols_f64(const CellItem &it, const Cell
   }
 }
 
+// FP32 columns [a, b) of the backward cell step.  A warp reads strips of whole
+// quads: L lanes (the smallest power of two that covers the block's quads, at most
+// 32) side by side along a row, 32 / L rows at a time, eight rows a lane in flight;
+// the rows are dealt over all such lane groups of the CTA.  Blocks of at most 32
+// quads, of equal width.  The sums of the lane groups meet by shuffles, then the
+// warps' in shared memory.  (A layout of quad pairs that balances the triangle had
+// lanes of a warp on different rows of G and half the loads in flight: 63^3 cells
+// backward 97, 57 and 48 us at levels 0 to 2; 70, 49 and 38 now with finer items.)
+template <typename T, int NT, typename TV>
+__device__ __forceinline__ void cell_bwd_cols_f32(const CellItem &it, const CellDesc &c,
+                                                  const int *__restrict__ I, const TV *__restrict__ G,
+                                                  const TV *__restrict__ V, long long vstride,
+                                                  const T *xs, const T *xb, T *part, T *__restrict__ x) {
+  constexpr int NW = NT / 32, kU = 8;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int qa = it.a / 4, qb = (it.b + 3) / 4;  // column quads [qa, qb)
+  const int nblk = (qb - qa + 31) / 32, per = nblk ? (qb - qa + nblk - 1) / nblk : 0;
+  int L = 1;
+  while (L < per) L <<= 1;
+  const int ql = lane & (L - 1), rg = (warp * 32 + lane) / L, RG = NT / L;
+  for (int q0 = qa; q0 < qb; q0 += per) {
+    const int q = q0 + ql;
+    const bool ok = ql < per && q < qb;
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    for (int i0 = 4 * q0 + rg; i0 < c.nI; i0 += kU * RG) {
+      T v[kU][4];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int i = i0 + u * RG;
+        ld4_stream(G + tri_off(i) + 4 * q, ok && i < c.nI && i >= 4 * q, v[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int i = i0 + u * RG;
+        const T xv = i < c.nI ? xs[i] : T(0);
+        acc[0] += v[u][0] * xv; acc[1] += v[u][1] * xv; acc[2] += v[u][2] * xv; acc[3] += v[u][3] * xv;
+      }
+    }
+    for (int r0 = rg; r0 < c.nB; r0 += kU * RG) {
+      T v[kU][4];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int r = r0 + u * RG;
+        ld4_stream(V + (long long)r * vstride + 4 * q, ok && r < c.nB, v[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int r = r0 + u * RG;
+        const T xv = r < c.nB ? xb[r] : T(0);
+        acc[0] -= v[u][0] * xv; acc[1] -= v[u][1] * xv; acc[2] -= v[u][2] * xv; acc[3] -= v[u][3] * xv;
+      }
+    }
+    for (int o = L; o < 32; o <<= 1) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+    }
+    if (lane < L) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) part[warp * 128 + 4 * lane + e] = acc[e];
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < 4 * per; t += NT) {
+      const int col = 4 * q0 + t;
+      T sum = part[t];
+#pragma unroll
+      for (int w = 1; w < NW; ++w) sum += part[w * 128 + t];
+      if (col < it.b) x[I[col]] = sum;
+    }
+    __syncthreads();
+  }
+}
+
 // Backward cell step (E_I): x_I <- G^T xI_I - V^T x_B, for columns [a, b)
-// (a a multiple of 4) of one cell.  A thread owns the column quad pair
-// (qa, qb) = (first + p, last - p), which balances the triangular row counts,
-// and reads both quads of a row with 16-byte loads.  The pairs take the
-// smallest power-of-two number of threads that covers them, the rest of the
-// CTA splits the rows into groups, and the row groups are added by a tree.
+// (a a multiple of 4) of one cell.  smem: 8 NT partial sums, x_I and x_B.
 template <typename T, int NT, typename TV = T, bool PDL = false>
 __device__ __forceinline__ void cell_bwd_unit(const CellItem &it, const CellDesc *__restrict__ cells,
                                               const int *__restrict__ idx, const TV *__restrict__ vals,
@@ -771,74 +901,12 @@ __device__ __forceinline__ void cell_bwd_unit(const CellItem &it, const CellDesc
   const TV *G = vals + c.G_off;
   const TV *V = vals + c.V_off;
   const long long vstride = pad4(c.nI);
-  if constexpr (sizeof(T) == 8) {
-    cell_bwd_cols_f64<NT>(it, c, I, G, V, vstride, xs, xb, part, x);
-    return;
-  }
-  const int q0 = it.a / 4, q1 = (it.b + 3) / 4;  // column quads [q0, q1)
-  const int npairs = (q1 - q0 + 1) / 2;
-  int PW, RG;
-  pow2_layout(npairs, NT, PW, RG);
-  const int pl = threadIdx.x % PW, rg = threadIdx.x / PW;
-  for (int p0 = 0; p0 < npairs; p0 += PW) {
-    const int p = p0 + pl;
-    const int qa = q0 + p, qb = q1 - 1 - p;
-    const bool okA = p < npairs;
-    const bool okB = okA && qb > qa;
-    T aA[4] = {T(0), T(0), T(0), T(0)}, aB[4] = {T(0), T(0), T(0), T(0)};
-    if (okA) {
-      // G rows i >= 4 qa with i = rg (mod RG); the quad of row i is inside
-      // the padded row whenever 4q <= i
-      const int ia = 4 * qa;
-      const int i0 = ia + ((rg - ia % RG) % RG + RG) % RG;
-#pragma unroll 4
-      for (int i = i0; i < c.nI; i += RG) {
-        const TV *row = G + tri_off(i);
-        const T xv = xs[i];
-        T v[4];
-        ld4(row + 4 * qa, v);
-        aA[0] += v[0] * xv; aA[1] += v[1] * xv; aA[2] += v[2] * xv; aA[3] += v[3] * xv;
-        if (okB && i >= 4 * qb) {
-          T w[4];
-          ld4(row + 4 * qb, w);
-          aB[0] += w[0] * xv; aB[1] += w[1] * xv; aB[2] += w[2] * xv; aB[3] += w[3] * xv;
-        }
-      }
-#pragma unroll 4
-      for (int q = rg; q < c.nB; q += RG) {
-        const TV *row = V + (long long)q * vstride;
-        const T xv = xb[q];
-        T v[4];
-        ld4(row + 4 * qa, v);
-        aA[0] -= v[0] * xv; aA[1] -= v[1] * xv; aA[2] -= v[2] * xv; aA[3] -= v[3] * xv;
-        if (okB) {
-          T w[4];
-          ld4(row + 4 * qb, w);
-          aB[0] -= w[0] * xv; aB[1] -= w[1] * xv; aB[2] -= w[2] * xv; aB[3] -= w[3] * xv;
-        }
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      part[k * NT + threadIdx.x] = aA[k];
-      part[(4 + k) * NT + threadIdx.x] = aB[k];
-    }
-    rowgroup_tree<T, NT, 8>(part, PW, RG);
-    if (rg == 0 && p < npairs) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int col = (k < 4 ? 4 * qa : 4 * qb) + (k & 3);
-        if (k >= 4 && qb <= qa) break;
-        if (col < it.a || col >= it.b) continue;
-        x[I[col]] = part[k * NT + pl];
-      }
-    }
-    __syncthreads();
-  }
+  if constexpr (sizeof(T) == 8) cell_bwd_cols_f64<NT>(it, c, I, G, V, vstride, xs, xb, part, x);
+  else cell_bwd_cols_f32<T, NT, TV>(it, c, I, G, V, vstride, xs, xb, part, x);
 }
 
 template <typename T, typename TV = T>
-__global__ void __launch_bounds__(kCellBwdThreads) k_cell_bwd(const CellItem *__restrict__ items,
+__global__ void __launch_bounds__(kCellBwdThreads, 4) k_cell_bwd(const CellItem *__restrict__ items,
                                                               const CellDesc *__restrict__ cells,
                                                               const int *__restrict__ idx,
                                                               const TV *__restrict__ vals,
@@ -1685,24 +1753,109 @@ __device__ __forceinline__ void root_cols_unit(int u, int nr, const int *__restr
   }
 }
 
-// A root above kRootSplitDofs: t = G_r x_r by row blocks, then x_r = G_r^T t
-// by column blocks, each a launch over ceil(n_r / kRootBlock) CTAs.
+// A root above kRootSplitDofs: t = G_r x_r by rows, a warp a row with up to eight
+// quads a lane in flight, then x_r = G_r^T t by blocks of 128 columns and
+// kRootRowChunk rows, whose partial sums the last CTA of a column block adds in
+// order (ticket counter).  Both prefetch their part of G_r into L2 before they wait
+// for the previous kernel.  In 64-row and 64-column blocks a root of 2909 DOFs kept
+// 46 CTAs busy for 111 us (34 MB); 21 us now.
+constexpr int kRootCols = 128;
 template <typename T, typename TV = T>
-__global__ void __launch_bounds__(256) k_root_rows(int nr, const int *__restrict__ ridx,
+__global__ void __launch_bounds__(256, 3) k_root_rows(int nr, const int *__restrict__ ridx,
                                                    const TV *__restrict__ G, const T *__restrict__ x,
                                                    T *__restrict__ t) {
-  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  root_rows_unit<T, 256, TV>(blockIdx.x, nr, ridx, G, x, t, reinterpret_cast<T *>(smem_raw));
+  T *xs = reinterpret_cast<T *>(smem_raw);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int step = 8 * (int)gridDim.x;
+  for (int r = blockIdx.x * 8 + warp; r < nr; r += step)
+    if (lane == 0) prefetch_block_l2(G + tri_off(r), pad4(r + 1));
+  pdl_enter();
+  const int nrp = (int)pad4(nr);
+  for (int i = threadIdx.x; i < nrp; i += 256) xs[i] = i < nr ? __ldcg(x + ridx[i]) : T(0);
+  __syncthreads();
+  constexpr int kU = sizeof(T) == 8 ? 4 : 8;
+  for (int r = blockIdx.x * 8 + warp; r < nr; r += step) {
+    const TV *row = G + tri_off(r);
+    const int nq = (r + 4) / 4;
+    T acc = T(0);
+    for (int q0 = lane; q0 < nq; q0 += 32 * kU) {
+      T v[kU][4];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        ld4_stream(row + 4 * (q0 + 32 * u), q0 + 32 * u < nq, v[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        T xv[4] = {T(0), T(0), T(0), T(0)};
+        if (q0 + 32 * u < nq) ld4(xs + 4 * (q0 + 32 * u), xv);
+        acc += v[u][0] * xv[0] + v[u][1] * xv[1] + v[u][2] * xv[2] + v[u][3] * xv[3];
+      }
+    }
+    acc = warp_reduce(acc);
+    if (lane == 0) t[r] = acc;
+  }
 }
 
+// grid = (column blocks, row chunks)
 template <typename T, typename TV = T>
-__global__ void __launch_bounds__(256) k_root_cols(int nr, const int *__restrict__ ridx,
+__global__ void __launch_bounds__(256, 4) k_root_cols(int nr, const int *__restrict__ ridx,
                                                    const TV *__restrict__ G, const T *__restrict__ t,
-                                                   T *__restrict__ x) {
+                                                   T *__restrict__ x, T *__restrict__ part,
+                                                   unsigned *__restrict__ tickets) {
+  __shared__ __align__(16) T sums[8 * kRootCols];
+  __shared__ bool last;
+  const int c0 = blockIdx.x * kRootCols, i0 = c0 + (int)blockIdx.y * kRootRowChunk;
+  const int i1 = min(nr, i0 + kRootRowChunk);
+  if (i0 < nr && threadIdx.x < kRootRowChunk && i0 + (int)threadIdx.x < i1) {
+    const int i = i0 + threadIdx.x;
+    prefetch_block_l2(G + tri_off(i) + c0, min((long long)kRootCols, pad4(i + 1) - c0));
+  }
   pdl_enter();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  root_cols_unit<T, 256, TV>(blockIdx.x, nr, ridx, G, t, x, reinterpret_cast<T *>(smem_raw));
+  if (i0 >= nr) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int col = c0 + 4 * lane;
+  constexpr int kU = 8;
+  T acc[4] = {T(0), T(0), T(0), T(0)};
+  for (int i = i0 + warp; i < i1; i += 8 * kU) {
+    T v[kU][4];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int r = i + 8 * u;
+      ld4_stream(G + tri_off(r) + col, r < i1 && col <= r, v[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const T tv = i + 8 * u < i1 ? __ldcg(t + i + 8 * u) : T(0);
+      acc[0] += v[u][0] * tv; acc[1] += v[u][1] * tv; acc[2] += v[u][2] * tv; acc[3] += v[u][3] * tv;
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) sums[warp * kRootCols + 4 * lane + e] = acc[e];
+  __syncthreads();
+  const int nch = (nr - c0 + kRootRowChunk - 1) / kRootRowChunk, j = threadIdx.x;
+  T s = T(0);
+  if (j < kRootCols) {
+    s = sums[j];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += sums[w * kRootCols + j];
+  }
+  if (nch > 1) {
+    T *pb = part + (long long)blockIdx.x * gridDim.y * kRootCols;
+    if (j < kRootCols) pb[(long long)blockIdx.y * kRootCols + j] = s;
+    __threadfence();
+    __syncthreads();
+    if (j == 0) last = atomicAdd(&tickets[blockIdx.x], 1u) == (unsigned)nch - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (j == 0) tickets[blockIdx.x] = 0u;
+    if (j < kRootCols) {
+      s = T(0);
+      for (int k = 0; k < nch; ++k) s += __ldcg(pb + (long long)k * kRootCols + j);
+    }
+  }
+  if (j < kRootCols && c0 + j < nr) x[ridx[c0 + j]] = s;
 }
 
 template <typename T, typename TV = T>
@@ -2509,21 +2662,23 @@ int apply_levels(Handle *h, const FactorValues<T> &fv, T *x, cudaStream_t s) {
         note_launch();
       }
     } else if (h->root_split) {  // row blocks, then column blocks, over many CTAs
-      const int units = (h->root_n + kRootBlock - 1) / kRootBlock;
-      const size_t sm1 = (size_t)pad4(h->root_n) * sizeof(T), sm2 = ((size_t)h->root_n + 256) * sizeof(T);
+      const int rows = std::min((h->root_n + 7) / 8, 4 * 152);
+      const dim3 cols((h->root_n + kRootCols - 1) / kRootCols, (h->root_n + kRootRowChunk - 1) / kRootRowChunk);
+      const size_t sm1 = (size_t)pad4(h->root_n) * sizeof(T);
+      T *part = reinterpret_cast<T *>(h->root_part);
       bool done = false;
       if constexpr (sizeof(T) == 4) {
         if (b16) {
           const bf16 *G = static_cast<const bf16 *>(h->bf16_vals) + h->root_G_off;
-          HIF_CUDA_TRY(launch_k(k_root_rows<T, bf16>, units, 256, sm1, s, h->root_n, ridx, G, x, rt));
-          HIF_CUDA_TRY(launch_k(k_root_cols<T, bf16>, units, 256, sm2, s, h->root_n, ridx, G, rt, x));
+          HIF_CUDA_TRY(launch_k(k_root_rows<T, bf16>, rows, 256, sm1, s, h->root_n, ridx, G, x, rt));
+          HIF_CUDA_TRY(launch_k(k_root_cols<T, bf16>, cols, 256, 0, s, h->root_n, ridx, G, rt, x, part, h->root_tk));
           done = true;
         }
       }
       if (!done) {
         const T *G = fv.vals + h->root_G_off;
-        HIF_CUDA_TRY(launch_k(k_root_rows<T>, units, 256, sm1, s, h->root_n, ridx, G, x, rt));
-        HIF_CUDA_TRY(launch_k(k_root_cols<T>, units, 256, sm2, s, h->root_n, ridx, G, rt, x));
+        HIF_CUDA_TRY(launch_k(k_root_rows<T>, rows, 256, sm1, s, h->root_n, ridx, G, x, rt));
+        HIF_CUDA_TRY(launch_k(k_root_cols<T>, cols, 256, 0, s, h->root_n, ridx, G, rt, x, part, h->root_tk));
       }
       note_launch();
     } else {

@@ -73,7 +73,9 @@ constexpr int kSplitDofs = 256;
 // default CTAs per launch the G-form cell items are cut for (hif_autotune
 // picks per level among multiples of the SM count)
 constexpr int kDefaultItemTarget = 152 * 4;
+constexpr double kItemBytes = 96 * 1024;  // FP32 factor bytes of an item (see build_items)
 constexpr int kRootSplitDofs = 512;
+constexpr int kRootRowChunk = 128;  // rows of a CTA of the split root's transposed product
 constexpr int kSplitRows = 32;   // rows of H per CTA (forward)
 constexpr int kSplitCols = 64;   // columns of H per CTA (backward)
 __host__ __device__ inline long long tri_off(long long i) {
@@ -290,6 +292,8 @@ struct hif_handle {
   hifcn::UpperLevel *upper_levels = nullptr;  // device
   void *upper_rt = nullptr;                   // device root scratch (root_n doubles)
   bool root_split = false;                    // root applied by row- and column-block launches
+  void *root_part = nullptr;                  // its partial column sums and
+  unsigned *root_tk = nullptr;                // ticket counters (zero between launches)
   // small FP32 roots: A_L^{-1} = G_r^T G_r as a full symmetric matrix (FP32,
   // rows padded to root_S_ld), applied by one pass of row dots
   float *root_S = nullptr;
