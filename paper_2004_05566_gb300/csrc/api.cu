@@ -322,7 +322,8 @@ int finish_device_factor(Handle *h, cudaStream_t s) {
   if (!lean) HIF_TRY(dev_alloc(h, (void **)&h->f64.contrib, h->max_contrib * sizeof(double)));
   if (h->opt.precision == HIF_FP32 || h->opt.precision == HIF_FP32_BF16TOP) {
     if (!lean) HIF_TRY(dev_alloc(h, (void **)&h->f32.vals, h->nvals * sizeof(float)));
-    HIF_TRY(dev_alloc(h, (void **)&h->f32.contrib, h->max_contrib * sizeof(float)));
+    // twice the largest level: the fused upper levels keep two levels' contributions
+    HIF_TRY(dev_alloc(h, (void **)&h->f32.contrib, 2 * pad4(h->max_contrib) * sizeof(float)));
     HIF_TRY(dev_alloc(h, (void **)&h->f32.work, h->N * sizeof(float)));
     HIF_TRY(dev_alloc(h, (void **)&h->f32.xI, h->N * sizeof(float)));
     HIF_TRY(dev_alloc(h, (void **)&h->f32.gs, std::max<long long>(gs_max, 1) * sizeof(float)));
@@ -347,6 +348,7 @@ int finish_device_factor(Handle *h, cudaStream_t s) {
   HIF_TRY(make_root_dense(h, s));
   HIF_CUDA_TRY(cudaStreamSynchronize(s));
   HIF_TRY(build_upper_plan(h));
+  HIF_TRY(build_level_plan(h));
   HIF_TRY(build_view(h));
   return HIF_OK;
 }
@@ -465,6 +467,7 @@ int create_handle(const hif_grid *grid, const double *a_nodes, double dt, const 
 // stencil stay).
 void release_factor(Handle *h) {
   destroy_pcg_graphs(h);
+  destroy_level_plan(h);
   destroy_multi_state(h);  // its buffers are among the allocations freed below
   for (size_t i = h->factor_alloc_begin; i < h->allocations.size(); ++i) dev_free(h->allocations[i]);
   h->allocations.resize(h->factor_alloc_begin);
@@ -663,6 +666,7 @@ hif_handle::~hif_handle() {
   cudaDeviceSynchronize();
   hifcn::destroy_pcg_graphs(this);
   hifcn::destroy_multi_state(this);
+  hifcn::destroy_level_plan(this);
   for (auto &r : stat_pending) {
     cudaEventDestroy(r.a);
     cudaEventDestroy(r.b);
@@ -1047,6 +1051,7 @@ int hif_autotune(hif_handle *h, hif_stream stream) {
   HIF_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const bool stats_was = h->stats_on;
   h->stats_on = true;
+  h->fuse_off = true;
   const int L = h->L, reps = 5;
   const std::vector<int> cand = {sms, 2 * sms, 4 * sms, 8 * sms, 16 * sms};
   std::vector<std::vector<double>> t(L, std::vector<double>(cand.size(), 1e30));
@@ -1095,6 +1100,8 @@ int hif_autotune(hif_handle *h, hif_stream stream) {
     }
   }
   h->tma_ctas = cbest;
+  h->fuse_off = false;
+  h->fuse_lb = fused_start(h);  // the levels of the bulk-copy kernels may have changed
   destroy_pcg_graphs(h);
   h->stats_on = stats_was;
   int cnt = 0;

@@ -341,13 +341,14 @@ __global__ void __launch_bounds__(kCellFwdThreads, sizeof(T) == 4 ? 3 : 4) k_cel
                                           reinterpret_cast<T *>(smem_raw));
 }
 
-// Forward group step (K^T C^T): x_g <- H (x_g - sum of the cells' contributions).
+// Forward group step (K^T C^T): x_g <- H (x_g - sum of the cells' contributions),
+// from xin to x (the same vector, or another one).
 template <typename T, int NT, typename TV = T, bool PDL = false>
 __device__ __forceinline__ void group_fwd_unit(const GroupDesc &g, const int *__restrict__ idx,
                                                const long long *__restrict__ cptr,
                                                const long long *__restrict__ cslot,
                                                const TV *__restrict__ vals,
-                                               const T *__restrict__ contrib, T *__restrict__ x,
+                                               const T *__restrict__ contrib, const T *xin, T *x,
                                                T *xs) {
   const int *gi = idx + g.idx_off;
   const int np = (int)pad4(g.n);
@@ -357,7 +358,7 @@ __device__ __forceinline__ void group_fwd_unit(const GroupDesc &g, const int *__
   for (int i = threadIdx.x; i < np; i += NT) {
     T v = T(0);
     if (i < g.n) {
-      v = __ldcg(x + gi[i]);
+      v = __ldcg(xin + gi[i]);
       const long long a = cptr[g.cptr_off + i], b = cptr[g.cptr_off + i + 1];
       for (long long s = a; s < b; ++s) v -= __ldcg(contrib + cslot[s]);
     }
@@ -397,7 +398,7 @@ __device__ __forceinline__ void group_fwd_small_warp(const GroupDesc &g, const i
                                                      const long long *__restrict__ cslot,
                                                      const TV *__restrict__ vals,
                                                      const T *__restrict__ contrib,
-                                                     T *__restrict__ x, T *xs) {
+                                                     const T *xin, T *x, T *xs) {
   const int lane = threadIdx.x & 31;
   const int *gi = idx + g.idx_off;
   const int nq = (int)pad4(g.n) / 4;
@@ -431,7 +432,7 @@ __device__ __forceinline__ void group_fwd_small_warp(const GroupDesc &g, const i
   unit_dependency_point<PDL>();
   T v = T(0);
   if (lane < g.n) {
-    v = __ldcg(x + dof);
+    v = __ldcg(xin + dof);
 #pragma unroll
     for (int k = 0; k < kSlots; ++k)
       if (a + k < b) v -= __ldcg(contrib + sl[k]);
@@ -463,7 +464,7 @@ __device__ __forceinline__ void group_fwd_small_warp(const GroupDesc &g, const i
 
 template <typename T, typename TV = T, bool PDL = false, bool kPreload = false>
 __device__ __forceinline__ void group_bwd_small_warp(const GroupDesc &g, const int *__restrict__ idx,
-                                                     const TV *__restrict__ vals, T *__restrict__ x,
+                                                     const TV *__restrict__ vals, const T *xin, T *x,
                                                      T *xs) {
   const int lane = threadIdx.x & 31;
   const int *gi = idx + g.idx_off;
@@ -484,7 +485,7 @@ __device__ __forceinline__ void group_bwd_small_warp(const GroupDesc &g, const i
     if (lane < g.n) prefetch_block_l2(H + (long long)lane * np, np);
   }
   unit_dependency_point<PDL>();
-  xs[lane] = lane < g.n ? __ldcg(x + dof) : T(0);
+  xs[lane] = lane < g.n ? __ldcg(xin + dof) : T(0);
   __syncwarp();
   if (lane < g.n) {
     T acc = T(0);
@@ -541,14 +542,14 @@ __device__ __forceinline__ void rowgroup_tree(T *part, int CW, int RG) {
 // holds pad4(n) + 4 NT elements.
 template <typename T, int NT, typename TV = T, bool PDL = false>
 __device__ __forceinline__ void group_bwd_unit(const GroupDesc &g, const int *__restrict__ idx,
-                                               const TV *__restrict__ vals, T *__restrict__ x, T *xs) {
+                                               const TV *__restrict__ vals, const T *xin, T *x, T *xs) {
   const int np = (int)pad4(g.n), nq = np / 4;
   T *part = xs + np;  // 4 * NT
   const int *gi = idx + g.idx_off;
   if constexpr (PDL)
     if (threadIdx.x == 0) prefetch_block_l2(vals + g.H_off, (long long)g.n * np);
   unit_dependency_point<PDL>();
-  for (int i = threadIdx.x; i < g.n; i += NT) xs[i] = __ldcg(x + gi[i]);
+  for (int i = threadIdx.x; i < g.n; i += NT) xs[i] = __ldcg(xin + gi[i]);
   __syncthreads();
   const TV *H = vals + g.H_off;
   int CW, RG;
@@ -592,13 +593,13 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_group_fwd_level(
   T *sm = reinterpret_cast<T *>(smem_raw);
   const int u = blockIdx.x;
   if (u < nlarge) {
-    group_fwd_unit<T, kSmallWarps * 32, TV, true>(groups[large[u]], idx, cptr, cslot, vals, contrib, x, sm);
+    group_fwd_unit<T, kSmallWarps * 32, TV, true>(groups[large[u]], idx, cptr, cslot, vals, contrib, x, x, sm);
     return;
   }
   const int warp = threadIdx.x >> 5;
   const int t = (u - nlarge) * kSmallWarps + warp;
   if (t < nsmall)
-    group_fwd_small_warp<T, TV, true, true>(groups[small[t]], idx, cptr, cslot, vals, contrib, x,
+    group_fwd_small_warp<T, TV, true, true>(groups[small[t]], idx, cptr, cslot, vals, contrib, x, x,
                                       sm + 32 * warp);
   else
     pdl_enter();  // a warp without an entity
@@ -613,13 +614,13 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_group_bwd_level(
   T *sm = reinterpret_cast<T *>(smem_raw);
   const int u = blockIdx.x;
   if (u < nlarge) {
-    group_bwd_unit<T, kSmallWarps * 32, TV, true>(groups[large[u]], idx, vals, x, sm);
+    group_bwd_unit<T, kSmallWarps * 32, TV, true>(groups[large[u]], idx, vals, x, x, sm);
     return;
   }
   const int warp = threadIdx.x >> 5;
   const int t = (u - nlarge) * kSmallWarps + warp;
   if (t < nsmall)
-    group_bwd_small_warp<T, TV, true, true>(groups[small[t]], idx, vals, x, sm + 32 * warp);
+    group_bwd_small_warp<T, TV, true, true>(groups[small[t]], idx, vals, x, x, sm + 32 * warp);
   else
     pdl_enter();  // a warp without an entity
 }
@@ -1858,6 +1859,8 @@ __global__ void __launch_bounds__(256, 4) k_root_cols(int nr, const int *__restr
   if (j < kRootCols && c0 + j < nr) x[ridx[c0 + j]] = s;
 }
 
+#include "fused_levels.cuh"
+
 template <typename T, typename TV = T>
 __global__ void __launch_bounds__(kUpperThreads) k_upper_sweep(
     const UpperPhase *__restrict__ phases, int nphase, const UpperLevel *__restrict__ levels,
@@ -1881,11 +1884,11 @@ __global__ void __launch_bounds__(kUpperThreads) k_upper_sweep(
           break;
         case kPhaseGroupFwd:
           if (u < L.nlarge) {
-            group_fwd_unit<T, NT, TV>(L.groups[L.large[u]], idx, cptr, cslot, vals, contrib, x, sm);
+            group_fwd_unit<T, NT, TV>(L.groups[L.large[u]], idx, cptr, cslot, vals, contrib, x, x, sm);
           } else {
             const int t = (u - L.nlarge) * NW + warp;
             if (t < L.nsmall)
-              group_fwd_small_warp<T, TV>(L.groups[L.small[t]], idx, cptr, cslot, vals, contrib, x,
+              group_fwd_small_warp<T, TV>(L.groups[L.small[t]], idx, cptr, cslot, vals, contrib, x, x,
                                       sm + 32 * warp);
           }
           break;
@@ -1897,10 +1900,10 @@ __global__ void __launch_bounds__(kUpperThreads) k_upper_sweep(
           break;
         case kPhaseGroupBwd:
           if (u < L.nlarge) {
-            group_bwd_unit<T, NT, TV>(L.groups[L.large[u]], idx, vals, x, sm);
+            group_bwd_unit<T, NT, TV>(L.groups[L.large[u]], idx, vals, x, x, sm);
           } else {
             const int t = (u - L.nlarge) * NW + warp;
-            if (t < L.nsmall) group_bwd_small_warp<T, TV>(L.groups[L.small[t]], idx, vals, x, sm + 32 * warp);
+            if (t < L.nsmall) group_bwd_small_warp<T, TV>(L.groups[L.small[t]], idx, vals, x, x, sm + 32 * warp);
           }
           break;
         default:  // kPhaseCellBwd
@@ -1980,11 +1983,11 @@ __device__ __forceinline__ void flow_run_unit(int type, const UpperLevel &L, int
       break;
     case kPhaseGroupFwd:
       if (u < L.nlarge) {
-        group_fwd_unit<T, NT, TV>(L.groups[L.large[u]], idx, cptr, cslot, vals, contrib, x, sm);
+        group_fwd_unit<T, NT, TV>(L.groups[L.large[u]], idx, cptr, cslot, vals, contrib, x, x, sm);
       } else {
         const int t = (u - L.nlarge) * NW + warp;
         if (t < L.nsmall)
-          group_fwd_small_warp<T, TV>(L.groups[L.small[t]], idx, cptr, cslot, vals, contrib, x,
+          group_fwd_small_warp<T, TV>(L.groups[L.small[t]], idx, cptr, cslot, vals, contrib, x, x,
                                       sm + 32 * warp);
       }
       break;
@@ -1996,10 +1999,10 @@ __device__ __forceinline__ void flow_run_unit(int type, const UpperLevel &L, int
       break;
     case kPhaseGroupBwd:
       if (u < L.nlarge) {
-        group_bwd_unit<T, NT, TV>(L.groups[L.large[u]], idx, vals, x, sm);
+        group_bwd_unit<T, NT, TV>(L.groups[L.large[u]], idx, vals, x, x, sm);
       } else {
         const int t = (u - L.nlarge) * NW + warp;
-        if (t < L.nsmall) group_bwd_small_warp<T, TV>(L.groups[L.small[t]], idx, vals, x, sm + 32 * warp);
+        if (t < L.nsmall) group_bwd_small_warp<T, TV>(L.groups[L.small[t]], idx, vals, x, x, sm + 32 * warp);
       }
       break;
     default:  // kPhaseCellBwd
@@ -2243,31 +2246,31 @@ __global__ void __launch_bounds__(256) k_merged_phase(const int *__restrict__ pr
     } else if constexpr (KIND == kPhaseGroupFwd) {
       if (u < L.nlarge) {
         const GroupDesc g = L.groups[L.large[u]];
-        if (b16) group_fwd_unit<float, 256, __nv_bfloat16>(g, idx, v->cptr, v->cslot, vals16, v->contrib, v->z, sm);
-        else group_fwd_unit<float, 256>(g, idx, v->cptr, v->cslot, vals, v->contrib, v->z, sm);
+        if (b16) group_fwd_unit<float, 256, __nv_bfloat16>(g, idx, v->cptr, v->cslot, vals16, v->contrib, v->z, v->z, sm);
+        else group_fwd_unit<float, 256>(g, idx, v->cptr, v->cslot, vals, v->contrib, v->z, v->z, sm);
       } else {
         const int warp = threadIdx.x >> 5;
         const int t = (u - L.nlarge) * 8 + warp;
         if (t < L.nsmall) {
           const GroupDesc g = L.groups[L.small[t]];
           if (b16)
-            group_fwd_small_warp<float, __nv_bfloat16>(g, idx, v->cptr, v->cslot, vals16, v->contrib, v->z,
+            group_fwd_small_warp<float, __nv_bfloat16>(g, idx, v->cptr, v->cslot, vals16, v->contrib, v->z, v->z,
                                                        sm + 32 * warp);
-          else group_fwd_small_warp<float>(g, idx, v->cptr, v->cslot, vals, v->contrib, v->z, sm + 32 * warp);
+          else group_fwd_small_warp<float>(g, idx, v->cptr, v->cslot, vals, v->contrib, v->z, v->z, sm + 32 * warp);
         }
       }
     } else {  // kPhaseGroupBwd
       if (u < L.nlarge) {
         const GroupDesc g = L.groups[L.large[u]];
-        if (b16) group_bwd_unit<float, 256, __nv_bfloat16>(g, idx, vals16, v->z, sm);
-        else group_bwd_unit<float, 256>(g, idx, vals, v->z, sm);
+        if (b16) group_bwd_unit<float, 256, __nv_bfloat16>(g, idx, vals16, v->z, v->z, sm);
+        else group_bwd_unit<float, 256>(g, idx, vals, v->z, v->z, sm);
       } else {
         const int warp = threadIdx.x >> 5;
         const int t = (u - L.nlarge) * 8 + warp;
         if (t < L.nsmall) {
           const GroupDesc g = L.groups[L.small[t]];
-          if (b16) group_bwd_small_warp<float, __nv_bfloat16>(g, idx, vals16, v->z, sm + 32 * warp);
-          else group_bwd_small_warp<float>(g, idx, vals, v->z, sm + 32 * warp);
+          if (b16) group_bwd_small_warp<float, __nv_bfloat16>(g, idx, vals16, v->z, v->z, sm + 32 * warp);
+          else group_bwd_small_warp<float>(g, idx, vals, v->z, v->z, sm + 32 * warp);
         }
       }
     }
@@ -2298,6 +2301,13 @@ int set_smem_limits() {
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_group_fwd_level<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_group_bwd_level<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_root<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+  if constexpr (sizeof(T) == 4) {
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_level_fwd<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_level_fwd<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_level_bwd<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_level_bwd<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_level_top, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+  }
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_root_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_root_cols<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_group_rows_split<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
@@ -2617,6 +2627,59 @@ int launch_upper(Handle *h, const FactorValues<T> &fv, T *x, cudaStream_t s) {
   return HIF_OK;
 }
 
+// shared memory of the fused launches of a level (fused_levels.cuh), in elements
+size_t fused_fwd_elems(const FusedLevel &F) {
+  return std::max<size_t>({2 * (size_t)F.max_sum + pad4(F.max_nI), (size_t)pad4(F.max_ng), (size_t)F.nt});
+}
+size_t fused_bwd_elems(const FusedLevel &F) {
+  return std::max<size_t>({2 * (size_t)pad4(F.max_nI) + pad4(F.max_nB) + 2 * (size_t)F.max_sum + 4 * (size_t)F.nt,
+                           (size_t)pad4(F.max_ng) + 4 * (size_t)F.nt});
+}
+size_t fused_top_elems(const FusedLevel &F, int nr) {
+  return 2 * (size_t)F.max_sum + 2 * (size_t)pad4(nr) + 4 * kFuseTopThreads;
+}
+
+// levels fl .. L - 1 (entity steps) and the root through the fused launches
+int launch_fused_levels(Handle *h, const FactorValues<float> &fv, int fl, float *x, cudaStream_t s) {
+  using T = float;
+  const std::vector<FusedLevel> &plan = *static_cast<const std::vector<FusedLevel> *>(h->fuse_plan);
+  const int L = h->L;
+  const double E = sizeof(T);
+  T *buf[2] = {x, fv.alt};
+  T *con[2] = {fv.contrib, fv.contrib + h->fuse_contrib_off};
+  auto units = [](const FusedLevel &F, int first, int warps) { return first + F.nlarge + (F.nsmall + warps - 1) / warps; };
+  for (int l = fl; l < L - 1; ++l) {
+    const FusedLevel &F = plan[l];
+    const LevelDev &g = h->lv[l], &c = h->lv[l + 1];
+    const int k = (l - fl) & 1;
+    StatScope sc(h, "level_fwd", l, (g.vals_group + c.vals_cell + g.vec_group + g.contrib + c.vec_cell_fwd + c.contrib) * E +
+                 g.idx_group + g.cslot_bytes + c.idx_cell_fwd, s);
+    HIF_CUDA_TRY(launch_k(F.nt == 256 ? k_level_fwd<256> : k_level_fwd<512>, units(F, F.nitems, F.nt / 32), F.nt,
+                          fused_fwd_elems(F) * sizeof(T), s, F, h->idx, h->cptr, h->cslot, fv.vals, con[k],
+                          con[1 - k], fv.xI, buf[k], buf[1 - k]));
+  }
+  {
+    const FusedLevel &F = plan[L - 1];
+    const LevelDev &g = h->lv[L - 1];
+    const int k = (L - 1 - fl) & 1;
+    const double nr = h->root_n;
+    StatScope sc(h, "level_top", -1, (2 * g.vals_group + 2 * g.vec_group + g.contrib + nr * (nr + 3)) * E + g.idx_group, s);
+    HIF_CUDA_TRY(launch_k(k_level_top, 1, kFuseTopThreads, fused_top_elems(F, h->root_n) * sizeof(T), s, F,
+                          h->root_n, fv.vals, h->cslot, h->root_S, h->root_S_ld, con[k],
+                          buf[k], buf[k]));
+  }
+  for (int l = L - 2; l >= fl; --l) {
+    const FusedLevel &F = plan[l];
+    const LevelDev &g = h->lv[l], &c = h->lv[l + 1];
+    const int k = (l - fl) & 1;
+    StatScope sc(h, "level_bwd", l, (g.vals_group + c.vals_cell + g.vec_group + c.vec_cell_bwd) * E + g.idx_group_bwd +
+                 c.idx_cell_bwd, s);
+    HIF_CUDA_TRY(launch_k(F.nt == 256 ? k_level_bwd<256> : k_level_bwd<512>, units(F, F.ncells, F.nt / 32), F.nt,
+                          fused_bwd_elems(F) * sizeof(T), s, F, h->idx, fv.vals, fv.xI, buf[1 - k], buf[k]));
+  }
+  return HIF_OK;
+}
+
 template <typename T>
 int apply_levels(Handle *h, const FactorValues<T> &fv, T *x, cudaStream_t s) {
   HIF_TRY(set_smem_limits<T>());
@@ -2637,6 +2700,22 @@ int apply_levels(Handle *h, const FactorValues<T> &fv, T *x, cudaStream_t s) {
   const bool flow = h->use_flow && h->flow_grid[pi] > 0;
   const bool fused = !flow && h->use_upper && h->upper_grid[pi] > 0;
   const int lb = flow ? h->flow_lb : fused ? h->upper_lb : h->L;  // levels >= lb in one launch
+  if constexpr (sizeof(T) == 4) {
+    const int fl = !flow && !fused && !h->fuse_off ? h->fuse_lb : -1;
+    if (fl >= 0) {  // the small upper levels, one launch per level and direction
+      for (int l = 0; l <= fl; ++l) {
+        HIF_TRY(launch_cell_fwd<T>(h, h->lv[l], l, fv, x, s));
+        if (l < fl) HIF_TRY(launch_group_fwd<T>(h, h->lv[l], l, fv, x, s));
+      }
+      HIF_TRY(launch_fused_levels(h, fv, fl, x, s));
+      for (int l = fl; l >= 0; --l) {
+        if (l < fl) HIF_TRY(launch_group_bwd<T>(h, h->lv[l], l, fv, x, s));
+        HIF_TRY(launch_cell_bwd<T>(h, h->lv[l], l, fv, x, s));
+      }
+      HIF_CUDA_TRY(cudaGetLastError());
+      return HIF_OK;
+    }
+  }
   for (int l = 0; l < lb; ++l) {
     HIF_TRY(launch_cell_fwd<T>(h, h->lv[l], l, fv, x, s));
     if (flow && l == lb - 1) break;
@@ -3279,8 +3358,180 @@ int build_upper_plan(Handle *h) {
   return HIF_OK;
 }
 
-namespace {
-}  // namespace
+// Plan of the fused upper-level launches (fused_levels.cuh) of the FP32 apply: per
+// level l the cells of level l + 1 (for the last level the root) with their inner
+// entities, from the index lists of the factor.
+// Each level is taken only if it has the structure the kernels rely on (an entity's
+// surviving DOFs lie in the interior of one cell, or all on boundaries) and fits
+// them; a level that does not ends the fused range above it.
+int build_level_plan(Handle *h) {
+  h->fuse_lb = -1;
+  const char *off = std::getenv("HIFCN_NO_LEVEL_FUSE");
+  if ((off && off[0] == '1') || !h->has_f32 || h->has_bf16 || !h->root_S) return HIF_OK;
+  const int L = h->L;
+  if (!h->fuse_plan) h->fuse_plan = new std::vector<FusedLevel>();
+  auto &plan = *static_cast<std::vector<FusedLevel> *>(h->fuse_plan);
+  plan.assign(L, FusedLevel{});
+  std::vector<int> grp(h->N, -1), at(h->N, -1);  // entity of a DOF of level l, interior index in a cell
+  int fl = L;
+  const size_t lim = 100 * 1024;
+  for (int l = L - 1; l >= 0; --l) {
+    const LevelHost &H = h->lv_host[l];
+    const LevelDev &D = h->lv[l];
+    if (D.split || H.groups.empty()) break;
+    const bool top = l == L - 1;
+    if (!top && h->lv[l + 1].max_nI > kFuseMaxNI) break;
+    std::vector<CellDesc> parents;
+    if (top) {
+      CellDesc r{};
+      r.nI = h->root_n;
+      r.I_off = h->root_idx_off;
+      parents.push_back(r);
+    } else {
+      parents = h->lv_host[l + 1].cells;
+    }
+    for (int g = 0; g < (int)H.groups.size(); ++g)
+      for (int i = 0; i < H.groups[g].n; ++i) grp[h->idx_host[H.groups[g].idx_off + i]] = g;
+    std::vector<char> onb(h->N, 0);  // DOFs of level l + 1's entities
+    bool ok = true;
+    if (!top)
+      for (const GroupDesc &G : h->lv_host[l + 1].groups)
+        for (int i = 0; i < G.n; ++i) {
+          const int d = h->idx_host[G.idx_off + i];
+          onb[d] = 1;
+          ok = ok && grp[d] >= 0;
+        }
+    std::vector<char> inner(H.groups.size(), 0);
+    std::vector<FusedCell> fc;
+    std::vector<FusedItem> items;
+    std::vector<FusedGroup> fg;
+    std::vector<FusedPos> pos;
+    std::vector<int> imap;
+    FusedLevel F{};
+    std::vector<int> soff(H.groups.size(), 0);
+    for (const CellDesc &c : parents) {
+      if (!ok) break;
+      FusedCell f{};
+      f.c = c;
+      f.cat_off = (long long)pos.size();
+      f.map_off = (long long)imap.size();
+      f.g_off = (int)fg.size();
+      const int *I = h->idx_host.data() + c.I_off;
+      for (int i = 0; i < c.nI; ++i) {
+        const int g = grp[I[i]];
+        if (g < 0) ok = false;
+        at[I[i]] = i;
+        if (g < 0 || inner[g] == 2) continue;
+        if (inner[g] == 1) ok = false;  // inside two cells
+        inner[g] = 2;
+        const GroupDesc &G = H.groups[g];
+        soff[g] = f.nsum;
+        fg.push_back(FusedGroup{G.H_off, G.n, f.nsum});
+        f.nsum += (int)pad4(G.n);
+        ++f.ng;
+      }
+      if (!ok) break;
+      for (int k = 0; k < f.ng; ++k) {
+        const FusedGroup &G = fg[f.g_off + k];
+        const GroupDesc *gd = nullptr;
+        for (int i = 0; i < c.nI && !gd; ++i)
+          if (soff[grp[I[i]]] == G.soff) gd = &H.groups[grp[I[i]]];
+        const int np = (int)pad4(G.n);
+        for (int i = 0; i < np; ++i) {
+          FusedPos p{G.H_off + (long long)i * np, -1, G.soff, 0, -1, G.n, 0, 0, 0};
+          if (i < G.n) {
+            p.dof = h->idx_host[gd->idx_off + i];
+            p.nq = np / 4;
+            p.ipos = at[p.dof];
+            if (p.ipos < 0 && onb[p.dof]) ok = false;  // survives, but outside the cell
+            p.c0 = (int)h->cptr_host[gd->cptr_off + i];
+            p.nc = (int)(h->cptr_host[gd->cptr_off + i + 1] - h->cptr_host[gd->cptr_off + i]);
+          }
+          pos.push_back(p);
+        }
+      }
+      std::vector<int> where(c.nI, -1);
+      for (int t = 0; t < f.nsum; ++t)
+        if (pos[f.cat_off + t].ipos >= 0) where[pos[f.cat_off + t].ipos] = t;
+      for (int i = 0; i < c.nI; ++i) {
+        ok = ok && where[i] >= 0;
+        imap.push_back(where[i]);
+        at[I[i]] = -1;
+        inner[grp[I[i]]] = 1;
+      }
+      F.max_sum = std::max(F.max_sum, f.nsum);
+      F.max_nI = std::max(F.max_nI, c.nI);
+      F.max_nB = std::max(F.max_nB, c.nB);
+      fc.push_back(f);
+    }
+    for (const GroupDesc &G : H.groups)
+      for (int i = 0; i < G.n; ++i) grp[h->idx_host[G.idx_off + i]] = -1;
+    if (!ok || F.max_sum > kFuseMaxSum || h->cslot_host.size() > 0x7fffffffu) break;
+    std::vector<int> sm, lg;
+    for (int g = 0; g < (int)H.groups.size(); ++g)
+      if (!inner[g]) (H.groups[g].n <= 32 ? sm : lg).push_back(g);
+    if (top && !(sm.empty() && lg.empty())) break;  // an entity the root does not hold
+    F.max_ng = D.max_ng;
+    if (!top) {
+      // items: at most kFuseItems CTAs where the cells are fewer, at least 32 rows each
+      const int nc = (int)fc.size();
+      for (int c = 0; c < nc; ++c) {
+        const int rows = fc[c].c.nB + fc[c].c.nI;
+        const int chunks = std::max(1, std::min(kFuseItems / nc, (rows + 31) / 32));
+        const int per = std::max(32, ((rows + chunks - 1) / chunks + 31) / 32 * 32);
+        for (int a = 0; a < std::max(rows, 1); a += per)
+          items.push_back(FusedItem{c, a, std::min(rows, a + per), a == 0 ? 1 : 0});
+      }
+    }
+    F.nitems = (int)items.size();
+    F.nt = (int)fc.size() <= kFuseWideCells ? 512 : 256;
+    F.ncells = (int)fc.size();
+    F.nsmall = (int)sm.size();
+    F.nlarge = (int)lg.size();
+    F.groups = D.groups;
+    if (std::max({fused_fwd_elems(F), fused_bwd_elems(F), top ? fused_top_elems(F, h->root_n) : 0}) * sizeof(float) > lim)
+      break;
+    auto up = [&](auto &v, auto **out) -> int {
+      using E = typename std::remove_reference<decltype(v[0])>::type;
+      E *d = nullptr;
+      HIF_TRY(dev_alloc(h, (void **)&d, std::max<size_t>(1, v.size()) * sizeof(E)));
+      if (!v.empty()) HIF_CUDA_TRY(cudaMemcpy(d, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice));
+      *out = d;
+      return HIF_OK;
+    };
+    HIF_TRY(up(fc, &F.cells));
+    HIF_TRY(up(items, &F.items));
+    HIF_TRY(up(fg, &F.fgroups));
+    HIF_TRY(up(pos, &F.pos));
+    HIF_TRY(up(imap, &F.imap));
+    HIF_TRY(up(sm, &F.small));
+    HIF_TRY(up(lg, &F.large));
+    plan[l] = F;
+    fl = l;
+  }
+  if (fl >= L) return HIF_OK;
+  // contributions of consecutive levels side by side
+  h->fuse_contrib_off = pad4(h->max_contrib);
+  HIF_TRY(dev_alloc(h, (void **)&h->f32.alt, h->N * sizeof(float)));
+  h->fuse_first = fl;
+  h->fuse_lb = fused_start(h);
+  return HIF_OK;
+}
+
+// the fused range starts above the levels of the bulk-copy kernels
+int fused_start(const Handle *h) {
+  if (!h->f32.alt) return -1;
+  int lb = h->fuse_first;
+  for (int l = lb + 1; l < h->L; ++l)
+    if (use_tma(h, h->lv[l], sizeof(float))) lb = l;
+  return lb;
+}
+
+void destroy_level_plan(Handle *h) {
+  delete static_cast<std::vector<FusedLevel> *>(h->fuse_plan);
+  h->fuse_plan = nullptr;
+  h->fuse_lb = -1;
+}
 
 int apply_inplace_f64(Handle *h, double *x, cudaStream_t s) { return apply_levels<double>(h, h->f64, x, s); }
 

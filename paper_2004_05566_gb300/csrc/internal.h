@@ -235,6 +235,7 @@ struct FactorValues {
   T *gs = nullptr;         // device scratch of the split entity steps (max gs_total)
   T *work = nullptr;       // device work vector (N) for the reduced-precision apply
   T *xI = nullptr;         // device N-vector: forward values of the cell interiors
+  T *alt = nullptr;        // device N-vector (FP32): the other vector of the fused upper levels
 };
 
 }  // namespace hifcn
@@ -325,6 +326,14 @@ struct hif_handle {
   size_t upper_smem[2] = {0, 0};              // dynamic shared memory, FP64 / FP32
   int upper_grid[2] = {0, 0};                 // CTAs of the cluster, FP64 / FP32
   double upper_bytes[2] = {0, 0};             // algorithmic bytes per launch, FP64 / FP32
+  // fused upper levels of the FP32 apply (fused_levels.cuh): per-level tables, the
+  // lowest level whose entity step is fused (-1: none), and the second part of the
+  // contribution scratch
+  void *fuse_plan = nullptr;
+  int fuse_lb = -1;
+  int fuse_first = 0;     // lowest level the tables cover
+  bool fuse_off = false;  // per-level launches while tuning
+  long long fuse_contrib_off = 0;
   bool use_graph = true;
   bool use_tma = true;                // bulk-copy staging of the leaf cell blocks
   double *partials = nullptr;  // per-block partial sums
@@ -403,6 +412,9 @@ int stencil_matvec(Handle *h, const double *x, double *y, cudaStream_t s);
 int build_device_factor(Handle *h, const std::vector<double> &vals64, cudaStream_t s);
 int apply_inverse(Handle *h, const double *x, double *y, int precision, cudaStream_t s);
 int build_upper_plan(Handle *h);
+int build_level_plan(Handle *h);
+void destroy_level_plan(Handle *h);
+int fused_start(const Handle *h);
 bool level_uses_sform(const Handle *h, int l);
 int build_view(Handle *h);
 int build_items(Handle *h, LevelDev &D, const LevelHost &H, int target, cudaStream_t s);
