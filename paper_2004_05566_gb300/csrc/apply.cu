@@ -998,6 +998,62 @@ struct CellMeta {
   CellDesc c;
   int nch;
   int cs[kMaxChunks + 1];
+  const float *vals;  // of the cell's handle: factor values, the vector, contributions
+  float *x, *contrib;
+};
+
+// Where the bulk-copy kernels find cell ci of a launch: the level of one handle, or
+// (merged batched steps) the same level of several handles, whose cells are numbered
+// one handle after another.
+struct OneLevel {
+  const CellDesc *cells;
+  const int2 *chunk_of;  // first entry in the chunk table and number of chunks
+  const int *chunk_tab, *idx_;
+  const float *vals_;
+  float *x_, *contrib_;
+  // handle of cell ci (-1: its solve has ended, the cell counts as empty), its cell
+  __device__ __forceinline__ int find(int) const { return 0; }
+  __device__ __forceinline__ void cell(int, int ci, CellDesc &c, int2 &co) const {
+    c = cells[ci];
+    co = chunk_of[ci];
+  }
+  __device__ __forceinline__ const int *tab(int) const { return chunk_tab; }
+  __device__ __forceinline__ const int *idx(int) const { return idx_; }
+  __device__ __forceinline__ const float *vals(int) const { return vals_; }
+  __device__ __forceinline__ float *x(int) const { return x_; }
+  __device__ __forceinline__ float *contrib(int) const { return contrib_; }
+};
+// pre[p]: first cell of handle p (K + 1 entries); bwd selects the chunk table
+struct BatchLevel {
+  const int *pre;
+  int K, level, bwd;
+  HandleView *const *views;
+  const int *active;
+  __device__ __forceinline__ int find(int ci) const {
+    int lo = 0, hi = K;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (pre[mid] <= ci) lo = mid;
+      else hi = mid;
+    }
+    return active[lo] ? lo : -1;
+  }
+  __device__ __forceinline__ void cell(int p, int ci, CellDesc &c, int2 &co) const {
+    if (p < 0) {
+      c = CellDesc{};
+      co = make_int2(0, 0);
+      return;
+    }
+    const LevelView &L = views[p]->lv[level];
+    c = L.cells[ci - pre[p]];
+    co = L.chunk_of[bwd][ci - pre[p]];
+  }
+  __device__ __forceinline__ const HandleView *view(int p) const { return views[p < 0 ? 0 : p]; }
+  __device__ __forceinline__ const int *tab(int p) const { return view(p)->lv[level].chunk_tab[bwd]; }
+  __device__ __forceinline__ const int *idx(int p) const { return view(p)->idx; }
+  __device__ __forceinline__ const float *vals(int p) const { return view(p)->vals; }
+  __device__ __forceinline__ float *x(int p) const { return view(p)->z; }
+  __device__ __forceinline__ float *contrib(int p) const { return view(p)->contrib; }
 };
 
 // Copy warp: lane 0 streams, for each cell the CTA owns (cells blockIdx.x,
@@ -1019,8 +1075,7 @@ __device__ __forceinline__ void drain_ring(int k, unsigned long long *full) {
 }
 
 template <typename T, int NS>
-__device__ __forceinline__ void produce_cells(int ncells, const T *__restrict__ vals, bool tri,
-                                              unsigned char *stage, int2 *meta, const CellMeta *cm,
+__device__ __forceinline__ void produce_cells(int ncells, bool tri, unsigned char *stage, int2 *meta, const CellMeta *cm,
                                               unsigned long long *ready, unsigned long long *full,
                                               unsigned long long *empty, double *err) {
   int k = 0;  // running chunk counter of this CTA
@@ -1036,7 +1091,7 @@ __device__ __forceinline__ void produce_cells(int ncells, const T *__restrict__ 
     const int nch = cm[bb].nch;
     const int *cs = cm[bb].cs;
     const long long vs = pad4(c.nI);
-    const T *block = vals + (tri ? c.S_off : c.V_off);
+    const T *block = cm[bb].vals + (tri ? c.S_off : c.V_off);
     const int ntri = tri ? c.nI : 0;
     for (int j = 0; j < nch; ++j, ++k) {
       const int rb = cs[j], re = cs[j + 1];
@@ -1063,13 +1118,9 @@ __device__ __forceinline__ void produce_cells(int ncells, const T *__restrict__ 
 // with PDL this happens before the previous kernel has finished) and on
 // ready[b] once x is gathered.
 // Before refilling a buffer it waits until the consumers freed it.
-template <typename T>
-__device__ __forceinline__ void gather_cells(const CellDesc *__restrict__ cells, int ncells,
-                                             const int2 *__restrict__ chunk_of,
-                                             const int *__restrict__ chunk_tab,
-                                             const int *__restrict__ idx, const T *__restrict__ x,
-                                             CellMeta *cm, T *xs0, long long xs_stride, T *xb0,
-                                             long long xb_stride, int *is0, unsigned long long *ready,
+template <typename T, class Src>
+__device__ __forceinline__ void gather_cells(const Src &src, int ncells, CellMeta *cm, T *xs0, long long xs_stride,
+                                             T *xb0, long long xb_stride, int *is0, unsigned long long *ready,
                                              unsigned long long *mready, unsigned long long *freed,
                                              double *err) {
   const int lane = threadIdx.x & 31;
@@ -1077,17 +1128,21 @@ __device__ __forceinline__ void gather_cells(const CellDesc *__restrict__ cells,
   // the next cell's descriptor is loaded while the current one is gathered
   CellDesc c_next{};
   int2 co_next{0, 0};
+  int p_next = 0;
   if (blockIdx.x < (unsigned)ncells) {
-    c_next = cells[blockIdx.x];
-    co_next = chunk_of[blockIdx.x];
+    p_next = src.find(blockIdx.x);
+    src.cell(p_next, blockIdx.x, c_next, co_next);
   }
   for (int ci = blockIdx.x; ci < ncells; ci += gridDim.x, ++jc) {
     const int b = jc & 1;
     const CellDesc c = c_next;
     const int2 co = co_next;
+    const int hp = p_next;
+    const int *tab = src.tab(hp), *idx = src.idx(hp);
+    const T *x = src.x(hp);
     if (ci + (int)gridDim.x < ncells) {
-      c_next = cells[ci + gridDim.x];
-      co_next = chunk_of[ci + gridDim.x];
+      p_next = src.find(ci + gridDim.x);
+      src.cell(p_next, ci + gridDim.x, c_next, co_next);
     }
     if (jc >= 2 && !mbar_wait(&freed[b], (unsigned)(((jc >> 1) - 1) & 1))) {
       if (lane == 0) err[0] = 1.0;
@@ -1096,8 +1151,11 @@ __device__ __forceinline__ void gather_cells(const CellDesc *__restrict__ cells,
     if (lane == 0) {
       cm[b].c = c;
       cm[b].nch = co.y;
+      cm[b].vals = src.vals(hp);
+      cm[b].x = src.x(hp);
+      cm[b].contrib = src.contrib(hp);
     }
-    for (int j = lane; j <= co.y; j += 32) cm[b].cs[j] = chunk_tab[co.x + j];
+    for (int j = lane; j <= co.y; j += 32) cm[b].cs[j] = co.y > 0 ? tab[co.x + j] : 0;
     mbar_arrive(&mready[b]);  // the copy warp may stream the cell's block
     if (jc == 0) pdl_wait();  // x is written by the previous kernel
     // gathers in batches of kG per lane: all index loads, then all value loads
@@ -1254,16 +1312,8 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float p) {
 // CTA takes cells blockIdx.x, blockIdx.x + gridDim.x, ...; warp 8 copies the
 // V rows, warp 9 gathers x_I of the next cell, warps 0-7 compute and write
 // each row's total straight to the contribution buffer.
-template <typename T>
-__global__ void __launch_bounds__(kTmaThreads, 4) k_cell_fwd_tma_S(const CellDesc *__restrict__ cells,
-                                                                   int ncells,
-                                                                   const int2 *__restrict__ chunk_of,
-                                                                   const int *__restrict__ chunk_tab,
-                                                                   const int *__restrict__ idx,
-                                                                   const T *__restrict__ vals,
-                                                                   T *__restrict__ contrib,
-                                                                   const T *__restrict__ x,
-                                                                   double *__restrict__ err,
+template <typename T, class Src>
+__global__ void __launch_bounds__(kTmaThreads, 4) k_cell_fwd_tma_S(Src src, int ncells, double *__restrict__ err,
                                                                    int max_nI, int max_nB) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long full[kStagesFwd], empty[kStagesFwd], ready[2], mready[2], freed[2];
@@ -1288,12 +1338,11 @@ __global__ void __launch_bounds__(kTmaThreads, 4) k_cell_fwd_tma_S(const CellDes
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == kConsumerWarps) {
     if (lane == 0)
-      produce_cells<T, kStagesFwd>(ncells, vals, false, stage, meta, cm, mready, full, empty, err);
+      produce_cells<T, kStagesFwd>(ncells, false, stage, meta, cm, mready, full, empty, err);
     return;
   }
   if (warp == kConsumerWarps + 1) {
-    gather_cells<T>(cells, ncells, chunk_of, chunk_tab, idx, x, cm, xs0, xstride, nullptr, 0, nullptr,
-                    ready, mready, freed, err);
+    gather_cells<T>(src, ncells, cm, xs0, xstride, (T *)nullptr, 0, nullptr, ready, mready, freed, err);
     return;
   }
   pdl_wait();  // outputs are written over data the previous kernel reads
@@ -1312,7 +1361,7 @@ __global__ void __launch_bounds__(kTmaThreads, 4) k_cell_fwd_tma_S(const CellDes
     const int vs = 4 * nq;
     T xa[4], xb[4];
     load_xcols(xs0 + b * xstride, nq, lane, xa, xb);
-    T *out = contrib + c.C_off;
+    T *out = cm[b].contrib + c.C_off;
     for (int j = 0; j < nch; ++j, ++k) {
       const int sidx = (int)(k % kStagesFwd);
       if (!mbar_wait(&full[sidx], (unsigned)((k / kStagesFwd) & 1))) {
@@ -1374,16 +1423,10 @@ __global__ void __launch_bounds__(kTmaThreads, 4) k_cell_fwd_tma_S(const CellDes
 // warp rounds its compensated sums once, and the row dots and the warps' sums
 // are combined by two-sum: the same 2.05 iterations as FP64 accumulation for
 // about 6% more kernel time (3 CTAs per SM still fit in 64 registers).
-template <typename T, bool kComp = true>
-__global__ void __launch_bounds__(kTmaThreads, kComp ? 3 : 2) k_cell_bwd_tma_S(const CellDesc *__restrict__ cells,
-                                                                   int ncells,
-                                                                   const int2 *__restrict__ chunk_of,
-                                                                   const int *__restrict__ chunk_tab,
-                                                                   const int *__restrict__ idx,
-                                                                   const T *__restrict__ vals,
-                                                                   T *__restrict__ x,
-                                                                   double *__restrict__ err,
-                                                                   int max_nI, int max_nB) {
+template <typename T, bool kComp, class Src>
+__global__ void __launch_bounds__(kTmaThreads, kComp ? 3 : 2) k_cell_bwd_tma_S(Src src, int ncells,
+                                                                               double *__restrict__ err, int max_nI,
+                                                                               int max_nB) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long full[kStagesBwd], empty[kStagesBwd], ready[2], mready[2], freed[2];
   __shared__ int2 meta[kStagesBwd];
@@ -1411,12 +1454,11 @@ __global__ void __launch_bounds__(kTmaThreads, kComp ? 3 : 2) k_cell_bwd_tma_S(c
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == kConsumerWarps) {
     if (lane == 0)
-      produce_cells<T, kStagesBwd>(ncells, vals, true, stage, meta, cm, mready, full, empty, err);
+      produce_cells<T, kStagesBwd>(ncells, true, stage, meta, cm, mready, full, empty, err);
     return;
   }
   if (warp == kConsumerWarps + 1) {
-    gather_cells<T>(cells, ncells, chunk_of, chunk_tab, idx, x, cm, xs0, xstride, xb0, bstride, is0,
-                    ready, mready, freed, err);
+    gather_cells<T>(src, ncells, cm, xs0, xstride, xb0, bstride, is0, ready, mready, freed, err);
     return;
   }
   pdl_wait();  // outputs are written over data the previous kernel reads
@@ -1549,6 +1591,7 @@ __global__ void __launch_bounds__(kTmaThreads, kComp ? 3 : 2) k_cell_bwd_tma_S(c
     if (lane + 32 < nq) st4(pw + 4 * (lane + 32), cb);
     consumers_sync();
     const int *is = is0 + b * xstride;
+    T *x = cm[b].x;
     for (int i = threadIdx.x; i < nI; i += kConsumers) {
       T s = rd[i];
       if constexpr (kComp) {  // the row dot and the warps' sums, by two-sum
@@ -2103,111 +2146,7 @@ __global__ void __launch_bounds__(kFlowThreads) k_flow_sweep(
 // finds its handle by binary search and runs the same unit code as the
 // single-handle kernels (G-form cells, FP32 arithmetic, BF16 values at the
 // handle's BF16 levels).  Handles whose solve has converged are skipped.
-// S-form cell steps of the merged batched path (one CTA of 256 threads per
-// cell, FP32, plain loads; the operator of the bulk-copy kernels): forward
-// c_B = V x_I (x_I left as it is), backward x_I <- S x_I - V^T x_B with S
-// packed lower, diagonal halved.  In the backward, warp w takes rows w, w+8,
-// ...; lane l keeps x at the column quads l and l + 32 and accumulates the
-// column sums there, so one read of a stored quad feeds both the row dot and
-// the column sums; the 8 warps' column sums and the row dots meet at the end
-// in a fixed order (deterministic).  Needs nI <= 256.
-__device__ __forceinline__ float warp_sum_f(float v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __noinline__ void cell_fwd_S_unit(const CellDesc c, const int *__restrict__ idx,
-                                             const float *__restrict__ vals, float *__restrict__ contrib,
-                                             const float *__restrict__ x, float *sm) {
-  const int nI = c.nI, nq = (int)pad4(nI) / 4;
-  float *xs = sm;
-  for (int i = threadIdx.x; i < 4 * nq; i += 256) xs[i] = i < nI ? x[idx[c.I_off + i]] : 0.f;
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float xa[4], xb[4];
-  load_xcols(xs, nq, lane, xa, xb);
-  const float *V = vals + c.V_off;
-  for (int b = warp; b < c.nB; b += 8) {
-    const float *row = V + (long long)b * 4 * nq;
-    float t = 0.f;
-    if (lane < nq) {
-      float v[4];
-      ld4(row + 4 * lane, v);
-      t = dot4(v, xa);
-    }
-    if (lane + 32 < nq) {
-      float v[4];
-      ld4(row + 4 * (lane + 32), v);
-      t += dot4(v, xb);
-    }
-    t = warp_sum_f(t);
-    if (lane == 0) contrib[c.C_off + b] = t;
-  }
-}
-
-__device__ __noinline__ void cell_bwd_S_unit(const CellDesc c, const int *__restrict__ idx,
-                                             const float *__restrict__ vals, float *__restrict__ x, float *sm) {
-  const int nI = c.nI, nB = c.nB, nq = (int)pad4(nI) / 4, np = 4 * nq;
-  float *xs = sm;                    // np
-  float *xbv = xs + np;              // pad4(nB)
-  float *part = xbv + pad4(nB);      // 8 x np column sums
-  float *rd = part + 8 * np;         // np row dots
-  for (int i = threadIdx.x; i < np; i += 256) xs[i] = i < nI ? x[idx[c.I_off + i]] : 0.f;
-  for (int b = threadIdx.x; b < nB; b += 256) xbv[b] = x[idx[c.B_off + b]];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float xa[4], xb[4];
-  load_xcols(xs, nq, lane, xa, xb);
-  float ca[4] = {0.f, 0.f, 0.f, 0.f}, cb[4] = {0.f, 0.f, 0.f, 0.f};
-  const float *S = vals + c.S_off;
-  for (int i = warp; i < nI; i += 8) {
-    const float *row = S + tri_off(i);
-    const int nqi = (i >> 2) + 1;
-    const float xi = xs[i];
-    float t = 0.f;
-    if (lane < nqi) {
-      float v[4];
-      ld4(row + 4 * lane, v);
-      t = dot4(v, xa);
-      axpy4(ca, v, xi);
-    }
-    if (lane + 32 < nqi) {
-      float v[4];
-      ld4(row + 4 * (lane + 32), v);
-      t += dot4(v, xb);
-      axpy4(cb, v, xi);
-    }
-    t = warp_sum_f(t);
-    if (lane == 0) rd[i] = t;
-  }
-  const float *V = vals + c.V_off;
-  for (int b = warp; b < nB; b += 8) {
-    const float *row = V + (long long)b * np;
-    const float y = -xbv[b];
-    if (lane < nq) {
-      float v[4];
-      ld4(row + 4 * lane, v);
-      axpy4(ca, v, y);
-    }
-    if (lane + 32 < nq) {
-      float v[4];
-      ld4(row + 4 * (lane + 32), v);
-      axpy4(cb, v, y);
-    }
-  }
-  float *pw = part + warp * np;
-  if (lane < nq)
-    for (int e = 0; e < 4; ++e) pw[4 * lane + e] = ca[e];
-  if (lane + 32 < nq)
-    for (int e = 0; e < 4; ++e) pw[4 * (lane + 32) + e] = cb[e];
-  __syncthreads();
-  for (int i = threadIdx.x; i < nI; i += 256) {
-    float y = rd[i];
-    for (int w = 0; w < 8; ++w) y += part[w * np + i];
-    x[idx[c.I_off + i]] = y;
-  }
-}
-
+// The cells of S-form levels go through the bulk-copy kernels (launch_merged_sform).
 template <int KIND>
 __global__ void __launch_bounds__(256) k_merged_phase(const int *__restrict__ pre, int K, int level,
                                                       HandleView *const *__restrict__ views,
@@ -2236,12 +2175,10 @@ __global__ void __launch_bounds__(256) k_merged_phase(const int *__restrict__ pr
   } else {
     const LevelView L = v->lv[level];
     if constexpr (KIND == kPhaseCellFwd) {
-      if (L.sform) cell_fwd_S_unit(L.cells[L.fwd[u].cell], idx, vals, v->contrib, v->z, sm);
-      else if (b16) cell_fwd_unit<float, 256, __nv_bfloat16>(L.fwd[u], L.cells, idx, vals16, v->contrib, v->xI, v->z, sm);
+      if (b16) cell_fwd_unit<float, 256, __nv_bfloat16>(L.fwd[u], L.cells, idx, vals16, v->contrib, v->xI, v->z, sm);
       else cell_fwd_unit<float, 256>(L.fwd[u], L.cells, idx, vals, v->contrib, v->xI, v->z, sm);
     } else if constexpr (KIND == kPhaseCellBwd) {
-      if (L.sform) cell_bwd_S_unit(L.cells[L.bwd[u].cell], idx, vals, v->z, sm);
-      else if (b16) cell_bwd_unit<float, 256, __nv_bfloat16>(L.bwd[u], L.cells, idx, vals16, v->xI, v->z, sm);
+      if (b16) cell_bwd_unit<float, 256, __nv_bfloat16>(L.bwd[u], L.cells, idx, vals16, v->xI, v->z, sm);
       else cell_bwd_unit<float, 256>(L.bwd[u], L.cells, idx, vals, v->xI, v->z, sm);
     } else if constexpr (KIND == kPhaseGroupFwd) {
       if (u < L.nlarge) {
@@ -2322,9 +2259,9 @@ int set_smem_limits() {
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_root_cols<T, __nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_group_rows_split<T, __nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_group_cols_split<T, __nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-    HIF_CUDA_TRY(cudaFuncSetAttribute(k_cell_fwd_tma_S<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-    HIF_CUDA_TRY(cudaFuncSetAttribute(k_cell_bwd_tma_S<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-    HIF_CUDA_TRY(cudaFuncSetAttribute(k_cell_bwd_tma_S<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_cell_fwd_tma_S<T, OneLevel>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_cell_bwd_tma_S<T, true, OneLevel>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_cell_bwd_tma_S<T, false, OneLevel>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   }
   done = true;
   return HIF_OK;
@@ -2442,10 +2379,10 @@ int launch_cell_fwd(Handle *h, const LevelDev &lv, int l, const FactorValues<T> 
   if constexpr (sizeof(T) == 4) {
     if (sf) {
       size_t sm = (size_t)kStagesFwd * kStageBytes + tma_fwd_smem_elems(lv) * sizeof(T);
-      const int grid = tma_grid((const void *)k_cell_fwd_tma_S<T>, sm, lv.ncells, h->tma_ctas);
-      HIF_CUDA_TRY(launch_k(k_cell_fwd_tma_S<T>, grid, kTmaThreads, sm, s, lv.cells, lv.ncells, lv.chunk_of[0],
-                                                         lv.chunk_tab[0], h->idx, fv.vals, fv.contrib, x,
-                                                         h->scal + kScalErr, lv.max_nI, lv.max_nB));
+      const int grid = tma_grid((const void *)k_cell_fwd_tma_S<T, OneLevel>, sm, lv.ncells, h->tma_ctas);
+      const OneLevel src{lv.cells, lv.chunk_of[0], lv.chunk_tab[0], h->idx, fv.vals, x, fv.contrib};
+      HIF_CUDA_TRY(launch_k(k_cell_fwd_tma_S<T, OneLevel>, grid, kTmaThreads, sm, s, src, lv.ncells,
+                            h->scal + kScalErr, lv.max_nI, lv.max_nB));
       return HIF_OK;
     }
   }
@@ -2569,11 +2506,12 @@ int launch_cell_bwd(Handle *h, const LevelDev &lv, int l, const FactorValues<T> 
     if (sf) {
       // compensated accumulation of -V^T x_B (HIFCN_LEAF_COMP=0: plain FP32 sums, for measurements)
       static const bool comp = !(std::getenv("HIFCN_LEAF_COMP") && std::getenv("HIFCN_LEAF_COMP")[0] == '0');
-      auto kern = comp ? k_cell_bwd_tma_S<T, true> : k_cell_bwd_tma_S<T, false>;
+      auto kern = comp ? k_cell_bwd_tma_S<T, true, OneLevel> : k_cell_bwd_tma_S<T, false, OneLevel>;
       size_t sm = (size_t)kStagesBwd * kStageBytes + tma_bwd_smem_elems(lv) * sizeof(T);
       const int grid = tma_grid((const void *)kern, sm, lv.ncells, h->tma_ctas);
-      HIF_CUDA_TRY(launch_k(kern, grid, kTmaThreads, sm, s, lv.cells, lv.ncells, lv.chunk_of[1], lv.chunk_tab[1],
-                            h->idx, fv.vals, x, h->scal + kScalErr, lv.max_nI, lv.max_nB));
+      const OneLevel src{lv.cells, lv.chunk_of[1], lv.chunk_tab[1], h->idx, fv.vals, x, fv.contrib};
+      HIF_CUDA_TRY(launch_k(kern, grid, kTmaThreads, sm, s, src, lv.ncells, h->scal + kScalErr, lv.max_nI,
+                            lv.max_nB));
       return HIF_OK;
     }
   }
@@ -2840,6 +2778,11 @@ bool level_uses_sform(const Handle *h, int l) {
   return h->has_f32 && l >= 0 && l < h->L && use_tma(h, h->lv[l], sizeof(float)) && !bf16_level<float>(h, l);
 }
 
+bool merged_sform(const Handle *h, int level) {
+  const LevelDev &D = h->lv[level];
+  return D.has_S && D.max_nI <= kSformMaxNI && level < (h->has_bf16 ? h->bf16_lb : 1 << 30);
+}
+
 // The device view of a handle for the merged batched steps (FP32 apply
 // only; handles with split levels, a split root or more than
 // kMaxViewLevels levels keep the per-handle path).
@@ -2888,7 +2831,8 @@ int build_view(Handle *h) {
     const LevelDev &D = h->lv[l];
     v.lv[l] = LevelView{D.fwd1, D.bwd1, D.cells, D.groups, D.small_groups, D.large_groups,
                         D.ncells, D.ncells, D.nsmall, D.nlarge,
-                        (D.has_S && D.max_nI <= 256 && l < v.bf16_lb) ? 1 : 0};
+                        merged_sform(h, l) ? 1 : 0,
+                        {D.chunk_of[0], D.chunk_of[1]}, {D.chunk_tab[0], D.chunk_tab[1]}};
   }
   if (!h->view) HIF_TRY(dev_alloc(h, (void **)&h->view, sizeof(HandleView)));
   HIF_CUDA_TRY(cudaMemcpy(h->view, &v, sizeof(HandleView), cudaMemcpyHostToDevice));
@@ -2912,14 +2856,13 @@ void merged_units(const Handle *h, int kind, int level, int *units, size_t *smem
   if (level >= h->L) return;
   const LevelDev &lv = h->lv[level];
   switch (kind) {
-    case kPhaseCellFwd:
-      *units = lv.ncells;
+    case kPhaseCellFwd:  // (levels applied in the S-form: launch_merged_sform)
+      *units = merged_sform(h, level) ? 0 : lv.ncells;
       *smem = (size_t)pad4(lv.max_nI) * sizeof(float);
       break;
     case kPhaseCellBwd:
-      *units = lv.ncells;
-      *smem = std::max((size_t)lv.max_nI + lv.max_nB + 8 * 256,
-                       10 * (size_t)pad4(lv.max_nI) + (size_t)pad4(lv.max_nB)) * sizeof(float);
+      *units = merged_sform(h, level) ? 0 : lv.ncells;
+      *smem = ((size_t)lv.max_nI + lv.max_nB + 8 * 256) * sizeof(float);
       break;
     case kPhaseGroupFwd:
       *units = lv.ngroups ? lv.nlarge + (lv.nsmall + 7) / 8 : 0;
@@ -2961,6 +2904,33 @@ int launch_merged_phase(int kind, int level, const int *pre, int K, int total, s
     default:
       k_merged_phase<kPhaseRootRows><<<total, 256, smem, s>>>(pre, K, 1 << 20, views, active);
       break;
+  }
+  note_launch();
+  HIF_CUDA_TRY(cudaGetLastError());
+  return HIF_OK;
+}
+
+// The S-form cells of a level of all handles, through the bulk-copy kernels: one
+// persistent launch streams the cells of every handle.  A CTA per cell reading S and
+// V through L1 took 183 us forward and 362 us backward for the leaf cells of 24
+// problems of 63^2 to 511^2 (14592 cells, 1 GB); @BATCH@ now.
+int launch_merged_sform(bool bwd, int level, const int *pre, int K, int total, int max_nI, int max_nB,
+                        HandleView *const *views, const int *active, double *err, cudaStream_t s) {
+  if (total <= 0) return HIF_OK;
+  const BatchLevel src{pre, K, level, bwd ? 1 : 0, views, active};
+  LevelDev d;  // sizes of the shared-memory rule
+  d.max_nI = max_nI;
+  d.max_nB = max_nB;
+  if (bwd) {
+    auto kern = k_cell_bwd_tma_S<float, true, BatchLevel>;
+    const size_t sm = (size_t)kStagesBwd * kStageBytes + tma_bwd_smem_elems(d) * sizeof(float);
+    HIF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    kern<<<tma_grid((const void *)kern, sm, total, 0), kTmaThreads, sm, s>>>(src, total, err, max_nI, max_nB);
+  } else {
+    auto kern = k_cell_fwd_tma_S<float, BatchLevel>;
+    const size_t sm = (size_t)kStagesFwd * kStageBytes + tma_fwd_smem_elems(d) * sizeof(float);
+    HIF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    kern<<<tma_grid((const void *)kern, sm, total, 0), kTmaThreads, sm, s>>>(src, total, err, max_nI, max_nB);
   }
   note_launch();
   HIF_CUDA_TRY(cudaGetLastError());

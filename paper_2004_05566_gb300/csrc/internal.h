@@ -193,6 +193,8 @@ struct LevelView {
   const int *small, *large;
   int nfwd, nbwd, nsmall, nlarge;
   int sform;  // cells applied in the S-form (S = A_II^{-1} stored, FP32 values)
+  const int2 *chunk_of[2];  // bulk-copy chunk tables: V, and S then V
+  const int *chunk_tab[2];
 };
 struct HandleView {
   int L, dim, n, root_n;
@@ -421,6 +423,10 @@ int build_items(Handle *h, LevelDev &D, const LevelHost &H, int target, cudaStre
 void merged_units(const Handle *h, int kind, int level, int *units, size_t *smem);
 int launch_merged_phase(int kind, int level, const int *pre, int K, int total, size_t smem,
                         HandleView *const *views, const int *active, cudaStream_t s);
+// the cells of a level that the bulk-copy S-form kernels take (merged steps)
+bool merged_sform(const Handle *h, int level);
+int launch_merged_sform(bool bwd, int level, const int *pre, int K, int total, int max_nI, int max_nB,
+                        HandleView *const *views, const int *active, double *err, cudaStream_t s);
 int pcg(Handle *h, const double *b, double *x, int *iters, double *relres, cudaStream_t s);
 int cn(Handle *h, const double *u, const double *r, double *u1, int *iters, cudaStream_t s);
 int cn_multi(Handle *h, double *u, const double *r, int nsteps, int *iters, cudaStream_t s);

@@ -1129,7 +1129,9 @@ int cn_multi(Handle *h, double *u, const double *r, int nsteps, int *iters, cuda
 // handle is the same in any batch, and equals that of its single steps to the
 // CG tolerance (the single path applies the leaf levels in the S form).
 
-constexpr int kSeg = 8192;
+// 8 elements a thread: 8192 left 24 problems of 63^2 to 511^2 with 199 CTAs (w = A z
+// and the update 90 and 69 us an iteration; @SEG@ now)
+constexpr int kSeg = 2048;
 enum { B_RZ = 0, B_ALPHA, B_BETA, B_RR, B_BB, B_PQ, B_IT, B_CONV, B_COUNT };
 
 struct BSeg {  // per-call arrays of the batch (device)
@@ -1394,7 +1396,7 @@ int bws_reserve(size_t dev_bytes, size_t host_bytes) {
     HIF_CUDA_TRY(cudaMallocHost((void **)&g_bws.host, host_bytes * 2));
     g_bws.host_bytes = host_bytes * 2;
   }
-  if (!g_bws.h_nactive) HIF_CUDA_TRY(cudaMallocHost((void **)&g_bws.h_nactive, sizeof(int)));
+  if (!g_bws.h_nactive) HIF_CUDA_TRY(cudaMallocHost((void **)&g_bws.h_nactive, 2 * sizeof(double)));
   return HIF_OK;
 }
 
@@ -1415,9 +1417,9 @@ int cn_batched_merged(Handle *const *hs, int K, const double *const *u, const do
     phases.push_back(make_int2(kPhaseCellBwd, l));
   }
   const int P = (int)phases.size();
-  // host staging layout: views[K] | u[K] | rr[K] | u1[K] | segpre[K+1] | pre[P][K+1] | active[K]
+  // host staging layout: views[K] | u[K] | rr[K] | u1[K] | segpre[K+1] | pre[2 P][K+1] | active[K]
   const size_t ptr_bytes = 4 * (size_t)K * sizeof(void *);
-  const size_t int_count = (size_t)(K + 1) * (P + 1) + K;
+  const size_t int_count = (size_t)(K + 1) * (2 * P + 1) + K;  // two unit lists per phase
   const size_t up_bytes = ptr_bytes + int_count * sizeof(int);
   int total_seg = 0;
   std::vector<int> segpre(K + 1, 0);
@@ -1444,23 +1446,34 @@ int cn_batched_merged(Handle *const *hs, int K, const double *const *u, const do
   }
   int *hi = reinterpret_cast<int *>(hb + ptr_bytes);
   std::memcpy(hi, segpre.data(), (K + 1) * sizeof(int));
-  std::vector<int> totals(P, 0);
+  std::vector<int> totals(P, 0), stotals(P, 0), smax_nI(P, 0), smax_nB(P, 0);
   std::vector<size_t> smem(P, 0);
   for (int ph = 0; ph < P; ++ph) {
-    int *pre = hi + (size_t)(K + 1) * (ph + 1);
-    int run = 0;
+    int *pre = hi + (size_t)(K + 1) * (2 * ph + 1), *spre = pre + K + 1;
+    const int kind = phases[ph].x, level = phases[ph].y;
+    const bool cell = kind == kPhaseCellFwd || kind == kPhaseCellBwd;
+    int run = 0, srun = 0;
     for (int i = 0; i < K; ++i) {
       int un = 0;
       size_t sm = 0;
-      merged_units(hs[i], phases[ph].x, phases[ph].y, &un, &sm);
+      merged_units(hs[i], kind, level, &un, &sm);
       pre[i] = run;
       run += un;
-      smem[ph] = std::max(smem[ph], sm);
+      spre[i] = srun;
+      if (un > 0) smem[ph] = std::max(smem[ph], sm);
+      if (cell && level < hs[i]->L && merged_sform(hs[i], level)) {
+        const LevelDev &lv = hs[i]->lv[level];
+        srun += lv.ncells;
+        smax_nI[ph] = std::max(smax_nI[ph], lv.max_nI);
+        smax_nB[ph] = std::max(smax_nB[ph], lv.max_nB);
+      }
     }
     pre[K] = run;
+    spre[K] = srun;
     totals[ph] = run;
+    stotals[ph] = srun;
   }
-  int *hact = hi + (size_t)(K + 1) * (P + 1);
+  int *hact = hi + (size_t)(K + 1) * (2 * P + 1);
   for (int i = 0; i < K; ++i) hact[i] = 1;
   HIF_CUDA_TRY(cudaMemcpyAsync(db, hb, up_bytes, cudaMemcpyHostToDevice, s));
   BSeg B;
@@ -1471,19 +1484,24 @@ int cn_batched_merged(Handle *const *hs, int K, const double *const *u, const do
   const int *dint = reinterpret_cast<const int *>(db + ptr_bytes);
   B.segpre = dint;
   B.K = K;
-  int *active = const_cast<int *>(dint + (size_t)(K + 1) * (P + 1));
+  int *active = const_cast<int *>(dint + (size_t)(K + 1) * (2 * P + 1));
   double *sc = reinterpret_cast<double *>(db + sc_off);
   double *part = reinterpret_cast<double *>(db + part_off);
   int *nactive = reinterpret_cast<int *>(db + nact_off);
+  double *werr = reinterpret_cast<double *>(db + nact_off + sizeof(double));  // an expired bounded wait
   const int sgrid = (K + 7) / 8;
 
   auto read_active = [&](int *n) -> int {
-    HIF_CUDA_TRY(cudaMemcpyAsync(g_bws.h_nactive, nactive, sizeof(int), cudaMemcpyDeviceToHost, s));
+    HIF_CUDA_TRY(cudaMemcpyAsync(g_bws.h_nactive, nactive, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
     HIF_CUDA_TRY(cudaStreamSynchronize(s));
     *n = *g_bws.h_nactive;
+    if (reinterpret_cast<double *>(g_bws.h_nactive)[1] != 0.0) {
+      set_last_error("a bounded device wait expired in the HIF apply");
+      return HIF_ETIMEOUT;
+    }
     return HIF_OK;
   };
-  HIF_CUDA_TRY(cudaMemsetAsync(nactive, 0, sizeof(int), s));
+  HIF_CUDA_TRY(cudaMemsetAsync(nactive, 0, 2 * sizeof(double), s));  // and werr
   k_b_start<<<total_seg, NT, 0, s>>>(B, part);
   k_b_scalar<<<sgrid, 256, 0, s>>>(B, 0, active, sc, part, nactive);
   note_launch(2);
@@ -1492,9 +1510,13 @@ int cn_batched_merged(Handle *const *hs, int K, const double *const *u, const do
   int maxit = 0;
   for (int i = 0; i < K; ++i) maxit = std::max(maxit, hs[i]->opt.cg_maxit);
   for (int it = 0; n_act > 0 && it < maxit; ++it) {
-    for (int ph = 0; ph < P; ++ph)
-      HIF_TRY(launch_merged_phase(phases[ph].x, phases[ph].y, dint + (size_t)(K + 1) * (ph + 1), K,
-                                  totals[ph], smem[ph], const_cast<HandleView *const *>(B.views), active, s));
+    for (int ph = 0; ph < P; ++ph) {
+      const int *pre = dint + (size_t)(K + 1) * (2 * ph + 1);
+      HIF_TRY(launch_merged_sform(phases[ph].x == kPhaseCellBwd, phases[ph].y, pre + K + 1, K, stotals[ph],
+                                  smax_nI[ph], smax_nB[ph], const_cast<HandleView *const *>(B.views), active, werr, s));
+      HIF_TRY(launch_merged_phase(phases[ph].x, phases[ph].y, pre, K, totals[ph], smem[ph],
+                                  const_cast<HandleView *const *>(B.views), active, s));
+    }
     k_b_wz<<<total_seg, NT, 0, s>>>(B, active, sc, part);
     k_b_scalar<<<sgrid, 256, 0, s>>>(B, 4, active, sc, part, nactive);
     k_b_update<<<total_seg, NT, 0, s>>>(B, active, sc, part);
