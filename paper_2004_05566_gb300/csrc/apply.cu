@@ -1674,12 +1674,10 @@ __global__ void __launch_bounds__(kRootThreads) k_root(int nr, const int *__rest
 // full symmetric matrix (rows of ld floats, zero padding): one pass of row
 // dots instead of the two dependent triangular passes of root_unit, whose
 // column pass is a long serial chain per thread for a root of ~100 DOFs.
-__global__ void __launch_bounds__(kRootThreads) k_root_dense(int nr, const int *__restrict__ ridx,
-                                                             const float *__restrict__ S, int ld,
-                                                             float *__restrict__ x) {
+__device__ __forceinline__ void root_dense_unit(int nr, const int *__restrict__ ridx, const float *__restrict__ S,
+                                                int ld, float *__restrict__ x, float *xs) {
+  if (threadIdx.x == 0) prefetch_block_l2(S, (long long)nr * ld);
   pdl_enter();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float *xs = reinterpret_cast<float *>(smem_raw);
   for (int i = threadIdx.x; i < ld; i += kRootThreads) xs[i] = i < nr ? x[ridx[i]] : 0.f;
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1701,6 +1699,13 @@ __global__ void __launch_bounds__(kRootThreads) k_root_dense(int nr, const int *
         if (r0 + u < nr) x[ridx[r0 + u]] = acc[u];
     }
   }
+}
+
+__global__ void __launch_bounds__(kRootThreads) k_root_dense(int nr, const int *__restrict__ ridx,
+                                                             const float *__restrict__ S, int ld,
+                                                             float *__restrict__ x) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  root_dense_unit(nr, ridx, S, ld, x, reinterpret_cast<float *>(smem_raw));
 }
 
 // S_r = G_r^T G_r from the packed FP32 G_r, accumulated in FP64 and rounded
@@ -2147,6 +2152,53 @@ __global__ void __launch_bounds__(kFlowThreads) k_flow_sweep(
 // single-handle kernels (G-form cells, FP32 arithmetic, BF16 values at the
 // handle's BF16 levels).  Handles whose solve has converged are skipped.
 // The cells of S-form levels go through the bulk-copy kernels (launch_merged_sform).
+// eight entities of at most 32 DOFs of handle v, one a warp
+template <bool kFwd>
+__device__ __forceinline__ void merged_small(const HandleView &v, int level, bool b16, int u, float *sm) {
+  const LevelView &L = v.lv[level];
+  const int warp = threadIdx.x >> 5, t = u * kSmallWarps + warp;
+  if (t >= L.nsmall) {
+    pdl_enter();
+    return;
+  }
+  const GroupDesc g = L.groups[L.small[t]];
+  float *xs = sm + 32 * warp;
+  const __nv_bfloat16 *v16 = static_cast<const __nv_bfloat16 *>(v.vals16);
+  if constexpr (kFwd) {
+    if (b16)
+      group_fwd_small_warp<float, __nv_bfloat16, true, true>(g, v.idx, v.cptr, v.cslot, v16, v.contrib, v.z, v.z, xs);
+    else group_fwd_small_warp<float, float, true, true>(g, v.idx, v.cptr, v.cslot, v.vals, v.contrib, v.z, v.z, xs);
+  } else {
+    // (columns neither preloaded nor prefetched: both cost the leaf levels more, in
+    // registers or in prefetch instructions, than they hide: 37 and 40 us against 32)
+    pdl_enter();
+    if (b16) group_bwd_small_warp<float, __nv_bfloat16>(g, v.idx, v16, v.z, v.z, xs);
+    else group_bwd_small_warp<float>(g, v.idx, v.vals, v.z, v.z, xs);
+  }
+}
+
+// A group phase in which no handle has a large entity (the leaf levels): the same
+// without the registers of the large entities' units, which left 3 CTAs an SM
+// (24 problems, 42 k leaf entities: forward 47 us, 34 now).
+template <bool kFwd>
+__global__ void __launch_bounds__(256) k_merged_small(const int *__restrict__ pre, int K, int level,
+                                                      HandleView *const *__restrict__ views,
+                                                      const int *__restrict__ active) {
+  __shared__ float sm[32 * kSmallWarps];
+  int lo = 0, hi = K;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (pre[mid] <= (int)blockIdx.x) lo = mid;
+    else hi = mid;
+  }
+  if (!active[lo]) {
+    pdl_enter();
+    return;
+  }
+  const HandleView *v = views[lo];
+  merged_small<kFwd>(*v, level, level >= v->bf16_lb, blockIdx.x - pre[lo], sm);
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(256) k_merged_phase(const int *__restrict__ pre, int K, int level,
                                                       HandleView *const *__restrict__ views,
@@ -2160,7 +2212,10 @@ __global__ void __launch_bounds__(256) k_merged_phase(const int *__restrict__ pr
     else hi = mid;
   }
   const int p = lo;
-  if (!active[p]) return;
+  if (!active[p]) {  // (written before the first launch of the iteration, which is no dependent one)
+    pdl_enter();
+    return;
+  }
   const int u = blockIdx.x - pre[p];
   const HandleView *v = views[p];
   const bool b16 = level >= v->bf16_lb;
@@ -2169,46 +2224,37 @@ __global__ void __launch_bounds__(256) k_merged_phase(const int *__restrict__ pr
   const int *idx = v->idx;
   if constexpr (KIND == kPhaseRootRows) {  // the whole root of handle p
     const int nr = v->root_n;
+    if (v->root_S) {
+      root_dense_unit(nr, v->ridx, v->root_S, v->root_S_ld, v->z, sm);
+      return;
+    }
+    pdl_enter();
     if (b16) root_unit<float, 256, __nv_bfloat16>(nr, v->ridx, vals16 + v->root_G_off, v->z, sm);
     else root_unit<float, 256>(nr, v->ridx, vals + v->root_G_off, v->z, sm);
     return;
   } else {
     const LevelView L = v->lv[level];
     if constexpr (KIND == kPhaseCellFwd) {
-      if (b16) cell_fwd_unit<float, 256, __nv_bfloat16>(L.fwd[u], L.cells, idx, vals16, v->contrib, v->xI, v->z, sm);
-      else cell_fwd_unit<float, 256>(L.fwd[u], L.cells, idx, vals, v->contrib, v->xI, v->z, sm);
+      if (b16) cell_fwd_unit<float, 256, __nv_bfloat16, true>(L.fwd[u], L.cells, idx, vals16, v->contrib, v->xI, v->z, sm);
+      else cell_fwd_unit<float, 256, float, true>(L.fwd[u], L.cells, idx, vals, v->contrib, v->xI, v->z, sm);
     } else if constexpr (KIND == kPhaseCellBwd) {
-      if (b16) cell_bwd_unit<float, 256, __nv_bfloat16>(L.bwd[u], L.cells, idx, vals16, v->xI, v->z, sm);
-      else cell_bwd_unit<float, 256>(L.bwd[u], L.cells, idx, vals, v->xI, v->z, sm);
+      if (b16) cell_bwd_unit<float, 256, __nv_bfloat16, true>(L.bwd[u], L.cells, idx, vals16, v->xI, v->z, sm);
+      else cell_bwd_unit<float, 256, float, true>(L.bwd[u], L.cells, idx, vals, v->xI, v->z, sm);
     } else if constexpr (KIND == kPhaseGroupFwd) {
       if (u < L.nlarge) {
         const GroupDesc g = L.groups[L.large[u]];
-        if (b16) group_fwd_unit<float, 256, __nv_bfloat16>(g, idx, v->cptr, v->cslot, vals16, v->contrib, v->z, v->z, sm);
-        else group_fwd_unit<float, 256>(g, idx, v->cptr, v->cslot, vals, v->contrib, v->z, v->z, sm);
+        if (b16) group_fwd_unit<float, 256, __nv_bfloat16, true>(g, idx, v->cptr, v->cslot, vals16, v->contrib, v->z, v->z, sm);
+        else group_fwd_unit<float, 256, float, true>(g, idx, v->cptr, v->cslot, vals, v->contrib, v->z, v->z, sm);
       } else {
-        const int warp = threadIdx.x >> 5;
-        const int t = (u - L.nlarge) * 8 + warp;
-        if (t < L.nsmall) {
-          const GroupDesc g = L.groups[L.small[t]];
-          if (b16)
-            group_fwd_small_warp<float, __nv_bfloat16>(g, idx, v->cptr, v->cslot, vals16, v->contrib, v->z, v->z,
-                                                       sm + 32 * warp);
-          else group_fwd_small_warp<float>(g, idx, v->cptr, v->cslot, vals, v->contrib, v->z, v->z, sm + 32 * warp);
-        }
+        merged_small<true>(*v, level, b16, u - L.nlarge, sm);
       }
     } else {  // kPhaseGroupBwd
       if (u < L.nlarge) {
         const GroupDesc g = L.groups[L.large[u]];
-        if (b16) group_bwd_unit<float, 256, __nv_bfloat16>(g, idx, vals16, v->z, v->z, sm);
-        else group_bwd_unit<float, 256>(g, idx, vals, v->z, v->z, sm);
+        if (b16) group_bwd_unit<float, 256, __nv_bfloat16, true>(g, idx, vals16, v->z, v->z, sm);
+        else group_bwd_unit<float, 256, float, true>(g, idx, vals, v->z, v->z, sm);
       } else {
-        const int warp = threadIdx.x >> 5;
-        const int t = (u - L.nlarge) * 8 + warp;
-        if (t < L.nsmall) {
-          const GroupDesc g = L.groups[L.small[t]];
-          if (b16) group_bwd_small_warp<float, __nv_bfloat16>(g, idx, vals16, v->z, v->z, sm + 32 * warp);
-          else group_bwd_small_warp<float>(g, idx, vals, v->z, v->z, sm + 32 * warp);
-        }
+        merged_small<false>(*v, level, b16, u - L.nlarge, sm);
       }
     }
   }
@@ -2834,6 +2880,8 @@ int build_view(Handle *h) {
                         merged_sform(h, l) ? 1 : 0,
                         {D.chunk_of[0], D.chunk_of[1]}, {D.chunk_tab[0], D.chunk_tab[1]}};
   }
+  v.root_S = h->root_S;
+  v.root_S_ld = h->root_S_ld;
   if (!h->view) HIF_TRY(dev_alloc(h, (void **)&h->view, sizeof(HandleView)));
   HIF_CUDA_TRY(cudaMemcpy(h->view, &v, sizeof(HandleView), cudaMemcpyHostToDevice));
   h->view_ok = true;
@@ -2875,7 +2923,16 @@ void merged_units(const Handle *h, int kind, int level, int *units, size_t *smem
   }
 }
 
-int launch_merged_phase(int kind, int level, const int *pre, int K, int total, size_t smem,
+// dep: the launch may start its prologue while the launch before it runs
+template <typename... KArgs, typename... Args>
+cudaError_t launch_merged(bool dep, void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
+                          Args &&...args) {
+  if (dep) return launch_k(kernel, grid, block, smem, s, std::forward<Args>(args)...);
+  kernel<<<grid, block, smem, s>>>(std::forward<Args>(args)...);
+  return cudaGetLastError();
+}
+
+int launch_merged_phase(int kind, int level, const int *pre, int K, int total, size_t smem, bool small_only, bool dep,
                         HandleView *const *views, const int *active, cudaStream_t s) {
   if (total <= 0) return HIF_OK;
   static bool attr = false;
@@ -2888,33 +2945,28 @@ int launch_merged_phase(int kind, int level, const int *pre, int K, int total, s
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_merged_phase<kPhaseRootRows>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     attr = true;
   }
-  switch (kind) {
-    case kPhaseCellFwd:
-      k_merged_phase<kPhaseCellFwd><<<total, 256, smem, s>>>(pre, K, level, views, active);
-      break;
-    case kPhaseCellBwd:
-      k_merged_phase<kPhaseCellBwd><<<total, 256, smem, s>>>(pre, K, level, views, active);
-      break;
-    case kPhaseGroupFwd:
-      k_merged_phase<kPhaseGroupFwd><<<total, 256, smem, s>>>(pre, K, level, views, active);
-      break;
-    case kPhaseGroupBwd:
-      k_merged_phase<kPhaseGroupBwd><<<total, 256, smem, s>>>(pre, K, level, views, active);
-      break;
-    default:
-      k_merged_phase<kPhaseRootRows><<<total, 256, smem, s>>>(pre, K, 1 << 20, views, active);
-      break;
+  if (small_only && (kind == kPhaseGroupFwd || kind == kPhaseGroupBwd)) {
+    HIF_CUDA_TRY(launch_merged(dep, kind == kPhaseGroupFwd ? k_merged_small<true> : k_merged_small<false>, total, 256,
+                               0, s, pre, K, level, views, active));
+    note_launch();
+    return HIF_OK;
   }
+  auto kern = k_merged_phase<kPhaseRootRows>;
+  if (kind == kPhaseCellFwd) kern = k_merged_phase<kPhaseCellFwd>;
+  if (kind == kPhaseCellBwd) kern = k_merged_phase<kPhaseCellBwd>;
+  if (kind == kPhaseGroupFwd) kern = k_merged_phase<kPhaseGroupFwd>;
+  if (kind == kPhaseGroupBwd) kern = k_merged_phase<kPhaseGroupBwd>;
+  HIF_CUDA_TRY(launch_merged(dep, kern, total, 256, smem, s, pre, K, kind == kPhaseRootRows ? 1 << 20 : level, views,
+                             active));
   note_launch();
-  HIF_CUDA_TRY(cudaGetLastError());
   return HIF_OK;
 }
 
 // The S-form cells of a level of all handles, through the bulk-copy kernels: one
 // persistent launch streams the cells of every handle.  A CTA per cell reading S and
 // V through L1 took 183 us forward and 362 us backward for the leaf cells of 24
-// problems of 63^2 to 511^2 (14592 cells, 1 GB); @BATCH@ now.
-int launch_merged_sform(bool bwd, int level, const int *pre, int K, int total, int max_nI, int max_nB,
+// problems of 63^2 to 511^2 (14592 cells, 1 GB); 76 and 156 us now.
+int launch_merged_sform(bool bwd, int level, const int *pre, int K, int total, int max_nI, int max_nB, bool dep,
                         HandleView *const *views, const int *active, double *err, cudaStream_t s) {
   if (total <= 0) return HIF_OK;
   const BatchLevel src{pre, K, level, bwd ? 1 : 0, views, active};
@@ -2925,12 +2977,14 @@ int launch_merged_sform(bool bwd, int level, const int *pre, int K, int total, i
     auto kern = k_cell_bwd_tma_S<float, true, BatchLevel>;
     const size_t sm = (size_t)kStagesBwd * kStageBytes + tma_bwd_smem_elems(d) * sizeof(float);
     HIF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    kern<<<tma_grid((const void *)kern, sm, total, 0), kTmaThreads, sm, s>>>(src, total, err, max_nI, max_nB);
+    HIF_CUDA_TRY(launch_merged(dep, kern, tma_grid((const void *)kern, sm, total, 0), kTmaThreads, sm, s, src, total,
+                               err, max_nI, max_nB));
   } else {
     auto kern = k_cell_fwd_tma_S<float, BatchLevel>;
     const size_t sm = (size_t)kStagesFwd * kStageBytes + tma_fwd_smem_elems(d) * sizeof(float);
     HIF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    kern<<<tma_grid((const void *)kern, sm, total, 0), kTmaThreads, sm, s>>>(src, total, err, max_nI, max_nB);
+    HIF_CUDA_TRY(launch_merged(dep, kern, tma_grid((const void *)kern, sm, total, 0), kTmaThreads, sm, s, src, total,
+                               err, max_nI, max_nB));
   }
   note_launch();
   HIF_CUDA_TRY(cudaGetLastError());

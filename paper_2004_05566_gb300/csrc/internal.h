@@ -207,6 +207,8 @@ struct HandleView {
   float *contrib, *xI, *z;
   const int *ridx;
   long long root_G_off;
+  const float *root_S;            // full symmetric root (or null), its row stride
+  int root_S_ld;
   // CG (FP64) and the stencil
   double *r, *p, *q, *g, *x, *w;
   const double *diag, *wx, *wy, *wz;
@@ -421,11 +423,11 @@ bool level_uses_sform(const Handle *h, int l);
 int build_view(Handle *h);
 int build_items(Handle *h, LevelDev &D, const LevelHost &H, int target, cudaStream_t s);
 void merged_units(const Handle *h, int kind, int level, int *units, size_t *smem);
-int launch_merged_phase(int kind, int level, const int *pre, int K, int total, size_t smem,
+int launch_merged_phase(int kind, int level, const int *pre, int K, int total, size_t smem, bool small_only, bool dep,
                         HandleView *const *views, const int *active, cudaStream_t s);
 // the cells of a level that the bulk-copy S-form kernels take (merged steps)
 bool merged_sform(const Handle *h, int level);
-int launch_merged_sform(bool bwd, int level, const int *pre, int K, int total, int max_nI, int max_nB,
+int launch_merged_sform(bool bwd, int level, const int *pre, int K, int total, int max_nI, int max_nB, bool dep,
                         HandleView *const *views, const int *active, double *err, cudaStream_t s);
 int pcg(Handle *h, const double *b, double *x, int *iters, double *relres, cudaStream_t s);
 int cn(Handle *h, const double *u, const double *r, double *u1, int *iters, cudaStream_t s);

@@ -1130,7 +1130,7 @@ int cn_multi(Handle *h, double *u, const double *r, int nsteps, int *iters, cuda
 // CG tolerance (the single path applies the leaf levels in the S form).
 
 // 8 elements a thread: 8192 left 24 problems of 63^2 to 511^2 with 199 CTAs (w = A z
-// and the update 90 and 69 us an iteration; @SEG@ now)
+// and the update 90 and 69 us an iteration; 42 and 34 now)
 constexpr int kSeg = 2048;
 enum { B_RZ = 0, B_ALPHA, B_BETA, B_RR, B_BB, B_PQ, B_IT, B_CONV, B_COUNT };
 
@@ -1448,6 +1448,7 @@ int cn_batched_merged(Handle *const *hs, int K, const double *const *u, const do
   std::memcpy(hi, segpre.data(), (K + 1) * sizeof(int));
   std::vector<int> totals(P, 0), stotals(P, 0), smax_nI(P, 0), smax_nB(P, 0);
   std::vector<size_t> smem(P, 0);
+  std::vector<char> small(P, 1);  // no handle has a large entity in the phase
   for (int ph = 0; ph < P; ++ph) {
     int *pre = hi + (size_t)(K + 1) * (2 * ph + 1), *spre = pre + K + 1;
     const int kind = phases[ph].x, level = phases[ph].y;
@@ -1461,6 +1462,7 @@ int cn_batched_merged(Handle *const *hs, int K, const double *const *u, const do
       run += un;
       spre[i] = srun;
       if (un > 0) smem[ph] = std::max(smem[ph], sm);
+      if (level < hs[i]->L && hs[i]->lv[level].nlarge > 0) small[ph] = 0;
       if (cell && level < hs[i]->L && merged_sform(hs[i], level)) {
         const LevelDev &lv = hs[i]->lv[level];
         srun += lv.ncells;
@@ -1510,20 +1512,34 @@ int cn_batched_merged(Handle *const *hs, int K, const double *const *u, const do
   int maxit = 0;
   for (int i = 0; i < K; ++i) maxit = std::max(maxit, hs[i]->opt.cg_maxit);
   for (int it = 0; n_act > 0 && it < maxit; ++it) {
+    // Dependent launches after the first one of the iteration: a launch starts its
+    // prologue (the handle's lookup, descriptors, factor prefetches) beside the launch
+    // before it.  It reads only what was written before the launch before it began:
+    // the active flags are set before the iteration's first launch, which is plain.
+    bool dep = false;
     for (int ph = 0; ph < P; ++ph) {
       const int *pre = dint + (size_t)(K + 1) * (2 * ph + 1);
       HIF_TRY(launch_merged_sform(phases[ph].x == kPhaseCellBwd, phases[ph].y, pre + K + 1, K, stotals[ph],
-                                  smax_nI[ph], smax_nB[ph], const_cast<HandleView *const *>(B.views), active, werr, s));
-      HIF_TRY(launch_merged_phase(phases[ph].x, phases[ph].y, pre, K, totals[ph], smem[ph],
+                                  smax_nI[ph], smax_nB[ph], dep, const_cast<HandleView *const *>(B.views), active, werr,
+                                  s));
+      dep = dep || stotals[ph] > 0;
+      HIF_TRY(launch_merged_phase(phases[ph].x, phases[ph].y, pre, K, totals[ph], smem[ph], small[ph] != 0, dep,
                                   const_cast<HandleView *const *>(B.views), active, s));
+      dep = dep || totals[ph] > 0;
     }
     k_b_wz<<<total_seg, NT, 0, s>>>(B, active, sc, part);
     k_b_scalar<<<sgrid, 256, 0, s>>>(B, 4, active, sc, part, nactive);
     k_b_update<<<total_seg, NT, 0, s>>>(B, active, sc, part);
-    k_b_true_res<<<total_seg, NT, 0, s>>>(B, active, sc, part);
+    bool true_res = false;  // the active handles are all at iteration it + 1
+    for (int i = 0; i < K; ++i)
+      true_res = true_res || (hs[i]->opt.true_res_period > 0 && (it + 1) % hs[i]->opt.true_res_period == 0);
+    if (true_res) {
+      k_b_true_res<<<total_seg, NT, 0, s>>>(B, active, sc, part);
+      note_launch();
+    }
     HIF_CUDA_TRY(cudaMemsetAsync(nactive, 0, sizeof(int), s));
     k_b_scalar<<<sgrid, 256, 0, s>>>(B, 3, active, sc, part, nactive);
-    note_launch(5);
+    note_launch(4);
     HIF_CUDA_TRY(cudaGetLastError());
     HIF_TRY(read_active(&n_act));
   }
