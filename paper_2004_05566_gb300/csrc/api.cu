@@ -372,7 +372,8 @@ int build_contrib_map(Handle *h, LevelHost &H) {
     tot += H.groups[g].n;
   }
   gstart[H.groups.size()] = tot;
-  std::vector<std::vector<long long>> slots(tot);
+  // counted, then filled in cell order
+  std::vector<int> at(tot + 1, 0);
   for (auto &c : H.cells) {
     const int *B = h->idx_host.data() + c.B_off;
     for (int b = 0; b < c.nB; ++b) {
@@ -380,16 +381,20 @@ int build_contrib_map(Handle *h, LevelHost &H) {
         set_last_error("cell boundary DOF is not a DOF of any group of its level");
         return HIF_EFORMAT;
       }
-      slots[gpos[B[b]]].push_back(c.C_off + b);
+      ++at[gpos[B[b]] + 1];
     }
   }
+  const long long base = (long long)h->cslot_host.size();
+  for (long long t = 0; t < tot; ++t) at[t + 1] += at[t];
+  h->cptr_host.reserve(h->cptr_host.size() + tot + H.groups.size());
   for (size_t g = 0; g < H.groups.size(); ++g) {
     H.groups[g].cptr_off = (long long)h->cptr_host.size();
-    for (int i = 0; i < H.groups[g].n; ++i) {
-      h->cptr_host.push_back((long long)h->cslot_host.size());
-      for (long long sl : slots[gstart[g] + i]) h->cslot_host.push_back(sl);
-    }
-    h->cptr_host.push_back((long long)h->cslot_host.size());
+    for (long long t = gstart[g]; t <= gstart[g + 1]; ++t) h->cptr_host.push_back(base + at[t]);
+  }
+  h->cslot_host.resize(base + at[tot]);
+  for (auto &c : H.cells) {
+    const int *B = h->idx_host.data() + c.B_off;
+    for (int b = 0; b < c.nB; ++b) h->cslot_host[base + at[gpos[B[b]]]++] = c.C_off + b;
   }
   return HIF_OK;
 }

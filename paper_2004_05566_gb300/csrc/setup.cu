@@ -1018,13 +1018,6 @@ struct Plan {
   std::vector<std::vector<int>> g_boff;  // offset of g inside each adjacent cell's B
 };
 
-void coords_of(long long d, int n, int dim, int c[3]) {
-  const long long S = n - 1;
-  c[0] = (int)(d % S) + 1;
-  c[1] = (int)((d / S) % S) + 1;
-  c[2] = dim == 3 ? (int)(d / (S * S)) + 1 : 0;
-}
-
 Plan make_plan(const std::vector<int> &active, int n, int dim, int leaf, int l) {
   Plan P;
   P.l = l;
@@ -1037,26 +1030,35 @@ Plan make_plan(const std::vector<int> &active, int n, int dim, int leaf, int l) 
   P.cI.assign(P.ncells, {});
   std::vector<int> gid_of_key(nkeys, -1);
   std::vector<int> key_of_dof(active.size());
-  // pass 1: which keys hold group DOFs
+  // pass 1: the cell (~cell) or the key of every DOF.  The DOFs ascend, so the grid
+  // row changes seldom and a coordinate's code (cell or separator plane along its
+  // axis) comes from a table: no divisions per DOF.
+  std::vector<int> code_of(n);
+  for (int c = 1; c < n; ++c) code_of[c] = 2 * (c / s) + (c % s != 0);
+  const long long S1 = n - 1;
+  std::vector<int> cell_count(P.ncells, 0);
+  long long row = -1;  // first DOF of the current grid row
+  int c1 = 0, c2 = 0;
   for (size_t t = 0; t < active.size(); ++t) {
-    int c[3];
-    coords_of(active[t], n, dim, c);
-    int code[3] = {0, 0, 0};
-    int codim = 0;
-    for (int ax = 0; ax < dim; ++ax) {
-      code[ax] = 2 * (c[ax] / s) + (c[ax] % s != 0);
-      if (code[ax] % 2 == 0) ++codim;
+    const long long d = active[t];
+    if (row < 0 || d >= row + S1) {
+      const long long r = d / S1;
+      row = r * S1;
+      c1 = code_of[r % S1 + 1];
+      c2 = dim == 3 ? code_of[r / S1 + 1] : 1;
     }
-    long long key = code[0] + (long long)D * code[1] + (long long)D * D * code[2];
-    if (codim == 0) {
-      int cid = (code[0] - 1) / 2 + nc * ((code[1] - 1) / 2) + (dim == 3 ? nc * nc * ((code[2] - 1) / 2) : 0);
-      P.cI[cid].push_back(active[t]);
-      key_of_dof[t] = -1;
+    const int c0 = code_of[d - row + 1];
+    if (c0 & c1 & c2 & 1) {
+      const int cid = c0 / 2 + nc * (c1 / 2) + (dim == 3 ? nc * nc * (c2 / 2) : 0);
+      key_of_dof[t] = ~cid;
+      ++cell_count[cid];
     } else {
-      gid_of_key[key] = 0;
+      const long long key = c0 + (long long)D * c1 + (dim == 3 ? (long long)D * D * c2 : 0);
       key_of_dof[t] = (int)key;
+      gid_of_key[key] = 0;
     }
   }
+  for (int c = 0; c < P.ncells; ++c) P.cI[c].reserve(cell_count[c]);
   // number groups in ascending key order
   int ng = 0;
   for (long long key = 0; key < nkeys; ++key)
@@ -1067,8 +1069,12 @@ Plan make_plan(const std::vector<int> &active, int n, int dim, int leaf, int l) 
   P.g_dofs.assign(ng, {});
   P.g_codim.assign(ng, 0);
   P.g_cells.assign(ng, {});
+  std::vector<int> g_count(ng, 0);
+  for (int k : key_of_dof)
+    if (k >= 0) ++g_count[gid_of_key[k]];
+  for (int g = 0; g < ng; ++g) P.g_dofs[g].reserve(g_count[g]);
   for (size_t t = 0; t < active.size(); ++t)
-    if (key_of_dof[t] >= 0) P.g_dofs[gid_of_key[key_of_dof[t]]].push_back(active[t]);
+    (key_of_dof[t] >= 0 ? P.g_dofs[gid_of_key[key_of_dof[t]]] : P.cI[~key_of_dof[t]]).push_back(active[t]);
   P.cG.assign(P.ncells, {});
   for (int g = 0; g < ng; ++g) {
     int key = P.g_key[g];
@@ -1096,25 +1102,19 @@ Plan make_plan(const std::vector<int> &active, int n, int dim, int leaf, int l) 
           P.cG[cid].push_back(g);
         }
   }
+  // boundary DOFs of a cell, and the offset of each entity in each of its cells (the
+  // cells of an entity ascend, as the outer loop does)
   P.cB.assign(P.ncells, {});
   P.g_boff.assign(ng, {});
-  std::vector<int> off_in_cell(ng, 0);
   for (int c = 0; c < P.ncells; ++c) {
-    int o = 0;
+    size_t nB = 0;
+    for (int g : P.cG[c]) nB += P.g_dofs[g].size();
+    P.cB[c].reserve(nB);
     for (int g : P.cG[c]) {
-      for (int d : P.g_dofs[g]) P.cB[c].push_back(d);
-      o += (int)P.g_dofs[g].size();
+      P.g_boff[g].push_back((int)P.cB[c].size());
+      P.cB[c].insert(P.cB[c].end(), P.g_dofs[g].begin(), P.g_dofs[g].end());
     }
   }
-  for (int g = 0; g < ng; ++g)
-    for (int c : P.g_cells[g]) {
-      int o = 0;
-      for (int g2 : P.cG[c]) {
-        if (g2 == g) break;
-        o += (int)P.g_dofs[g2].size();
-      }
-      P.g_boff[g].push_back(o);
-    }
   return P;
 }
 
