@@ -6,15 +6,15 @@
 // and the apply operators G = L^{-1} and V = A_BI A_II^{-1} = W^T G.
 //
 // The partial Cholesky is right-looking and blocked by panels of 32 columns:
-// per panel one launch factors the 32 x 32 diagonal block (a warp per cell),
+// per panel one launch factors the 32 x 32 diagonal block (a CTA per cell),
 // one solves the panel rows below it (many CTAs per cell, one row per thread),
 // and one applies the rank-32 update to the trailing lower triangle in 64 x 64
 // tiles (one CTA per tile).
 // So every cell of a level, small or large, spreads over as many CTAs as its
 // size gives, and the trailing matrix is read and written once per panel
 // instead of once per column.  G is formed by 32 x 32 blocks: the diagonal
-// blocks are inverted first, then each CTA owns one block column and walks down
-// it, G_rc = -G_rr sum_k L_rk G_kc.  V = W^T G is a 64 x 64-tiled product.
+// blocks are inverted first, then small cells walk down their block columns and
+// larger ones join neighbouring blocks by doubling, G21 = -G22 (L21 G11).  V = W^T G is a 64 x 64-tiled product.
 // Every sum runs in a fixed order, so the factor is the same on every run.
 //
 // The kernels are templates over the cell descriptor, which must provide
@@ -33,6 +33,10 @@ constexpr int kPanel = 32;   // panel width of the blocked Cholesky and G blocks
 constexpr int kTile = 64;    // tile edge of the trailing update and of V
 constexpr int kThreads = 256;
 constexpr int kMaxGridY = 65535;  // the launch limit of grid.y
+// up to this size a block column of the inverse has at most 28 dependent block
+// products and one launch does it (2D 511^2, cells of 53 to 121: 0.3 ms in all
+// against 1.2 in the launches of the doubling); above it the doubling spreads it
+constexpr int kInvColumn = 256;
 
 __host__ __device__ inline int ceil_div(long long a, int b) { return (int)((a + b - 1) / b); }
 
@@ -46,41 +50,64 @@ __device__ inline void tri_tile(int x, int &ti, int &tj) {
 }
 
 // Panel step j0, part 1: factor the diagonal block D = F[j0:j0+jb, j0:j0+jb]
-// (lower) in place.  grid = cells, one warp; lane i owns row i.  Non-positive
-// pivots set *err and are replaced by 1 so the kernel completes.
+// (lower) in place.  grid = cells, kThreads threads; the rank-1 update of a step is
+// spread over all of them (thread t owns entries t, t + 256, ... of the 32 x 32
+// block).  One warp with a row a lane took up to 31 dependent multiply-adds a step
+// on a pipe that starts a warp's every 64 cycles: 70 us a launch at 3D 47^3, and a
+// launch a panel; @DIAG@ now.  Non-positive pivots set *err and are replaced by 1 so
+// the kernel completes.
 template <class Cell>
-__global__ void __launch_bounds__(32) k_chol_diag(const Cell *__restrict__ cells,
-                                                  double *__restrict__ F, int j0,
-                                                  int *__restrict__ err) {
-  __shared__ double D[kPanel][kPanel + 1];
+__global__ void __launch_bounds__(kThreads) k_chol_diag(const Cell *__restrict__ cells,
+                                                        double *__restrict__ F, int j0,
+                                                        int *__restrict__ err) {
+  __shared__ double D[kPanel][kPanel + 1], s_r[3];
   const Cell c = cells[blockIdx.x];
   if (c.nI <= j0) return;
   const int nn = c.nI + c.nB;
   const int jb = min(kPanel, c.nI - j0);
   double *A = F + c.F_off;
-  const int lane = threadIdx.x;
-  for (int j = 0; j < jb; ++j)
-    D[lane][j] = (lane < jb && j <= lane) ? A[(j0 + lane) + (long long)(j0 + j) * nn] : 0.0;
-  __syncwarp();
-  for (int k = 0; k < jb; ++k) {
-    double d = D[k][k];
-    if (!(d > 0.0)) {
-      if (lane == 0) atomicExch(err, 1);
-      d = 1.0;
-    }
-    d = sqrt(d);
-    __syncwarp();
-    if (lane == k) D[k][k] = d;
-    if (lane > k && lane < jb) D[lane][k] /= d;
-    __syncwarp();
-    if (lane > k && lane < jb) {  // rank-1 update of row `lane`
-      const double lk = D[lane][k];
-      for (int j = k + 1; j <= lane; ++j) D[lane][j] -= lk * D[j][k];
-    }
-    __syncwarp();
+  const int i = threadIdx.x % kPanel, q = threadIdx.x / kPanel;  // row; columns q + 8 v
+  constexpr int kV = kPanel * kPanel / kThreads;
+#pragma unroll
+  for (int v = 0; v < kV; ++v) {
+    const int j = q + 8 * v;
+    D[i][j] = (i < jb && j <= i) ? A[(j0 + i) + (long long)(j0 + j) * nn] : 0.0;
   }
-  for (int j = 0; j < jb; ++j)
-    if (lane < jb && j <= lane) A[(j0 + lane) + (long long)(j0 + j) * nn] = D[lane][j];
+  __syncthreads();
+  for (int k = 0; k < jb; ++k) {
+    // L[i][k] = D[i][k] r with r = 1 / sqrt(D[k][k]), formed by one warp (a root is
+    // fifteen FP64 instructions, for every warp that takes it); the update uses D's
+    // column and r r, the column is scaled after the barrier
+    if (q == 0) {
+      double d = D[k][k];
+      if (!(d > 0.0)) {
+        if (i == 0) atomicExch(err, 1);
+        d = 1.0;
+      }
+      const double r = rsqrt(d);
+      if (i == 0) {
+        s_r[0] = r;
+        s_r[1] = r * r;
+        s_r[2] = d * r;
+      }
+    }
+    __syncthreads();
+    const double dik = D[i][k], li = dik * s_r[1];
+#pragma unroll
+    for (int v = 0; v < kV; ++v) {
+      const int j = q + 8 * v;
+      if (i > k && i < jb && j > k && j <= i) D[i][j] -= li * D[j][k];
+    }
+    __syncthreads();
+    if (q == 0 && i >= k && i < jb) D[i][k] = i == k ? s_r[2] : dik * s_r[0];
+    // (the next step reads columns > k only; column k is next read after the loop)
+  }
+  __syncthreads();
+#pragma unroll
+  for (int v = 0; v < kV; ++v) {
+    const int j = q + 8 * v;
+    if (i < jb && j <= i) A[(j0 + i) + (long long)(j0 + j) * nn] = D[i][j];
+  }
 }
 
 // Panel step j0, part 2: solve the rows below the factored diagonal block,
@@ -214,7 +241,7 @@ __global__ void __launch_bounds__(32) k_inv_diag_blocks(const Cell *__restrict__
     if (lane <= r) G[tri_off(b0 + r) + b0 + lane] = X[r][lane];
 }
 
-// Off-diagonal blocks of G, one block column per CTA:
+// Off-diagonal blocks of G of small cells (nI <= kInvColumn), one block column per CTA:
 // for rb > cb: G_{rb,cb} = -G_{rb,rb} sum_{kb=cb}^{rb-1} L_{rb,kb} G_{kb,cb}.
 // grid = (cells, block columns).  The CTA reads back the blocks it wrote.
 template <class Cell>
@@ -278,6 +305,85 @@ __global__ void __launch_bounds__(kThreads) k_inv_offdiag(const Cell *__restrict
       }
     }
     __syncthreads();  // G block visible to the next rb; shared buffers free
+  }
+}
+
+// Off-diagonal blocks of G of larger cells by doubling: with the inverses of two neighbouring
+// diagonal blocks of b rows known (rows [r0, r0 + b) and [r0 + b, r0 + 2 b)),
+//   G21 = -G22 (L21 G11),
+// as two products in 64 x 64 tiles, b = 32, 64, ...; every pair of every cell is a
+// CTA of its own, so a single large cell (the root) fills the chip.  The sum of the
+// products over the levels is that of the direct form, n^3 / 6 and the tiles' edges;
+// one CTA per block column walking down it took 20 ms for the 2108 root unknowns of
+// 3D 47^3, where the first column alone holds 2145 dependent block products; all
+// inverses there 30 -> 20 ms.
+// T = L21 G11 is kept in the unused upper triangle of A_II: T(i, j) at (j, i).
+// grid = (cells, pairs x tiles); kSecond: the second product.
+template <class Cell, bool kSecond>
+__global__ void __launch_bounds__(kThreads) k_inv_double(const Cell *__restrict__ cells,
+                                                         double *__restrict__ F,
+                                                         double *__restrict__ vals, int b) {
+  __shared__ double As[kPanel][kTile + 1];  // [k][i]
+  __shared__ double Bs[kPanel][kTile + 1];  // [k][j]
+  const Cell c = cells[blockIdx.x];
+  const int nI = c.nI, nn = nI + c.nB;
+  const int tpb = ceil_div(b, kTile), npair = ceil_div(nI, 2 * b);
+  double *A = F + c.F_off;
+  double *G = vals + c.G_off;
+  for (int y = blockIdx.y; y < npair * tpb * tpb; y += gridDim.y) {
+    const int p = y / (tpb * tpb), r1 = 2 * b * p + b, c0 = 2 * b * p;  // block 2 starts at r1
+    const int rend = min(nI, r1 + b);
+    const int i0 = r1 + (y % tpb) * kTile, j0 = c0 + (y / tpb % tpb) * kTile;
+    if (i0 >= rend) continue;
+    const int iend = min(rend, i0 + kTile), jend = min(r1, j0 + kTile);
+    double acc[4][4] = {};
+    // first: k over block 1 from j0 (G11 is lower); second: k over block 2 up to i
+    const int kb = kSecond ? r1 : j0, ke = kSecond ? iend : r1;
+    for (int k0 = kb; k0 < ke; k0 += kPanel) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < kPanel * kTile; e += kThreads) {
+        if (kSecond) {  // G22 rows run along k
+          const int ka = e % kPanel, i = i0 + e / kPanel, k = k0 + ka;
+          As[ka][e / kPanel] = i < iend && k < ke && k <= i ? G[tri_off(i) + k] : 0.0;
+        } else {
+          const int ka = e / kTile, i = i0 + e % kTile, k = k0 + ka;
+          As[ka][e % kTile] = i < iend && k < ke ? A[i + (long long)k * nn] : 0.0;
+        }
+        const int kk = e / kTile, j = j0 + e % kTile, k = k0 + kk;
+        double v = 0.0;
+        if (j < jend && k < ke) {
+          if (kSecond) v = A[j + (long long)k * nn];  // T(k, j)
+          else if (j <= k) v = G[tri_off(k) + j];
+        }
+        Bs[kk][e % kTile] = v;
+      }
+      __syncthreads();
+      const int tj = threadIdx.x % 16, ti = threadIdx.x / 16;
+#pragma unroll 8
+      for (int k = 0; k < kPanel; ++k) {
+        double a[4], x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          a[u] = As[k][ti + 16 * u];
+          x[u] = Bs[k][tj + 16 * u];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int v = 0; v < 4; ++v) acc[u][v] += a[u] * x[v];
+      }
+    }
+    const int tj = threadIdx.x % 16, ti = threadIdx.x / 16;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int i = i0 + ti + 16 * u, j = j0 + tj + 16 * v;
+        if (i >= iend || j >= jend) continue;
+        if (kSecond) G[tri_off(i) + j] = -acc[u][v];
+        else A[j + (long long)i * nn] = acc[u][v];
+      }
+    __syncthreads();  // As / Bs are refilled for the next tile
   }
 }
 
@@ -367,7 +473,7 @@ int eliminate_cells(const std::vector<Cell> &cells_h, const Cell *cells_d, doubl
     max_nn = max_nn > c.nI + c.nB ? max_nn : c.nI + c.nB;
   }
   for (int j0 = 0; j0 < max_nI; j0 += kPanel) {
-    k_chol_diag<Cell><<<ncells, 32, 0, s>>>(cells_d, F, j0, err);
+    k_chol_diag<Cell><<<ncells, kThreads, 0, s>>>(cells_d, F, j0, err);
     note_launch();
     const int rest = max_nn - (j0 + 1);  // upper bound on the rows below the panel over all cells
     if (rest > 0) {
@@ -384,9 +490,16 @@ int eliminate_cells(const std::vector<Cell> &cells_h, const Cell *cells_d, doubl
   if (nbk > 0) {
     k_inv_diag_blocks<Cell><<<dim3(ncells, nbk), 32, 0, s>>>(cells_d, F, vals);
     note_launch();
-    if (nbk > 1) {
+    if (nbk > 1 && max_nI <= kInvColumn) {
       k_inv_offdiag<Cell><<<dim3(ncells, nbk - 1), kThreads, 0, s>>>(cells_d, F, vals);
       note_launch();
+    }
+    for (int b = kPanel; max_nI > kInvColumn && b < max_nI; b *= 2) {
+      const long long t = (long long)ceil_div(b, kTile) * ceil_div(b, kTile) * ceil_div(max_nI, 2 * b);
+      const dim3 grid(ncells, (int)std::min<long long>(t, kMaxGridY));
+      k_inv_double<Cell, false><<<grid, kThreads, 0, s>>>(cells_d, F, vals, b);
+      k_inv_double<Cell, true><<<grid, kThreads, 0, s>>>(cells_d, F, vals, b);
+      note_launch(2);
     }
   }
   if (max_nB > 0 && max_nI > 0) {
