@@ -171,14 +171,46 @@ __device__ __forceinline__ T ldv(const __nv_bfloat16 *p) { return (T)__bfloat162
 // FP64 row dots of the apply.  GB300's FP64 pipe retires about two lane
 // operations per clock per SM, and the whole-warp sum of a row costs five
 // additions on all 32 lanes: more than the seven products a lane has in a row
-// of 225.  So eight lanes take a row and a warp four rows at a time (16-byte
-// loads, four in flight per lane): three additions per four rows.  Measured
-// on the 1023^2 leaf forward step (FP64 pipe bound, floor 274 us): 903 -> 444 us.
+// of 225.  So L lanes take a row and a warp 32 / L rows at a time: log2(L) + 1
+// additions for all of them, 16-byte loads, four in flight per lane.  maxp is
+// the longest row of the warp in pairs; a pair that no row of the warp has
+// costs no product.  The L lanes of a row return its sum.  kShared: the row is
+// in shared memory.  Measured on the 1023^2 leaf forward step (FP64 pipe bound,
+// floor 274 us): 903 us with a row per warp, 444 with L = 8, 375 with L = 4;
+// L = 4 needs eight rows a warp, so it is taken where every warp has them twice.
+template <int L, bool kShared = false>
+__device__ __forceinline__ double row_dot_f64(const double *row, int np2, int maxp, const double *xs) {
+  const int sub = threadIdx.x & (L - 1);
+  double a = 0.0, b = 0.0;
+  for (int p0 = 0; p0 < maxp; p0 += 4 * L) {
+    double2 v[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int p = p0 + sub + L * k;
+      if constexpr (kShared) v[k] = p < np2 ? *reinterpret_cast<const double2 *>(row + 2 * p) : make_double2(0.0, 0.0);
+      else ld2_stream(row + 2 * p, p < np2, v[k].x, v[k].y);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (p0 + L * k < maxp) {
+        const int p = min(p0 + sub + L * k, maxp - 1);
+        const double2 xv = *reinterpret_cast<const double2 *>(xs + 2 * p);
+        a += v[k].x * xv.x;
+        b += v[k].y * xv.y;
+      }
+    }
+  }
+  a += b;
+#pragma unroll
+  for (int o = L / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
 __device__ __forceinline__ void warp_rows_dot4_f64(const double *const (&rp)[kRows],
                                                    const int (&nq)[kRows], const double *xs,
                                                    double (&acc)[kRows]) {
   static_assert(kRows == 4, "a row per eight lanes");
-  const int lane = threadIdx.x & 31, sub = lane & 7;
+  const int lane = threadIdx.x & 31;
   const double *row = rp[0];
   int np2 = 2 * nq[0];  // pairs of the lane's row
 #pragma unroll
@@ -187,32 +219,33 @@ __device__ __forceinline__ void warp_rows_dot4_f64(const double *const (&rp)[kRo
       row = rp[u];
       np2 = 2 * nq[u];
     }
-  double a = 0.0, b = 0.0;
-  int p = sub;
-  for (; p + 24 < np2; p += 32) {
-    double2 v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) ld2_stream(row + 2 * (p + 8 * k), true, v[k].x, v[k].y);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const double2 xv = *reinterpret_cast<const double2 *>(xs + 2 * (p + 8 * k));
-      a += v[k].x * xv.x;
-      b += v[k].y * xv.y;
-    }
-  }
-#pragma unroll 3
-  for (; p < np2; p += 8) {
-    const double2 v = *reinterpret_cast<const double2 *>(row + 2 * p);
-    const double2 xv = *reinterpret_cast<const double2 *>(xs + 2 * p);
-    a += v.x * xv.x;
-    b += v.y * xv.y;
-  }
-  a += b;
-  a += __shfl_xor_sync(0xffffffffu, a, 4);
-  a += __shfl_xor_sync(0xffffffffu, a, 2);
-  a += __shfl_xor_sync(0xffffffffu, a, 1);
+  const int maxp = 2 * max(max(nq[0], nq[1]), max(nq[2], nq[3]));
+  const double a = row_dot_f64<8>(row, np2, maxp, xs);
 #pragma unroll
   for (int u = 0; u < kRows; ++u) acc[u] = __shfl_sync(0xffffffffu, a, 8 * u);
+}
+
+// Rows [a, b) of a cell's stacked [V; G] by NW warps, L lanes a row: each lane
+// finds its own row, so nothing is indexed by warp.
+template <int L, int NW>
+__device__ __forceinline__ void cell_fwd_rows_f64(const CellItem &it, const CellDesc &c, const int *I,
+                                                  const double *V, const double *G, int nIp, double *contrib,
+                                                  double *xI, const double *xs) {
+  constexpr int R = 32 / L;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int r0 = it.a + warp * R; r0 < it.b; r0 += NW * R) {
+    const int r = r0 + lane / L, last = min(r0 + R, it.b) - 1;
+    const int i = r - c.nB;
+    const int full = nIp / 2;
+    const int np2 = r >= it.b ? 0 : i < 0 ? full : 2 * ((i + 4) / 4);
+    const int maxp = r0 < c.nB ? full : 2 * ((last - c.nB + 4) / 4);
+    const double *row = r >= it.b ? V : i < 0 ? V + (long long)r * nIp : G + tri_off(i);
+    const double t = row_dot_f64<L>(row, np2, maxp, xs);
+    if (lane % L == 0 && r < it.b) {
+      if (i < 0) contrib[c.C_off + r] = t;
+      else xI[I[i]] = t;
+    }
+  }
 }
 
 // Dot products of kRows padded rows (pointers rp, lengths in quads nq) with
@@ -296,6 +329,12 @@ __device__ __forceinline__ void cell_fwd_unit(const CellItem &it, const CellDesc
   const TV *V = vals + c.V_off;
   const TV *G = vals + c.G_off;
   const int vq = nIp / 4;
+  if constexpr (std::is_same_v<TV, double>) {
+    // 16 rows per warp: the leaf cells whole or cut into a few items
+    if (it.b - it.a >= 16 * NW) cell_fwd_rows_f64<4, NW>(it, c, I, V, G, nIp, contrib, xI, xs);
+    else cell_fwd_rows_f64<8, NW>(it, c, I, V, G, nIp, contrib, xI, xs);
+    return;
+  }
   for (int r0 = it.a + warp * kRows; r0 < it.b; r0 += NW * kRows) {
     const TV *rp[kRows];
     int nq[kRows];
@@ -329,7 +368,7 @@ __device__ __forceinline__ void cell_fwd_unit(const CellItem &it, const CellDesc
 }
 
 template <typename T, typename TV = T>
-__global__ void __launch_bounds__(kCellFwdThreads, sizeof(T) == 4 ? 3 : 4) k_cell_fwd(const CellItem *__restrict__ items,
+__global__ void __launch_bounds__(kCellFwdThreads, sizeof(T) == 4 ? 3 : 5) k_cell_fwd(const CellItem *__restrict__ items,
                                                               const CellDesc *__restrict__ cells,
                                                               const int *__restrict__ idx,
                                                               const TV *__restrict__ vals,
@@ -1670,6 +1709,55 @@ __global__ void __launch_bounds__(kRootThreads) k_root(int nr, const int *__rest
   root_unit<T, kRootThreads, TV>(nr, ridx, G, x, reinterpret_cast<T *>(smem_raw));
 }
 
+// Small roots, FP64 apply.  root_unit waits for its predecessor and then reads
+// G_r from L2 twice, the second time one double per thread in a serial chain.
+// Here G_r is copied to shared memory before the dependency point, in the
+// predecessor's shadow, and both passes run from there; what is left is the
+// gather of x_r and the FP64 pipe of one SM (2 us for 84 DOFs).  Roots whose
+// packed G_r fits beside the vectors: up to kRootStageMax DOFs (190 KB).
+// With the eight-row dots: 511^2 apply 400 -> 361 us, 63^2 step 168 -> 157 us.
+constexpr int kRootStageMax = 212;
+constexpr int kRootStageThreads = 512;
+
+__global__ void __launch_bounds__(kRootStageThreads) k_root_stage(int nr, const int *__restrict__ ridx,
+                                                                  const double *__restrict__ G,
+                                                                  double *__restrict__ x) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nrp = (int)pad4(nr), ng = (int)tri_off(nr);
+  double *Gs = reinterpret_cast<double *>(smem_raw), *xs = Gs + ng, *ts = xs + nrp, *part = ts + nrp;
+  for (int i = 2 * threadIdx.x; i < ng; i += 2 * kRootStageThreads)  // ng is a multiple of 4
+    *reinterpret_cast<double2 *>(Gs + i) = *reinterpret_cast<const double2 *>(G + i);
+  pdl_enter();
+  for (int i = threadIdx.x; i < nrp; i += kRootStageThreads) xs[i] = i < nr ? x[ridx[i]] : 0.0;
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int NW = kRootStageThreads / 32, R = 4;
+  for (int r0 = warp * R; r0 < nr; r0 += NW * R) {  // t = G x
+    const int r = r0 + (lane >> 3), last = min(r0 + R, nr) - 1;
+    const double t = row_dot_f64<8, true>(Gs + tri_off(min(r, last)), r < nr ? 2 * ((r + 4) / 4) : 0,
+                                          2 * ((last + 4) / 4), xs);
+    if ((lane & 7) == 0 && r < nr) ts[r] = t;
+  }
+  __syncthreads();
+  int CW, RG;
+  col_layout(nr, kRootStageThreads, CW, RG);
+  const int cl = threadIdx.x % CW, rg = threadIdx.x / CW;
+  for (int c0 = 0; c0 < nr; c0 += CW) {  // y = G^T t
+    const int col = c0 + cl;
+    double acc = 0.0;
+    if (rg < RG && col < nr)
+      for (int i = col + ((rg - col % RG) + RG) % RG; i < nr; i += RG) acc += Gs[tri_off(i) + col] * ts[i];
+    part[threadIdx.x] = acc;
+    __syncthreads();
+    if (rg == 0 && col < nr) {
+      double sum = part[cl];
+      for (int q = 1; q < RG; ++q) sum += part[q * CW + cl];
+      x[ridx[col]] = sum;
+    }
+    __syncthreads();
+  }
+}
+
 // Small roots, FP32 apply: x_r <- S_r x_r with S_r = G_r^T G_r stored as a
 // full symmetric matrix (rows of ld floats, zero padding): one pass of row
 // dots instead of the two dependent triangular passes of root_unit, whose
@@ -2284,6 +2372,8 @@ int set_smem_limits() {
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_group_fwd_level<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_group_bwd_level<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   HIF_CUDA_TRY(cudaFuncSetAttribute(k_root<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+  if constexpr (sizeof(T) == 8)
+    HIF_CUDA_TRY(cudaFuncSetAttribute(k_root_stage, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
   if constexpr (sizeof(T) == 4) {
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_level_fwd<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
     HIF_CUDA_TRY(cudaFuncSetAttribute(k_level_fwd<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
@@ -2752,6 +2842,14 @@ int apply_levels(Handle *h, const FactorValues<T> &fv, T *x, cudaStream_t s) {
           HIF_CUDA_TRY(launch_k(k_root<T, bf16>, 1, kRootThreads, sm, s, h->root_n, ridx,
                                                       static_cast<const bf16 *>(h->bf16_vals) + h->root_G_off,
                                                       x));
+          done = true;
+        }
+      }
+      if constexpr (sizeof(T) == 8) {
+        if (h->root_n <= kRootStageMax) {
+          sm = (tri_off(h->root_n) + 2 * (size_t)pad4(h->root_n) + kRootStageThreads) * sizeof(T);
+          HIF_CUDA_TRY(launch_k(k_root_stage, 1, kRootStageThreads, sm, s, h->root_n, ridx,
+                                fv.vals + h->root_G_off, x));
           done = true;
         }
       }
