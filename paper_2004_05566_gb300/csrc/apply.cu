@@ -211,14 +211,10 @@ __device__ __forceinline__ void warp_rows_dot4_f64(const double *const (&rp)[kRo
                                                    double (&acc)[kRows]) {
   static_assert(kRows == 4, "a row per eight lanes");
   const int lane = threadIdx.x & 31;
-  const double *row = rp[0];
-  int np2 = 2 * nq[0];  // pairs of the lane's row
-#pragma unroll
-  for (int u = 1; u < kRows; ++u)
-    if ((lane >> 3) == u) {
-      row = rp[u];
-      np2 = 2 * nq[u];
-    }
+  // the lane's row by selects (a chain of tests became an indexed local array)
+  const bool hi = lane & 16, odd = lane & 8;
+  const double *r01 = odd ? rp[1] : rp[0], *r23 = odd ? rp[3] : rp[2], *row = hi ? r23 : r01;
+  const int n01 = odd ? nq[1] : nq[0], n23 = odd ? nq[3] : nq[2], np2 = 2 * (hi ? n23 : n01);
   const int maxp = 2 * max(max(nq[0], nq[1]), max(nq[2], nq[3]));
   const double a = row_dot_f64<8>(row, np2, maxp, xs);
 #pragma unroll
@@ -391,12 +387,32 @@ __device__ __forceinline__ void group_fwd_unit(const GroupDesc &g, const int *__
                                                T *xs) {
   const int *gi = idx + g.idx_off;
   const int np = (int)pad4(g.n);
-  if constexpr (PDL)
+  // static part: the first DOF of the thread and its contribution slots
+  // (otherwise three dependent loads follow the dependency point)
+  constexpr int kSlots = 4;
+  const int i0 = threadIdx.x;
+  int dof = 0;
+  long long a0 = 0, b0 = 0, sl[kSlots] = {};
+  if constexpr (PDL) {
     if (threadIdx.x == 0) prefetch_block_l2(vals + g.H_off, (long long)g.n * np);
+    if (i0 < g.n) {
+      dof = gi[i0];
+      a0 = cptr[g.cptr_off + i0];
+      b0 = cptr[g.cptr_off + i0 + 1];
+#pragma unroll
+      for (int k = 0; k < kSlots; ++k) sl[k] = a0 + k < b0 ? cslot[a0 + k] : 0;
+    }
+  }
   unit_dependency_point<PDL>();
-  for (int i = threadIdx.x; i < np; i += NT) {
+  for (int i = i0; i < np; i += NT) {
     T v = T(0);
-    if (i < g.n) {
+    if (PDL && i == i0 && i < g.n) {
+      v = __ldcg(xin + dof);
+#pragma unroll
+      for (int k = 0; k < kSlots; ++k)
+        if (a0 + k < b0) v -= __ldcg(contrib + sl[k]);
+      for (long long s = a0 + kSlots; s < b0; ++s) v -= __ldcg(contrib + cslot[s]);
+    } else if (i < g.n) {
       v = __ldcg(xin + gi[i]);
       const long long a = cptr[g.cptr_off + i], b = cptr[g.cptr_off + i + 1];
       for (long long s = a; s < b; ++s) v -= __ldcg(contrib + cslot[s]);
@@ -585,10 +601,11 @@ __device__ __forceinline__ void group_bwd_unit(const GroupDesc &g, const int *__
   const int np = (int)pad4(g.n), nq = np / 4;
   T *part = xs + np;  // 4 * NT
   const int *gi = idx + g.idx_off;
+  const int i0 = threadIdx.x, dof = PDL && i0 < g.n ? gi[i0] : 0;
   if constexpr (PDL)
     if (threadIdx.x == 0) prefetch_block_l2(vals + g.H_off, (long long)g.n * np);
   unit_dependency_point<PDL>();
-  for (int i = threadIdx.x; i < g.n; i += NT) xs[i] = __ldcg(xin + gi[i]);
+  for (int i = i0; i < g.n; i += NT) xs[i] = __ldcg(xin + (PDL && i == i0 ? dof : gi[i]));
   __syncthreads();
   const TV *H = vals + g.H_off;
   int CW, RG;
@@ -598,12 +615,17 @@ __device__ __forceinline__ void group_bwd_unit(const GroupDesc &g, const int *__
     const int q = q0 + cl;
     T acc[4] = {T(0), T(0), T(0), T(0)};
     if (q < nq) {
-#pragma unroll 4
-      for (int i = rg; i < g.n; i += RG) {
-        T v[4];
-        ld4(H + (long long)i * np + 4 * q, v);
-        const T xv = xs[i];
-        acc[0] += v[0] * xv; acc[1] += v[1] * xv; acc[2] += v[2] * xv; acc[3] += v[3] * xv;
+      constexpr int kR = sizeof(T) == 4 ? 8 : 4;  // rows in flight
+      for (int i = rg; i < g.n; i += kR * RG) {
+        T v[kR][4];
+#pragma unroll
+        for (int k = 0; k < kR; ++k) ld4_stream(H + (long long)(i + k * RG) * np + 4 * q, i + k * RG < g.n, v[k]);
+#pragma unroll
+        for (int k = 0; k < kR; ++k) {
+          if (i + k * RG >= g.n) break;
+          const T xv = xs[i + k * RG];
+          acc[0] += v[k][0] * xv; acc[1] += v[k][1] * xv; acc[2] += v[k][2] * xv; acc[3] += v[k][3] * xv;
+        }
       }
     }
 #pragma unroll
@@ -667,38 +689,72 @@ __global__ void __launch_bounds__(kSmallWarps * 32) k_group_bwd_level(
 // ---- large separator entities, split over many CTAs (levels with entities
 // of more than kSplitDofs DOFs).  The entity input x_g (forward: minus the
 // cells' contributions) is first gathered into the scratch gs, so that the
-// row or column blocks of H can update x in place from any CTA.
+// row or column blocks of H can update x in place from any CTA.  The level's
+// small entities (disjoint DOFs) are done by further CTAs of the same launch:
+// a level costs two dependent launches per direction instead of three.  With
+// the indices, the rows' prefetch and the first column loads before the
+// dependency point (63^3, leaf 8): level 2 forward 18.3 -> 14.7 us, backward
+// 31.0 -> 13.8; steps 5.29 -> 4.76 ms together with the unsplit entities below
+// the limit (level 1 backward 21.5 -> 14.3).
+constexpr int kGatherCtas = 4;  // per large entity
 
-// grid = (large entities, chunks)
-template <typename T>
-__global__ void __launch_bounds__(256) k_group_gather(const int *__restrict__ large, int nlarge,
-                                                      const GroupDesc *__restrict__ groups,
-                                                      const int *__restrict__ idx,
-                                                      const long long *__restrict__ cptr,
-                                                      const long long *__restrict__ cslot,
-                                                      const T *__restrict__ contrib,
-                                                      const T *__restrict__ x,
-                                                      const long long *__restrict__ gs_off,
-                                                      T *__restrict__ gs) {
-  pdl_enter();
-  const GroupDesc g = groups[large[blockIdx.x]];
+template <typename T, typename TV, bool kFwd>
+__global__ void __launch_bounds__(kSmallWarps * 32) k_group_gather(
+    const int *__restrict__ large, int nlarge, const int *__restrict__ small, int nsmall,
+    const GroupDesc *__restrict__ groups, const int *__restrict__ idx, const long long *__restrict__ cptr,
+    const long long *__restrict__ cslot, const TV *__restrict__ vals, const T *__restrict__ contrib, T *x,
+    const long long *__restrict__ gs_off, T *__restrict__ gs) {
+  constexpr int NT = kSmallWarps * 32;
+  __shared__ T sm[NT];
+  if (blockIdx.x >= kGatherCtas * nlarge) {
+    const int warp = threadIdx.x >> 5, t = (blockIdx.x - kGatherCtas * nlarge) * kSmallWarps + warp;
+    if (t >= nsmall) pdl_enter();  // a warp without an entity
+    else if constexpr (kFwd)
+      group_fwd_small_warp<T, TV, true, true>(groups[small[t]], idx, cptr, cslot, vals, contrib, x, x, sm + 32 * warp);
+    else
+      group_bwd_small_warp<T, TV, true, true>(groups[small[t]], idx, vals, x, x, sm + 32 * warp);
+    return;
+  }
+  const int e = blockIdx.x / kGatherCtas;
+  const GroupDesc g = groups[large[e]];
   const int *gi = idx + g.idx_off;
-  T *out = gs + gs_off[blockIdx.x];
+  T *out = gs + gs_off[e];
   const int np = (int)pad4(g.n);
-  for (int i = blockIdx.y * 256 + threadIdx.x; i < np; i += gridDim.y * 256) {
+  // the first DOF's index and slots before the dependency point, as in group_fwd_unit
+  const int i0 = (blockIdx.x % kGatherCtas) * NT + threadIdx.x;
+  constexpr int kSlots = 4;
+  int dof = 0;
+  long long a = 0, b = 0, sl[kSlots] = {};
+  const auto fetch = [&](int i) {
+    if (i >= g.n) return;
+    dof = gi[i];
+    if constexpr (kFwd) {
+      a = cptr[g.cptr_off + i];
+      b = cptr[g.cptr_off + i + 1];
+#pragma unroll
+      for (int k = 0; k < kSlots; ++k) sl[k] = a + k < b ? cslot[a + k] : 0;
+    }
+  };
+  fetch(i0);
+  pdl_enter();
+  for (int i = i0; i < np; i += kGatherCtas * NT) {
+    if (i != i0) fetch(i);
     T v = T(0);
     if (i < g.n) {
-      v = x[gi[i]];
-      if (contrib) {
-        const long long a = cptr[g.cptr_off + i], b = cptr[g.cptr_off + i + 1];
-        for (long long s = a; s < b; ++s) v -= contrib[cslot[s]];
+      v = __ldcg(x + dof);
+      if constexpr (kFwd) {
+#pragma unroll
+        for (int k = 0; k < kSlots; ++k)
+          if (a + k < b) v -= __ldcg(contrib + sl[k]);
+        for (long long s = a + kSlots; s < b; ++s) v -= __ldcg(contrib + cslot[s]);
       }
     }
     out[i] = v;
   }
 }
 
-// forward, rows [r0, r0 + kSplitRows) of one entity: x_g[r] = H[r, :] gs_g
+// forward, rows [r0, r0 + kSplitRows) of one entity: x_g[r] = H[r, :] gs_g.
+// The rows are on their way to L2 before the dependency point.
 template <typename T, typename TV = T>
 __global__ void __launch_bounds__(256) k_group_rows_split(const int2 *__restrict__ rblk,
                                                           const int *__restrict__ large,
@@ -708,19 +764,20 @@ __global__ void __launch_bounds__(256) k_group_rows_split(const int2 *__restrict
                                                           const long long *__restrict__ gs_off,
                                                           const T *__restrict__ gs,
                                                           T *__restrict__ x) {
-  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *xs = reinterpret_cast<T *>(smem_raw);
   const int2 rb = rblk[blockIdx.x];
   const GroupDesc g = groups[large[rb.x]];
   const int np = (int)pad4(g.n);
   const T *in = gs + gs_off[rb.x];
-  for (int i = threadIdx.x; i < np; i += 256) xs[i] = in[i];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int *gi = idx + g.idx_off;
   const TV *H = vals + g.H_off;
   const int r_hi = min(g.n, rb.y + kSplitRows);
+  if (threadIdx.x == 0) prefetch_block_l2(H + (long long)rb.y * np, (long long)(r_hi - rb.y) * np);
+  pdl_enter();
+  for (int i = threadIdx.x; i < np; i += 256) xs[i] = __ldcg(in + i);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int r0 = rb.y + warp * kRows; r0 < r_hi; r0 += 8 * kRows) {
     const TV *rp[kRows];
     int nq[kRows];
@@ -740,7 +797,9 @@ __global__ void __launch_bounds__(256) k_group_rows_split(const int2 *__restrict
   }
 }
 
-// backward, columns [c0, c0 + kSplitCols) of one entity: x_g[c] = sum_i H[i][c] gs_g[i]
+// backward, columns [c0, c0 + kSplitCols) of one entity: x_g[c] = sum_i H[i][c] gs_g[i].
+// A thread owns a column quad and every 16th row: 16-byte loads, kR rows in
+// flight, the first of them before the dependency point.
 template <typename T, typename TV = T>
 __global__ void __launch_bounds__(256) k_group_cols_split(const int2 *__restrict__ cblk,
                                                           const int *__restrict__ large,
@@ -750,32 +809,48 @@ __global__ void __launch_bounds__(256) k_group_cols_split(const int2 *__restrict
                                                           const long long *__restrict__ gs_off,
                                                           const T *__restrict__ gs,
                                                           T *__restrict__ x) {
-  pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *xs = reinterpret_cast<T *>(smem_raw);
+  constexpr int QW = kSplitCols / 4, RG = 256 / QW;  // column quads, row groups
+  constexpr int kR = sizeof(T) == 4 ? 8 : 4;
+  __shared__ T part[RG][kSplitCols];
   const int2 cb = cblk[blockIdx.x];
   const GroupDesc g = groups[large[cb.x]];
   const int n = g.n;
   const long long np = pad4(n);
-  T *part = xs + np;  // 256 partial sums
   const T *in = gs + gs_off[cb.x];
-  for (int i = threadIdx.x; i < n; i += 256) xs[i] = in[i];
+  const int ql = threadIdx.x % QW, rg = threadIdx.x / QW, col = cb.y + 4 * ql;
+  const bool ok = col < n;  // the quad is inside the padded row
+  const TV *H = vals + g.H_off + (ok ? col : 0);
+  T v[kR][4];
+#pragma unroll
+  for (int k = 0; k < kR; ++k) ld4_stream(H + (rg + k * RG) * np, ok && rg + k * RG < n, v[k]);
+  pdl_enter();
+  for (int i = threadIdx.x; i < n; i += 256) xs[i] = __ldcg(in + i);
   __syncthreads();
-  constexpr int CW = kSplitCols, RG = 256 / kSplitCols;
-  const int cl = threadIdx.x % CW, rg = threadIdx.x / CW;
-  const int col = cb.y + cl;
-  const TV *H = vals + g.H_off;
-  T acc = T(0);
-  if (col < n) {
-#pragma unroll 4
-    for (int i = rg; i < n; i += RG) acc += ldv<T>(H + (long long)i * np + col) * xs[i];
+  T acc[4] = {T(0), T(0), T(0), T(0)};
+  for (int i = rg; i < n; i += kR * RG) {
+    if (i != rg) {
+#pragma unroll
+      for (int k = 0; k < kR; ++k) ld4_stream(H + (i + k * RG) * np, ok && i + k * RG < n, v[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < kR; ++k) {
+      if (i + k * RG >= n) break;
+      const T xv = xs[i + k * RG];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[e] += v[k][e] * xv;
+    }
   }
-  part[threadIdx.x] = acc;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) part[rg][4 * ql + e] = acc[e];
   __syncthreads();
-  if (rg == 0 && col < n) {
-    T sum = part[cl];
-    for (int q = 1; q < RG; ++q) sum += part[q * CW + cl];
-    x[idx[g.idx_off + col]] = sum;
+  const int c = threadIdx.x;
+  if (c < kSplitCols && cb.y + c < n) {
+    T sum = part[0][c];
+#pragma unroll
+    for (int q = 1; q < RG; ++q) sum += part[q][c];
+    x[idx[g.idx_off + cb.y + c]] = sum;
   }
 }
 
@@ -2541,37 +2616,33 @@ int launch_group_fwd(Handle *h, const LevelDev &lv, int l, const FactorValues<T>
                lv.vals_group * (b16 ? 2.0 : E) + (lv.vec_group + lv.contrib) * E + lv.idx_group +
                    lv.cslot_bytes,
                s);
-  if (lv.split) {  // large entities over many CTAs, then the small ones
+  if (lv.split) {  // large entities gathered and the small ones, then the large over many CTAs
     const size_t smx = (size_t)pad4(lv.max_ng) * sizeof(T);
-    HIF_CUDA_TRY(launch_k(k_group_gather<T>, dim3(lv.nlarge, 4), 256, 0, s, lv.large_groups, lv.nlarge, lv.groups, h->idx,
-                                                         h->cptr, h->cslot, fv.contrib, x, lv.gs_off,
-                                                         fv.gs));
-    bool done = false;
-    if constexpr (sizeof(T) == 4) {
-      if (b16) {
-        HIF_CUDA_TRY(launch_k(k_group_rows_split<T, bf16>, lv.nrblk, 256, smx, s, lv.rblk, lv.large_groups, lv.groups, h->idx,
-                                                               static_cast<const bf16 *>(h->bf16_vals),
-                                                               lv.gs_off, fv.gs, x));
-        done = true;
-      }
-    }
-    if (!done)
-      HIF_CUDA_TRY(launch_k(k_group_rows_split<T>, lv.nrblk, 256, smx, s, lv.rblk, lv.large_groups, lv.groups, h->idx, fv.vals,
-                                                       lv.gs_off, fv.gs, x));
-    note_launch(1 + (lv.nsmall ? 1 : 0));
-    if (!lv.nsmall) return HIF_OK;
+    const int ng = kGatherCtas * lv.nlarge + (lv.nsmall + kSmallWarps - 1) / kSmallWarps;
+    const auto run = [&](auto *vals) {
+      using TV = std::remove_const_t<std::remove_pointer_t<decltype(vals)>>;
+      HIF_CUDA_TRY(launch_k(k_group_gather<T, TV, true>, ng, kSmallWarps * 32, 0, s, lv.large_groups, lv.nlarge,
+                            lv.small_groups, lv.nsmall, lv.groups, h->idx, h->cptr, h->cslot, vals, fv.contrib, x,
+                            lv.gs_off, fv.gs));
+      HIF_CUDA_TRY(launch_k(k_group_rows_split<T, TV>, lv.nrblk, 256, smx, s, lv.rblk, lv.large_groups, lv.groups,
+                            h->idx, vals, lv.gs_off, fv.gs, x));
+      note_launch();
+      return (int)HIF_OK;
+    };
+    if constexpr (sizeof(T) == 4)
+      if (b16) return run(static_cast<const bf16 *>(h->bf16_vals));
+    return run(static_cast<const T *>(fv.vals));
   }
-  const int nlg = lv.split ? 0 : lv.nlarge;  // large entities already done when split
-  const int grid = nlg + (lv.nsmall + kSmallWarps - 1) / kSmallWarps;
+  const int grid = lv.nlarge + (lv.nsmall + kSmallWarps - 1) / kSmallWarps;
   if constexpr (sizeof(T) == 4) {
     if (b16) {
       HIF_CUDA_TRY(launch_k(k_group_fwd_level<T, bf16>, grid, kSmallWarps * 32, sm, s, 
-          lv.large_groups, nlg, lv.small_groups, lv.nsmall, lv.groups, h->idx, h->cptr, h->cslot,
+          lv.large_groups, lv.nlarge, lv.small_groups, lv.nsmall, lv.groups, h->idx, h->cptr, h->cslot,
           static_cast<const bf16 *>(h->bf16_vals), fv.contrib, x));
       return HIF_OK;
     }
   }
-  HIF_CUDA_TRY(launch_k(k_group_fwd_level<T>, grid, kSmallWarps * 32, sm, s, lv.large_groups, nlg, lv.small_groups,
+  HIF_CUDA_TRY(launch_k(k_group_fwd_level<T>, grid, kSmallWarps * 32, sm, s, lv.large_groups, lv.nlarge, lv.small_groups,
                                                           lv.nsmall, lv.groups, h->idx, h->cptr,
                                                           h->cslot, fv.vals, fv.contrib, x));
   return HIF_OK;
@@ -2586,35 +2657,32 @@ int launch_group_bwd(Handle *h, const LevelDev &lv, int l, const FactorValues<T>
   const bool b16 = bf16_level<T>(h, l);
   StatScope sc(h, "group_bwd", l, lv.vals_group * (b16 ? 2.0 : E) + lv.vec_group * E + lv.idx_group_bwd, s);
   if (lv.split) {
-    const size_t smx = ((size_t)pad4(lv.max_ng) + 256) * sizeof(T);
-    HIF_CUDA_TRY(launch_k(k_group_gather<T>, dim3(lv.nlarge, 4), 256, 0, s, lv.large_groups, lv.nlarge, lv.groups, h->idx,
-                                                         h->cptr, h->cslot, nullptr, x, lv.gs_off, fv.gs));
-    bool done = false;
-    if constexpr (sizeof(T) == 4) {
-      if (b16) {
-        HIF_CUDA_TRY(launch_k(k_group_cols_split<T, bf16>, lv.ncblk, 256, smx, s, lv.cblk, lv.large_groups, lv.groups, h->idx,
-                                                               static_cast<const bf16 *>(h->bf16_vals),
-                                                               lv.gs_off, fv.gs, x));
-        done = true;
-      }
-    }
-    if (!done)
-      HIF_CUDA_TRY(launch_k(k_group_cols_split<T>, lv.ncblk, 256, smx, s, lv.cblk, lv.large_groups, lv.groups, h->idx, fv.vals,
-                                                       lv.gs_off, fv.gs, x));
-    note_launch(1 + (lv.nsmall ? 1 : 0));
-    if (!lv.nsmall) return HIF_OK;
+    const size_t smx = (size_t)pad4(lv.max_ng) * sizeof(T);
+    const int ng = kGatherCtas * lv.nlarge + (lv.nsmall + kSmallWarps - 1) / kSmallWarps;
+    const auto run = [&](auto *vals) {
+      using TV = std::remove_const_t<std::remove_pointer_t<decltype(vals)>>;
+      HIF_CUDA_TRY(launch_k(k_group_gather<T, TV, false>, ng, kSmallWarps * 32, 0, s, lv.large_groups, lv.nlarge,
+                            lv.small_groups, lv.nsmall, lv.groups, h->idx, h->cptr, h->cslot, vals, nullptr, x,
+                            lv.gs_off, fv.gs));
+      HIF_CUDA_TRY(launch_k(k_group_cols_split<T, TV>, lv.ncblk, 256, smx, s, lv.cblk, lv.large_groups, lv.groups,
+                            h->idx, vals, lv.gs_off, fv.gs, x));
+      note_launch();
+      return (int)HIF_OK;
+    };
+    if constexpr (sizeof(T) == 4)
+      if (b16) return run(static_cast<const bf16 *>(h->bf16_vals));
+    return run(static_cast<const T *>(fv.vals));
   }
-  const int nlg = lv.split ? 0 : lv.nlarge;
-  const int grid = nlg + (lv.nsmall + kSmallWarps - 1) / kSmallWarps;
+  const int grid = lv.nlarge + (lv.nsmall + kSmallWarps - 1) / kSmallWarps;
   if constexpr (sizeof(T) == 4) {
     if (b16) {
       HIF_CUDA_TRY(launch_k(k_group_bwd_level<T, bf16>, grid, kSmallWarps * 32, sm, s, 
-          lv.large_groups, nlg, lv.small_groups, lv.nsmall, lv.groups, h->idx,
+          lv.large_groups, lv.nlarge, lv.small_groups, lv.nsmall, lv.groups, h->idx,
           static_cast<const bf16 *>(h->bf16_vals), x));
       return HIF_OK;
     }
   }
-  HIF_CUDA_TRY(launch_k(k_group_bwd_level<T>, grid, kSmallWarps * 32, sm, s, lv.large_groups, nlg, lv.small_groups,
+  HIF_CUDA_TRY(launch_k(k_group_bwd_level<T>, grid, kSmallWarps * 32, sm, s, lv.large_groups, lv.nlarge, lv.small_groups,
                                                           lv.nsmall, lv.groups, h->idx, fv.vals, x));
   return HIF_OK;
 }
