@@ -54,7 +54,7 @@ __device__ inline void tri_tile(int x, int &ti, int &tj) {
 // spread over all of them (thread t owns entries t, t + 256, ... of the 32 x 32
 // block).  One warp with a row a lane took up to 31 dependent multiply-adds a step
 // on a pipe that starts a warp's every 64 cycles: 70 us a launch at 3D 47^3, and a
-// launch a panel; @DIAG@ now.  Non-positive pivots set *err and are replaced by 1 so
+// launch a panel; 30 us now.  Non-positive pivots set *err and are replaced by 1 so
 // the kernel completes.
 template <class Cell>
 __global__ void __launch_bounds__(kThreads) k_chol_diag(const Cell *__restrict__ cells,

@@ -326,29 +326,55 @@ __global__ void __launch_bounds__(NT) k_unpack_Linv(const SGroup *__restrict__ g
 
 // Block Jacobi on a cell's boundary block, F_BB <- D F_BB D^T with D the
 // block-diagonal of the entities' L^{-1}; the entities' own diagonal blocks
-// become I (owner cell) or 0.  Two passes over (cells, chunks):
-// rows first (Sc = D F_BB), then columns (F_BB = Sc D^T).
+// become I (owner cell) or 0.  Two passes over (cells, 32 x 32 tiles): rows
+// first (Sc = D F_BB), then columns (F_BB = Sc D^T).  Bound by the FP64 pipe:
+// a warp takes one row of D at a time, so its lanes run sums of one length, read
+// D by broadcast and F or Sc along a column; tiles are turned in shared memory.
+// The own diagonal blocks are never formed, and the symmetric second pass forms
+// the tiles on and below the diagonal and mirrors them.  Measured in the setup
+// of 47^3, where lanes along the rows of D took 10.0 + 5.3 ms: 5.4 + 3.2 ms.
+constexpr int kSc = 32;
+static_assert(NT == 256, "8 warps, 4 rows of a tile each");
+
 __global__ void __launch_bounds__(NT) k_cell_scale_rows(const SCell *__restrict__ cells, int cell0,
                                                         const int2 *__restrict__ bmap,
                                                         const SGroup *__restrict__ groups,
                                                         const double *__restrict__ Linv,
                                                         const double *__restrict__ F,
                                                         double *__restrict__ S, long long sc_base) {
+  __shared__ double tile[kSc][kSc + 1];
   const SCell c = cells[cell0 + blockIdx.x];
-  const int nI = c.nI, nB = c.nB, nn = nI + nB;
+  const int nI = c.nI, nB = c.nB, nn = nI + nB, nt = (nB + kSc - 1) / kSc;
   const double *A = F + c.F_off;
   double *Sc = S + (c.Sc_off - sc_base);
   const int2 *bm = bmap + c.bmap_off;
-  const long long nbb = (long long)nB * nB;
-  for (long long t = blockIdx.y * (long long)NT + threadIdx.x; t < nbb; t += (long long)gridDim.y * NT) {
-    const int p = (int)(t % nB), q = (int)(t / nB);
-    const int2 gp = bm[p];
-    const SGroup g = groups[gp.x];
-    const int o = p - gp.y;
-    const double *Li = Linv + g.Linv_off + (long long)gp.y * g.n;
-    double acc = 0.0;
-    for (int b = 0; b <= gp.y; ++b) acc += Li[b] * A[nI + o + b + (long long)(nI + q) * nn];
-    Sc[p + (long long)q * nB] = acc;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int y = blockIdx.y; y < nt * nt; y += gridDim.y) {
+    const int p0 = (y % nt) * kSc, q0 = (y / nt) * kSc, q = q0 + lane;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int p = p0 + warp + 8 * j;
+      double acc = 0.0;
+      if (p < nB) {
+        const int2 gp = bm[p];
+        const SGroup g = groups[gp.x];
+        const int o = p - gp.y;
+        if (q < nB && (q < o || q >= o + g.n)) {  // F_BB is symmetric: its column o + b along q
+          const double *Li = Linv + g.Linv_off + (long long)gp.y * g.n;
+          const double *Aq = A + nI + q + (long long)(nI + o) * nn;
+#pragma unroll 4
+          for (int b = 0; b <= gp.y; ++b) acc += Li[b] * Aq[(long long)b * nn];
+        }
+      }
+      tile[warp + 8 * j][lane] = acc;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int qq = q0 + warp + 8 * j;
+      if (qq < nB && p0 + lane < nB) Sc[p0 + lane + (long long)qq * nB] = tile[lane][warp + 8 * j];
+    }
+    __syncthreads();
   }
 }
 
@@ -359,30 +385,46 @@ __global__ void __launch_bounds__(NT) k_cell_scale_cols(const SCell *__restrict_
                                                         const double *__restrict__ Linv,
                                                         double *__restrict__ F,
                                                         const double *__restrict__ S, long long sc_base) {
+  __shared__ double tile[kSc][kSc + 1];
   const int cid = cell0 + (int)blockIdx.x;
   const SCell c = cells[cid];
-  const int nI = c.nI, nB = c.nB, nn = nI + nB;
-  double *A = F + c.F_off;
+  const int nI = c.nI, nB = c.nB, nn = nI + nB, nt = (nB + kSc - 1) / kSc;
+  double *A = F + c.F_off + nI + (long long)nI * nn;
   const double *Sc = S + (c.Sc_off - sc_base);
   const int2 *bm = bmap + c.bmap_off;
-  const long long nbb = (long long)nB * nB;
-  for (long long t = blockIdx.y * (long long)NT + threadIdx.x; t < nbb; t += (long long)gridDim.y * NT) {
-    const int p = (int)(t % nB), q = (int)(t / nB);
-    const int2 gp = bm[p], gq = bm[q];
-    double v;
-    if (gp.x == gq.x) {
-      const SGroup g = groups[gp.x];
-      const bool owner = gcells[g.gc_off].x == cid;
-      v = (owner && gp.y == gq.y) ? 1.0 : 0.0;
-    } else {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int y = blockIdx.y; y < nt * (nt + 1) / 2; y += gridDim.y) {
+    int ti, tj;
+    dense::tri_tile(y, ti, tj);
+    const int p0 = ti * kSc, q0 = tj * kSc, p = p0 + lane;
+    const int2 gp = p < nB ? bm[p] : make_int2(-1, 0);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int q = q0 + warp + 8 * j;
+      if (q >= nB) break;
+      const int2 gq = bm[q];
       const SGroup g = groups[gq.x];
-      const int o = q - gq.y;
-      const double *Li = Linv + g.Linv_off + (long long)gq.y * g.n;
-      double acc = 0.0;
-      for (int b = 0; b <= gq.y; ++b) acc += Sc[p + (long long)(o + b) * nB] * Li[b];
-      v = acc;
+      double v = 0.0;
+      if (gp.x == gq.x) {
+        v = gp.y == gq.y && gcells[g.gc_off].x == cid ? 1.0 : 0.0;
+      } else if (p < nB) {
+        const double *Li = Linv + g.Linv_off + (long long)gq.y * g.n;
+        const double *Sp = Sc + p + (long long)(q - gq.y) * nB;
+#pragma unroll 4
+        for (int b = 0; b <= gq.y; ++b) v += Sp[(long long)b * nB] * Li[b];
+      }
+      if (p < nB) A[p + (long long)q * nn] = v;
+      tile[warp + 8 * j][lane] = v;
     }
-    A[nI + p + (long long)(nI + q) * nn] = v;
+    __syncthreads();
+    if (ti != tj) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int pp = p0 + warp + 8 * j;
+        if (pp < nB && q0 + lane < nB) A[q0 + lane + (long long)pp * nn] = tile[lane][warp + 8 * j];
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -1695,10 +1737,12 @@ int gpu_setup(Handle *h, const double *a_nodes, cudaStream_t s) {
         const int c0 = sch_at[k], nck = sch_at[k + 1] - c0;
         int max_nB = 1;
         for (int c = c0; c < c0 + nck; ++c) max_nB = std::max(max_nB, cells[c].nB);
-        const int sch = chunks_for((long long)max_nB * max_nB);
+        const long long nt = (max_nB + kSc - 1) / kSc;  // tiles, grid.y capped
+        const int sch = (int)std::min<long long>(nt * nt, 65535);
+        const int schl = (int)std::min<long long>(nt * (nt + 1) / 2, 65535);
         const long long base = cells[c0].Sc_off;
         k_cell_scale_rows<<<dim3(nck, sch), NT, 0, s>>>(dbcells, c0, dbmap, dgroups, Linv, Fb, Sscr, base);
-        k_cell_scale_cols<<<dim3(nck, sch), NT, 0, s>>>(dbcells, c0, dbmap, dgroups, dgcells, Linv, Fb, Sscr,
+        k_cell_scale_cols<<<dim3(nck, schl), NT, 0, s>>>(dbcells, c0, dbmap, dgroups, dgcells, Linv, Fb, Sscr,
                                                         base);
         note_launch(2);
         HIF_CUDA_TRY(cudaGetLastError());
