@@ -778,6 +778,8 @@ __global__ void __launch_bounds__(kQrThreads) k_skel_qr(const SSkel *__restrict_
       best_j = j;
     }
   }
+  // every CTA of the cluster has started before one stores into another's shared memory
+  cluster_sync();
   const int tmax = R < n ? R : n;
   double r00 = 0.0;
   int k = 0;
