@@ -99,8 +99,11 @@ __global__ void __launch_bounds__(kThreads) k_chol_diag(const Cell *__restrict__
       if (i > k && i < jb && j > k && j <= i) D[i][j] -= li * D[j][k];
     }
     __syncthreads();
-    if (q == 0 && i >= k && i < jb) D[i][k] = i == k ? s_r[2] : dik * s_r[0];
     // (the next step reads columns > k only; column k is next read after the loop)
+    if (q == 0) {
+      if (i >= k && i < jb) D[i][k] = i == k ? s_r[2] : dik * s_r[0];
+      __syncwarp();  // lane 0 writes the next step's s_r
+    }
   }
   __syncthreads();
 #pragma unroll

@@ -26,3 +26,13 @@ def test_cluster_has_started_before_its_shared_memory_is_written():
     assert 0 <= body.find("cluster_sync();") < body.find("cluster_store(")
     # and none of its CTAs leaves while another may still store
     assert body.rfind("cluster_sync();") > body.rfind("cluster_store(")
+
+
+def test_scalars_of_a_panel_step_are_read_before_the_next_are_written():
+    body = _body("dense_batched.cuh", "k_chol_diag")
+    loop = body[body.index("for (int k = 0; k < jb; ++k)"):]
+    # one warp writes and reads s_r; its reads after the last CTA barrier of a step
+    # end at a warp barrier
+    tail = loop[loop.index("if (q == 0)", loop.rindex("D[i][j] -=")):]
+    read = max(tail.index("s_r[0]"), tail.index("s_r[2]"))
+    assert "__syncwarp();" in tail[read:tail.index("A[(j0 + i)")].split("__syncthreads();")[0]
