@@ -1191,7 +1191,8 @@ __device__ __forceinline__ void drain_ring(int k, unsigned long long *full) {
 template <typename T, int NS>
 __device__ __forceinline__ void produce_cells(int ncells, bool tri, unsigned char *stage, int2 *meta, const CellMeta *cm,
                                               unsigned long long *ready, unsigned long long *full,
-                                              unsigned long long *empty, double *err) {
+                                              unsigned long long *empty, unsigned long long *freed,
+                                              double *err) {
   int k = 0;  // running chunk counter of this CTA
   int jc = 0;
   for (int ci = blockIdx.x; ci < ncells; ci += gridDim.x, ++jc) {
@@ -1220,6 +1221,7 @@ __device__ __forceinline__ void produce_cells(int ncells, bool tri, unsigned cha
       bulk_load(stage + (size_t)sidx * kStageBytes, block + a, (unsigned)((b - a) * sizeof(T)),
                 &full[sidx]);
     }
+    mbar_arrive(&freed[bb]);  // cm[bb] is no longer read here
   }
   drain_ring<NS>(k, full);
 }
@@ -1231,7 +1233,9 @@ __device__ __forceinline__ void produce_cells(int ncells, bool tri, unsigned cha
 // the descriptor and chunk bounds are in place (only the factor was read:
 // with PDL this happens before the previous kernel has finished) and on
 // ready[b] once x is gathered.
-// Before refilling a buffer it waits until the consumers freed it.
+// Before refilling a buffer it waits until the consumers and the copy warp freed
+// it (an empty cell has no chunk on which the consumers would wait for the copy
+// warp).
 template <typename T, class Src>
 __device__ __forceinline__ void gather_cells(const Src &src, int ncells, CellMeta *cm, T *xs0, long long xs_stride,
                                              T *xb0, long long xb_stride, int *is0, unsigned long long *ready,
@@ -1444,7 +1448,7 @@ __global__ void __launch_bounds__(kTmaThreads, 4) k_cell_fwd_tma_S(Src src, int 
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ready[b], 32);
       mbar_init(&mready[b], 32);
-      mbar_init(&freed[b], kConsumerWarps);
+      mbar_init(&freed[b], kConsumerWarps + 1);  // and the copy warp
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1452,7 +1456,7 @@ __global__ void __launch_bounds__(kTmaThreads, 4) k_cell_fwd_tma_S(Src src, int 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == kConsumerWarps) {
     if (lane == 0)
-      produce_cells<T, kStagesFwd>(ncells, false, stage, meta, cm, mready, full, empty, err);
+      produce_cells<T, kStagesFwd>(ncells, false, stage, meta, cm, mready, full, empty, freed, err);
     return;
   }
   if (warp == kConsumerWarps + 1) {
@@ -1560,7 +1564,7 @@ __global__ void __launch_bounds__(kTmaThreads, kComp ? 3 : 2) k_cell_bwd_tma_S(S
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ready[b], 32);
       mbar_init(&mready[b], 32);
-      mbar_init(&freed[b], kConsumerWarps);
+      mbar_init(&freed[b], kConsumerWarps + 1);  // and the copy warp
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1568,7 +1572,7 @@ __global__ void __launch_bounds__(kTmaThreads, kComp ? 3 : 2) k_cell_bwd_tma_S(S
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == kConsumerWarps) {
     if (lane == 0)
-      produce_cells<T, kStagesBwd>(ncells, true, stage, meta, cm, mready, full, empty, err);
+      produce_cells<T, kStagesBwd>(ncells, true, stage, meta, cm, mready, full, empty, freed, err);
     return;
   }
   if (warp == kConsumerWarps + 1) {

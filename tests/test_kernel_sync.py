@@ -36,3 +36,16 @@ def test_scalars_of_a_panel_step_are_read_before_the_next_are_written():
     tail = loop[loop.index("if (q == 0)", loop.rindex("D[i][j] -=")):]
     read = max(tail.index("s_r[0]"), tail.index("s_r[2]"))
     assert "__syncwarp();" in tail[read:tail.index("A[(j0 + i)")].split("__syncthreads();")[0]
+
+
+def test_copy_warp_releases_the_cell_buffer():
+    # cm[b] is read by the consumers and by the copy warp: the gather warp refills it
+    # after both have arrived
+    for kernel in ("k_cell_fwd_tma_S", "k_cell_bwd_tma_S"):
+        body = _body("apply.cu", kernel)
+        assert re.search(r"mbar_init\(&freed\[b\], kConsumerWarps \+ 1\);", body)
+        assert re.search(r"produce_cells<[^;]*\bfreed\b[^;]*;", body)
+    body = _body("apply.cu", "produce_cells")
+    chunks = body[body.index("for (int j = 0; j < nch"):]
+    assert chunks.index("mbar_arrive(&freed[bb]);") > chunks.index("bulk_load(")
+    assert "cm[" not in chunks
