@@ -35,7 +35,9 @@ constexpr int kThreads = 256;
 constexpr int kMaxGridY = 65535;  // the launch limit of grid.y
 // up to this size a block column of the inverse has at most 28 dependent block
 // products and one launch does it (2D 511^2, cells of 53 to 121: 0.3 ms in all
-// against 1.2 in the launches of the doubling); above it the doubling spreads it
+// against 1.2 in the launches of the doubling); above it the doubling spreads it.
+// Each cell goes by its own size: the sums of one do not depend on the others in
+// its launch, whose number depends on the free memory.
 constexpr int kInvColumn = 256;
 
 __host__ __device__ inline int ceil_div(long long a, int b) { return (int)((a + b - 1) / b); }
@@ -257,7 +259,7 @@ __global__ void __launch_bounds__(kThreads) k_inv_offdiag(const Cell *__restrict
   const Cell c = cells[blockIdx.x];
   const int cb = blockIdx.y;
   const int nb = ceil_div(c.nI, kPanel);
-  if (cb >= nb - 1) return;
+  if (c.nI > kInvColumn || cb >= nb - 1) return;
   const int nn = c.nI + c.nB;
   const double *A = F + c.F_off;
   double *G = vals + c.G_off;
@@ -321,7 +323,8 @@ __global__ void __launch_bounds__(kThreads) k_inv_offdiag(const Cell *__restrict
 // 3D 47^3, where the first column alone holds 2145 dependent block products; all
 // inverses there 30 -> 20 ms.
 // T = L21 G11 is kept in the unused upper triangle of A_II: T(i, j) at (j, i).
-// grid = (cells, pairs x tiles); kSecond: the second product.
+// grid = (cells, pairs x tiles); kSecond: the second product.  Cells of at most
+// kInvColumn rows are left to k_inv_offdiag.
 template <class Cell, bool kSecond>
 __global__ void __launch_bounds__(kThreads) k_inv_double(const Cell *__restrict__ cells,
                                                          double *__restrict__ F,
@@ -329,6 +332,7 @@ __global__ void __launch_bounds__(kThreads) k_inv_double(const Cell *__restrict_
   __shared__ double As[kPanel][kTile + 1];  // [k][i]
   __shared__ double Bs[kPanel][kTile + 1];  // [k][j]
   const Cell c = cells[blockIdx.x];
+  if (c.nI <= kInvColumn) return;
   const int nI = c.nI, nn = nI + c.nB;
   const int tpb = ceil_div(b, kTile), npair = ceil_div(nI, 2 * b);
   double *A = F + c.F_off;
@@ -469,9 +473,10 @@ int eliminate_cells(const std::vector<Cell> &cells_h, const Cell *cells_d, doubl
                     int *err, cudaStream_t s) {
   const int ncells = (int)cells_h.size();
   if (ncells == 0) return HIF_OK;
-  int max_nI = 0, max_nn = 0, max_nB = 0;
+  int max_nI = 0, max_nn = 0, max_nB = 0, max_col = 0;  // max_col: of the cells by block columns
   for (const Cell &c : cells_h) {
     max_nI = max_nI > c.nI ? max_nI : c.nI;
+    if (c.nI <= kInvColumn) max_col = max_col > c.nI ? max_col : c.nI;
     max_nB = max_nB > c.nB ? max_nB : c.nB;
     max_nn = max_nn > c.nI + c.nB ? max_nn : c.nI + c.nB;
   }
@@ -493,8 +498,8 @@ int eliminate_cells(const std::vector<Cell> &cells_h, const Cell *cells_d, doubl
   if (nbk > 0) {
     k_inv_diag_blocks<Cell><<<dim3(ncells, nbk), 32, 0, s>>>(cells_d, F, vals);
     note_launch();
-    if (nbk > 1 && max_nI <= kInvColumn) {
-      k_inv_offdiag<Cell><<<dim3(ncells, nbk - 1), kThreads, 0, s>>>(cells_d, F, vals);
+    if (max_col > kPanel) {
+      k_inv_offdiag<Cell><<<dim3(ncells, ceil_div(max_col, kPanel) - 1), kThreads, 0, s>>>(cells_d, F, vals);
       note_launch();
     }
     for (int b = kPanel; max_nI > kInvColumn && b < max_nI; b *= 2) {
