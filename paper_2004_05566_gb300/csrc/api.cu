@@ -128,8 +128,9 @@ int make_root_dense(Handle *h, cudaStream_t s);
 // the FP32 copy (values already on the device in h->f64.vals).
 // Work items of one level's G-form cell kernels: each cell is cut into row
 // ranges (forward) and column ranges (backward) so that a launch has about
-// `target` CTAs when the level has fewer cells than that.  The arrays of an
-// earlier call stay allocated until the handle is destroyed.
+// `target` CTAs when the level has fewer cells than that; kAutoItemTarget leaves
+// the number to the rule below.  The arrays of an earlier call stay allocated
+// until the handle is destroyed.
 int build_items(Handle *h, LevelDev &D, const LevelHost &H, int target, cudaStream_t s) {
   std::vector<CellItem> fw, bw;
   const int ncell = (int)H.cells.size();
@@ -137,10 +138,13 @@ int build_items(Handle *h, LevelDev &D, const LevelHost &H, int target, cudaStre
   // default count would leave more (3D levels of a few hundred large cells: an SM
   // with three such items waits on its loads; 63^3 cells forward, with twice the
   // loads in flight: 108, 69 and 56 -> 69, 46 and 37 us at levels 0 to 2)
-  if (target == kDefaultItemTarget && ncell < target) {
-    double vals = 0;
-    for (const CellDesc &cd : H.cells) vals += (double)cd.nI * (cd.nI + 1) / 2 + (double)cd.nB * cd.nI;
-    target = (int)std::max<double>(target, std::min(4.0 * vals / kItemBytes, 152.0 * 32));
+  if (target == kAutoItemTarget) {
+    target = kDefaultItemTarget;
+    if (ncell < target) {
+      double vals = 0;
+      for (const CellDesc &cd : H.cells) vals += (double)cd.nI * (cd.nI + 1) / 2 + (double)cd.nB * cd.nI;
+      target = (int)std::max<double>(target, std::min(4.0 * vals / kItemBytes, 152.0 * 32));
+    }
   }
   for (int c = 0; c < ncell; ++c) {
     const CellDesc &cd = H.cells[c];
@@ -160,7 +164,6 @@ int build_items(Handle *h, LevelDev &D, const LevelHost &H, int target, cudaStre
   D.nbwd = (int)bw.size();
   D.fwd_host = fw;
   D.bwd_host = bw;
-  D.item_target = target;
   HIF_TRY(dev_alloc(h, (void **)&D.fwd, std::max<size_t>(1, fw.size()) * sizeof(CellItem)));
   HIF_TRY(dev_alloc(h, (void **)&D.bwd, std::max<size_t>(1, bw.size()) * sizeof(CellItem)));
   if (!fw.empty())
@@ -214,7 +217,7 @@ int finish_device_factor(Handle *h, cudaStream_t s) {
                                    cudaMemcpyHostToDevice, s));
     // HIFCN_ITEM_TARGET overrides the CTAs per launch the cells are cut for
     // (1: cells are never cut, so every level that fits runs the S-form kernels)
-    int target = kDefaultItemTarget;
+    int target = kAutoItemTarget;
     if (const char *e = std::getenv("HIFCN_ITEM_TARGET")) target = std::max(1, std::atoi(e));
     HIF_TRY(build_items(h, D, H, target, s));
     {
@@ -1058,7 +1061,7 @@ int hif_autotune(hif_handle *h, hif_stream stream) {
   h->stats_on = true;
   h->fuse_off = true;
   const int L = h->L, reps = 5;
-  const std::vector<int> cand = {sms, 2 * sms, 4 * sms, 8 * sms, 16 * sms};
+  const std::vector<int> cand = {kAutoItemTarget, sms, 2 * sms, 4 * sms, 8 * sms, 16 * sms};
   std::vector<std::vector<double>> t(L, std::vector<double>(cand.size(), 1e30));
   std::map<std::string, double> per;
   int st = HIF_OK;
@@ -1077,7 +1080,7 @@ int hif_autotune(hif_handle *h, hif_stream stream) {
       if (v > 0.0) t[l][c] = v;
     }
   }
-  std::vector<int> best(L, kDefaultItemTarget);
+  std::vector<int> best(L, kAutoItemTarget);
   for (int l = 0; l < L && st == HIF_OK; ++l) {
     size_t bi = 0;
     for (size_t c = 1; c < cand.size(); ++c)

@@ -70,9 +70,10 @@ constexpr int kRootDenseMax = 512;
 // Separator entities above this size are applied split over many CTAs, and
 // roots above kRootSplitDofs by a row-block and a column-block launch.
 constexpr int kSplitDofs = 256;
-// default CTAs per launch the G-form cell items are cut for (hif_autotune
-// picks per level among multiples of the SM count)
+// CTAs per launch the G-form cell items are cut for by default (hif_autotune picks
+// per level between that and multiples of the SM count)
 constexpr int kDefaultItemTarget = 152 * 4;
+constexpr int kAutoItemTarget = 0;  // the default, and finer where items would be large
 constexpr double kItemBytes = 96 * 1024;  // FP32 factor bytes of an item (see build_items)
 constexpr int kRootSplitDofs = 512;
 constexpr int kRootRowChunk = 128;  // rows of a CTA of the split root's transposed product
@@ -118,7 +119,6 @@ struct LevelDev {
   CellItem *fwd = nullptr, *bwd = nullptr;  // device
   std::vector<CellItem> fwd_host, bwd_host;  // host copies (dependency analysis)
   CellItem *fwd1 = nullptr, *bwd1 = nullptr;  // device: one item per cell (merged batched steps)
-  int item_target = 0;                // CTAs per launch the items were cut for (see build_items)
   bool has_S = false;                 // S = A_II^{-1} stored for the cells (S-form possible)
   // bulk-copy chunk tables of the FP32 cell blocks (row boundaries): cell c's
   // chunks are rows [tab[o + k], tab[o + k + 1]) for k < n, (o, n) = of[c];
