@@ -1071,9 +1071,14 @@ int hif_autotune(hif_handle *h, hif_stream stream) {
     return build_upper_plan(h);
   };
   // item cut of the G-form levels (and with it, at levels whose cells no
-  // longer split, the S-form kernels): each level takes its fastest target
+  // longer split, the S-form kernels): each level takes its fastest target.
+  // The fused launches take whole cells, and a level of uncut cells ends their
+  // range, so the levels they cover under the automatic cut keep it (1023^2 FP32,
+  // an apply: 278 us untuned, 281 with level 1 uncut and out of the fused range)
+  int fused = -1;  // levels above it have their cells in the fused launches
   for (size_t c = 0; c < cand.size() && st == HIF_OK; ++c) {
     st = set_all(cand[c]);
+    if (c == 0) fused = fused_start(h);
     if (st == HIF_OK) st = time_applies(h, reps, s, &per);
     for (int l = 0; l < L && st == HIF_OK; ++l) {
       const double v = level_cell_us(per, l);
@@ -1085,7 +1090,7 @@ int hif_autotune(hif_handle *h, hif_stream stream) {
     size_t bi = 0;
     for (size_t c = 1; c < cand.size(); ++c)
       if (t[l][c] < t[l][bi]) bi = c;
-    if (t[l][bi] < 1e29) best[l] = cand[bi];
+    if (t[l][bi] < 1e29 && (fused < 0 || l <= fused)) best[l] = cand[bi];
     st = build_items(h, h->lv[l], h->lv_host[l], best[l], s);
   }
   // CTAs per SM of the S-form kernels
