@@ -3047,7 +3047,6 @@ int build_view(Handle *h) {
     const LevelDev &D = h->lv[l];
     v.lv[l] = LevelView{D.fwd1, D.bwd1, D.cells, D.groups, D.small_groups, D.large_groups,
                         D.ncells, D.ncells, D.nsmall, D.nlarge,
-                        merged_sform(h, l) ? 1 : 0,
                         {D.chunk_of[0], D.chunk_of[1]}, {D.chunk_tab[0], D.chunk_tab[1]}};
   }
   v.root_S = h->root_S;

@@ -192,7 +192,6 @@ struct LevelView {
   const GroupDesc *groups;
   const int *small, *large;
   int nfwd, nbwd, nsmall, nlarge;
-  int sform;  // cells applied in the S-form (S = A_II^{-1} stored, FP32 values)
   const int2 *chunk_of[2];  // bulk-copy chunk tables: V, and S then V
   const int *chunk_tab[2];
 };
