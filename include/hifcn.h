@@ -94,7 +94,10 @@ typedef struct {
   int dim, n, leaf, levels;
   int root_size;          /* active DOFs left at the root (size of A_L, Eq. 3_4)          */
   int64_t factor_entries; /* stored factor values (all levels, both precisions counted once) */
-  int64_t apply_bytes;    /* algorithmic bytes one hif_apply streams in the active precision */
+  int64_t apply_bytes;    /* algorithmic bytes one hif_apply streams in the active precision,
+                             every cell counted in the G-form (G and V read per sweep); levels
+                             applied in the S-form stream less (V, then S and V): the sum of
+                             hif_stats_read's bytes over one apply is what its launches move */
   int64_t device_bytes;   /* device memory the handle holds                                */
   int precision;
   double setup_seconds;   /* wall time of the last hif_setup / import                      */
@@ -309,11 +312,12 @@ int hif_set_coefficient(hif_handle *h, const double *a_nodes, hif_stream stream)
 int hif_refactor(hif_handle *h, const double *a_nodes, hif_stream stream);
 
 /* hif_autotune - choose, by timing on this GPU, how the handle's apply is cut
- * into CTAs: per level, the number of CTAs its cell work is spread over (a
- * multiple of the SM count; levels whose cells are no longer cut use the
- * bulk-copy S-form kernels), and the CTAs per SM of those kernels.  Runs the
- * apply about 30 times (on the handle's own work vectors) and keeps the
- * fastest choice for each; the result of the apply is unchanged up to the
+ * into CTAs: per level, the number of CTAs its cell work is spread over (the
+ * default or a multiple of the SM count; levels whose cells are no longer cut
+ * use the bulk-copy S-form kernels; levels inside the fused launches keep the
+ * default), and the CTAs per SM of those kernels.  Runs the apply about 60
+ * times (on the handle's own work vectors) and keeps the fastest choice for
+ * each; the result of the apply is unchanged up to the
  * rounding order of the cell kernels.  Not part of the paper's method (an
  * implementation choice of this library).  Call between solves; it waits for
  * the device and rebuilds the handle's captured solve graphs on next use.

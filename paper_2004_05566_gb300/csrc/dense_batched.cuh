@@ -14,8 +14,9 @@
 // size gives, and the trailing matrix is read and written once per panel
 // instead of once per column.  G is formed by 32 x 32 blocks: the diagonal
 // blocks are inverted first, then small cells walk down their block columns and
-// larger ones join neighbouring blocks by doubling, G21 = -G22 (L21 G11).  V = W^T G is a 64 x 64-tiled product.
-// Every sum runs in a fixed order, so the factor is the same on every run.
+// larger ones join neighbouring blocks by doubling, G21 = -G22 (L21 G11).
+// V = W^T G is a 64 x 64-tiled product.  Every sum runs in a fixed order that depends
+// on its cell alone, so the factor is the same on every run and in every chunking.
 //
 // The kernels are templates over the cell descriptor, which must provide
 // nI, nB, F_off (frontal matrix), G_off (packed padded lower triangle) and

@@ -14,10 +14,10 @@
 // FP32 in tensor memory: the result is that of BF16 factor blocks applied to
 // the FP32 vectors, the arithmetic of the single-column BF16 levels.
 //
-// Kernel (one CTA of 128 threads per 128-row tile of one box): the K
+// Kernel (one CTA of 256 threads per 128-row tile of one box): the K
 // dimension is walked in chunks of 64; each chunk of A and of X_hi / X_lo is
 // staged by the threads into shared memory in the canonical K-major layout
-// without swizzle (8 x 16-byte core matrices), double buffered; one thread
+// without swizzle (8 x 16-byte core matrices), three chunks deep; one thread
 // issues tcgen05.mma (M = 128, N = k rounded up to 16, K = 16 per
 // instruction, kind::f16 with BF16 operands and FP32 accumulation) and
 // commits each chunk to an mbarrier, so the staging of chunk c + 1 overlaps the
@@ -26,8 +26,8 @@
 // before chunk c is stored, and a transposed block goes out as 16-byte rows
 // (63^3, 16 columns: level-1 cells backward 283 -> 171 us, forward 154 -> 73 us;
 // root 54 + 52 -> 29 + 37 us).  The accumulator lives in tensor memory (128 lanes x N
-// columns, allocated per CTA) and is read back with tcgen05.ld by the four
-// warps, one 32-lane quarter each.  Every mbarrier wait is bounded; on expiry
+// columns, allocated per CTA) and is read back with tcgen05.ld, a 32-lane
+// quarter and half the columns by each of the eight warps.  Every mbarrier wait is bounded; on expiry
 // the CTA records the failure in the handle's error slot and skips its
 // results (reported as HIF_ETIMEOUT by the solve).
 #include "internal.h"
@@ -476,11 +476,11 @@ __global__ void __launch_bounds__(kMThreads, NQ <= 8 ? 3 : 2) k_box_mma(MArgs a,
 // 128 threads takes a 128-row tile of a box; K is walked in chunks of 32,
 // A and the gathered X staged by asynchronous copies three chunks deep.  A
 // thread owns 4 rows x NC / 4 columns: per four K it reads 4 + 4 quads of
-// shared memory for 4 NC multiply-adds (two NC = 16 FMAs per byte of A), which
-// keeps the kernel near the HBM rate at k = 16 (a chip-wide FP32 rate of 40e12
-// FMA/s against 1.7e12 values/s of A times 16).  Each chunk is summed on its
-// own and added to the total, so a sum of K products rounds like one of
-// 32 + K / 32.  kComp (the levels whose single-column backward step sums the
+// shared memory for 4 NC multiply-adds.  A value of A enters NC products (four a
+// byte at NC = 16), so at k = 16 the chip's 40e12 FMA/s would take 2.5e12 values/s,
+// more than HBM delivers (1.7e12); the kernel stays below both (see the figures).
+// Each chunk is summed on its own and added to the total, so a sum of K products
+// rounds like one of 32 + K / 32.  kComp (the levels whose single-column backward step sums the
 // boundary products with compensation): four products at a time enter the
 // total by Kahan's summation.  Backward cells: the K index runs over the G
 // rows padded to a multiple of 64, then the V rows, whose chunks are
@@ -489,8 +489,9 @@ __global__ void __launch_bounds__(kMThreads, NQ <= 8 ? 3 : 2) k_box_mma(MArgs a,
 // (quads of a staged row swizzled instead of padded), and tiles skip the chunks
 // that are zero by the triangle of G.
 // Measured at 63^3 with 16 columns (level 0, 353 MB of blocks), per apply:
-// forward 1720 us column by column, 206 at three CTAs, 165 now; backward 1568,
-// 263, 227.
+// forward 1720 us column by column, 206 at three CTAs, 162 now; backward 1568,
+// 263, 222 (52 each at the copy rate).  Every tile of a box gathers the box's X
+// again, 2.6 times the blocks' bytes in L2 sectors.
 constexpr int kFThreads = 128;
 constexpr int kFC = 32;          // K of a staged chunk
 constexpr int kFStages = 3;

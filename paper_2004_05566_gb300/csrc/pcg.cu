@@ -1125,9 +1125,11 @@ int cn_multi(Handle *h, double *u, const double *r, int nsteps, int *iters, cuda
 // handle's partial sums never mix with another's and do not depend on the
 // batch), one warp per handle for the scalar phases, and the merged apply
 // phases.  A handle whose PCG has converged stops updating; the loop ends when
-// no handle is active (one 4-byte read per iteration).  The arithmetic of a
+// no handle is active (one 16-byte read per iteration).  The arithmetic of a
 // handle is the same in any batch, and equals that of its single steps to the
-// CG tolerance (the single path applies the leaf levels in the S form).
+// CG tolerance: the operators are the same, their sums not always (the single
+// path runs the upper levels fused, and S-form only where cells are whole; here
+// every level with S stored is).
 
 // 8 elements a thread: 8192 left 24 problems of 63^2 to 511^2 with 199 CTAs (w = A z
 // and the update 90 and 69 us an iteration; 42 and 34 now)

@@ -1,7 +1,7 @@
 """The factorization of the diagonal blocks gives the same bits on every run.
 
-Panels of 1 to 32 columns (interiors of 5 to 65 DOFs above the leaf level, roots of
-31 to 253), many cells and one.  Bars: exported factors equal byte for byte over
+Panels of 1 to 32 columns (interiors of 5 to 125 DOFs above the leaf level, roots of
+29 to 331), many cells and one.  Bars: exported factors equal byte for byte over
 repeated setups, and A applied to F^{-1} b gives b back within 1e-9 (eps = 0).
 """
 
